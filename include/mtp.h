@@ -315,8 +315,7 @@ mtp_status mtp_fit_bfgs(mtp_model* model, const mtp_batch* batch, const mtp_nbr*
  * specialised single-kernel mixed pass, 1, 2, 4 for the generic kernel; blocks per SM then
  * follow from the occupancy) and, for the level-20 shape of the single kernel, with the
  * forward part of the contraction schedule in shared or in global memory; for the mixed path
- * also the three-kernel pass (4 or 8 warps per block, 1 or 2 neighborhoods per contraction
- * warp) unless mtp_set_mixed_pass fixed the single kernel.  Keeps the fastest in the model for
+ * also the three-kernel pass (4 or 8 warps per block of its per-pair kernels) unless mtp_set_mixed_pass fixed the single kernel.  Keeps the fastest in the model for
  * later calls of this precision (with mixed pass 0, also which pass), and returns the single
  * kernel's warps (HOST warps) and the best time of three of the chosen shape (HOST ms) --
  * either may be NULL.  Synchronises `stream`. */
@@ -340,20 +339,22 @@ mtp_status mtp_get_launch_shape(const mtp_model* model, int32_t* warps_fast, int
  * MTP_ERR_UNSUPPORTED for 2 when the shape has no three-kernel pass.  No GPU work. */
 mtp_status mtp_set_mixed_pass(mtp_model* model, int pass);
 
-/* Launch shape of the three-kernel pass (what mtp_autotune sets): warps per block of its
- * per-pair kernels (4 or 8; 0 = default 8), neighborhoods per warp of its contraction (1 or 2;
- * 0 = default 1), schedule words per step per lane there (2 or 4, or 8 with two neighborhoods per
- * warp; 0 = default 2) and where the
- * contraction reads its schedule (1 = shared memory; 2 = streamed from global memory through a
- * shared-memory ring, the block's warps in step; 3 = tensor memory, the first 512 rows of 128 B,
- * the rest in shared memory; 0 = shared memory where it fits beside four warps' value arrays).
+/* Launch shape of the three-kernel pass: warps per block of its per-pair kernels (4 or 8; 0 =
+ * default 8; what mtp_autotune sets).  The others, all 0, run the grouped contraction (four
+ * neighborhoods side by side, fastest at every level); any of them set asks for the contraction
+ * with 1 or 2 neighborhoods per warp (0 = 1), 2 or 4 schedule words per step per lane, or 8 with
+ * two neighborhoods per warp (0 = 2), and its schedule read from 1 = shared memory; 2 = global
+ * memory, streamed through a shared-memory ring, the block's warps in step; 3 = tensor memory, the
+ * first 512 rows of 128 B, the rest in shared memory; 0 = shared memory where it fits beside four
+ * warps' value arrays.
  * A schedule that fits neither shared nor tensor memory is always streamed; a placement that
  * does not apply falls back to the automatic one.  Results do not depend on it.  MTP_ERR_ARG
  * outside these values.  No GPU work. */
 mtp_status mtp_set_split_shape(mtp_model* model, int warps_pair, int nb_contract, int unroll, int schedule);
 
 /* The shape set above (or by mtp_autotune), HOST outputs, any may be NULL; *schedule_used is
- * where the last three-kernel pass read its schedule (1, 2 or 3 as above; 0 before any). */
+ * where the last three-kernel pass read its schedule (1, 2 (the grouped contraction: straight from
+ * global memory) or 3 as above; 0 before any). */
 mtp_status mtp_get_split_shape(const mtp_model* model, int32_t* warps_pair, int32_t* nb_contract, int32_t* unroll,
                                int32_t* schedule, int32_t* schedule_used);
 

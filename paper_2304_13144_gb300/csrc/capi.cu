@@ -62,23 +62,26 @@ namespace {
 // Orders the terms of one round (lists[l] for lanes l) into L iterations so that, at each
 // iteration, the 32 lanes' two shared-memory operands fall into distinct banks as far as a
 // greedy choice allows (same address = broadcast, free).  `bank_a/b` map a word to the
-// word offset it reads; `swap` (optional) may exchange the two operands of a word.
+// word offset it reads; `swap` (optional) may exchange the two operands of a word.  `phase` lanes
+// are served together from `phase` banks: 32 for 32-bit operands, 8 for the 128-bit ones of the
+// grouped contraction (a quarter warp per wavefront).
 template <class BankA, class BankB, class Swap>
 std::vector<std::vector<uint32_t>> bank_order(std::vector<std::vector<uint32_t>> lists, int L, BankA bank_a,
-                                              BankB bank_b, Swap swap) {
+                                              BankB bank_b, Swap swap, uint32_t phase = 32) {
   std::vector<std::vector<uint32_t>> out(lists.size());
   for (int it = 0; it < L; ++it) {
     std::vector<std::vector<uint32_t>> addr_a(32), addr_b(32);
-    auto cost = [&](uint32_t w) {
-      const uint32_t oa = bank_a(w), ob = bank_b(w);
-      int c = 0;
-      auto& va = addr_a[oa & 31];
-      if (std::find(va.begin(), va.end(), oa) == va.end()) c += static_cast<int>(va.size());
-      auto& vb = addr_b[ob & 31];
-      if (std::find(vb.begin(), vb.end(), ob) == vb.end()) c += static_cast<int>(vb.size());
-      return c;
-    };
     for (size_t l = 0; l < lists.size(); ++l) {
+      const uint32_t bank0 = static_cast<uint32_t>(l) / phase * phase, mask = phase - 1;   // this phase's banks
+      auto cost = [&](uint32_t w) {
+        const uint32_t oa = bank_a(w), ob = bank_b(w);
+        int c = 0;
+        auto& va = addr_a[bank0 + (oa & mask)];
+        if (std::find(va.begin(), va.end(), oa) == va.end()) c += static_cast<int>(va.size());
+        auto& vb = addr_b[bank0 + (ob & mask)];
+        if (std::find(vb.begin(), vb.end(), ob) == vb.end()) c += static_cast<int>(vb.size());
+        return c;
+      };
       auto& lst = lists[l];
       if (lst.empty()) continue;
       size_t best = 0;
@@ -96,9 +99,9 @@ std::vector<std::vector<uint32_t>> bank_order(std::vector<std::vector<uint32_t>>
       }
       const uint32_t w = best_sw ? swap(lst[best]) : lst[best];
       lst.erase(lst.begin() + static_cast<long>(best));
-      auto& va = addr_a[bank_a(w) & 31];
+      auto& va = addr_a[bank0 + (bank_a(w) & mask)];
       if (std::find(va.begin(), va.end(), bank_a(w)) == va.end()) va.push_back(bank_a(w));
-      auto& vb = addr_b[bank_b(w) & 31];
+      auto& vb = addr_b[bank0 + (bank_b(w) & mask)];
       if (std::find(vb.begin(), vb.end(), bank_b(w)) == vb.end()) vb.push_back(bank_b(w));
       out[l].push_back(w);
     }
@@ -194,6 +197,9 @@ void upload_schedule(mtp_model* md) {
   // packed rounds for the three-kernel pass's contraction (same words): a long list may take an
   // aligned group of 2..32 lanes, each lane an equal share, combined by a butterfly; lane entry =
   // -1 (idle) or dst | log2(group) << 16 | leader << 20; round = {L, off, end_of_wave, grouped}
+  const size_t group_bytes = 32 * static_cast<size_t>(padded_nv(nv));   // values and adjoints of four neighborhoods
+  const int group_warps = 12 * group_bytes <= 227 * 1024 && nm <= 160 ? kGroupWarpsSmall
+                          : (4 * group_bytes <= 227 * 1024 && nm <= 320 ? kGroupWarpsMid : kGroupWarpsLarge);
   std::vector<uint32_t> pfslab, prslab;
   std::vector<int> pfr_dst, prr_val, pfround, prround;
   if (packable) {
@@ -245,7 +251,7 @@ void upload_schedule(mtp_model* md) {
     auto pack_wave = [&](const std::vector<int>& items, auto&& list_of, std::vector<uint32_t>& slab,
                          std::vector<int>& lane_item, std::vector<int>& rounds, auto&& bank_a, auto&& bank_b,
                          auto&& swap) {
-      constexpr double kRoundCost = 300.0;
+      const double kRoundCost = group_warps == kGroupWarpsLarge ? 60.0 : 300.0;   // (more rounds balance better)
       auto np2 = [](int x) { int g = 1; while (g < x) g *= 2; return g; };
       const int n = static_cast<int>(items.size());
       int i = 0;
@@ -293,7 +299,7 @@ void upload_schedule(mtp_model* md) {
         }
         rounds.insert(rounds.end(), {L, static_cast<int>(slab.size()), j == n ? 1 : 0, grouped ? 1 : 0});
         lane_item.insert(lane_item.end(), entry.begin(), entry.end());
-        auto ord = bank_order(lists, L, bank_a, bank_b, swap);
+        auto ord = bank_order(lists, L, bank_a, bank_b, swap, 8);
         for (int it = 0; it < L; ++it)
           for (int l = 0; l < 32; ++l) slab.push_back(it < static_cast<int>(ord[l].size()) ? ord[l][it] : pad);
         i = j;
@@ -404,7 +410,72 @@ void upload_schedule(mtp_model* md) {
     for (int x : S.basis_idx)
       if (x < 0 || x >= nv) bad("basis values");
   }
+  // the packed rounds dealt to the warps of a group of the grouped contraction: each wave's rounds
+  // go longest first to the warp with the least work (rows and a round's fixed cost)
+  std::vector<uint32_t> gslab;
+  std::vector<int2> ground;
+  std::vector<uint16_t> gent;
+  std::vector<int4> gmeta;
+  if (packable) {
+    constexpr long kRoundRows = 4;
+    struct Mine { std::vector<int> f, r; };   // packed rounds, -1 = an empty one that ends the wave
+    std::vector<Mine> mine(group_warps);
+    auto deal = [&](const std::vector<int>& rounds, std::vector<int> Mine::* part) {
+      const int n = static_cast<int>(rounds.size() / 4);
+      for (int r0 = 0; r0 < n;) {
+        int r1 = r0;
+        while (r1 < n && !rounds[4 * r1 + 2]) ++r1;
+        r1 = std::min(n, r1 + 1);
+        std::vector<int> order(r1 - r0);
+        for (int k = r0; k < r1; ++k) order[k - r0] = k;
+        if (group_warps > 1)
+          std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return rounds[4 * a] > rounds[4 * b]; });
+        std::vector<long> load(group_warps, 0);
+        for (int k : order) {
+          const int w = static_cast<int>(std::min_element(load.begin(), load.end()) - load.begin());
+          (mine[w].*part).push_back(k);
+          load[w] += rounds[4 * k] + kRoundRows;
+        }
+        for (int w = 0; w < group_warps; ++w) (mine[w].*part).push_back(-1);
+        r0 = r1;
+      }
+    };
+    deal(pfround, &Mine::f);
+    deal(prround, &Mine::r);
+    for (int w = 0; w < group_warps; ++w) {
+      int4 meta;
+      meta.x = static_cast<int>(ground.size());
+      meta.w = static_cast<int>(gslab.size() / 32);
+      auto emit = [&](const std::vector<int>& list, const std::vector<int>& rounds, const std::vector<int>& entries,
+                      const std::vector<uint32_t>& slab) {
+        const size_t first = ground.size();
+        for (int k : list) {
+          if (k < 0) {   // ends the wave: the flag goes to the warp's last round of it, if it has one
+            if (ground.size() > first && !(ground.back().y & 1)) { ground.back().y |= 1; continue; }
+            ground.push_back(make_int2(0, 1));
+            gent.insert(gent.end(), 32, 0);
+            continue;
+          }
+          int steps = 0;
+          for (int l = 0; l < 32; ++l) {
+            const int e = entries[32 * k + l];
+            const int lg = e < 0 ? 0 : (e >> 16) & 15;
+            steps = std::max(steps, lg);
+            gent.push_back(static_cast<uint16_t>(e < 0 ? 0 : (e & 4095) | (lg << 12) | (((e >> 20) & 1) << 15)));
+          }
+          ground.push_back(make_int2(rounds[4 * k], steps << 1));
+          gslab.insert(gslab.end(), slab.begin() + rounds[4 * k + 1], slab.begin() + rounds[4 * k + 1] + 32 * rounds[4 * k]);
+        }
+        return static_cast<int>(ground.size() - first);
+      };
+      meta.y = emit(mine[w].f, pfround, pfr_dst, pfslab);
+      meta.z = emit(mine[w].r, prround, prr_val, prslab);
+      gmeta.push_back(meta);
+      gslab.insert(gslab.end(), 32 * kGroupPad, 0u);
+    }
+  }
   std::vector<char> blob;
+  const size_t o_gs = put(blob, gslab), o_gr = put(blob, ground), o_ge = put(blob, gent), o_gm = put(blob, gmeta);
   const size_t o_tpk = put(blob, tri_pk), o_upk = put(blob, use_pk), o_cf = put(blob, coef_f);
   const size_t o_fs = put(blob, fslab), o_fr = put(blob, fround), o_frd = put(blob, fr_dst), o_rs = put(blob, rslab),
                o_rr = put(blob, rround), o_rrv = put(blob, rr_val);
@@ -465,6 +536,13 @@ void upload_schedule(mtp_model* md) {
   D.prr_val = reinterpret_cast<const int*>(base + o_prv);
   D.n_prround = static_cast<int>(prround.size() / 4);
   D.prslab_words = static_cast<int>(prslab.size());
+  D.gslab = packable ? reinterpret_cast<const uint32_t*>(base + o_gs) : nullptr;
+  D.ground = reinterpret_cast<const int2*>(base + o_gr);
+  D.gent = reinterpret_cast<const uint16_t*>(base + o_ge);
+  D.gmeta = reinterpret_cast<const int4*>(base + o_gm);
+  D.n_ground = static_cast<int>(ground.size());
+  D.n_grows = static_cast<int>(gslab.size() / 32);
+  D.group_warps = group_warps;
 }
 
 void upload_theta(mtp_model* md) {
@@ -830,40 +908,31 @@ mtp_status mtp_autotune(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mt
       }
     }
     // the three-kernel mixed pass, when the model has one: warps per block of its per-pair
-    // kernels x neighborhoods per warp of its contraction x words in flight x schedule placement
-    // (results are the same for every shape)
-    int best_sw = 0, best_snb = 0, best_sun = 0, best_sg = 0;
+    // kernels (its contraction: the grouped one, faster at every level than the shapes of
+    // mtp_set_split_shape; results are the same for every shape)
+    int best_sw = 0;
     float best_split = 0.f;
     const int keep_split = md->tune_split;
     md->mixed_pass = keep_pass;
     if (split_ok) {
       md->tune_split = 1;
-      for (int sg : {1, 2, 3})
-      for (int sw : {4, 8})
-        for (int sc : {12, 14, 22, 24, 28}) {
-          const int snb = sc / 10, sun = sc % 10;
-          // level 24 (6 radial functions): only the streamed schedule applies
-          if (md->ds.n_rad >= 6 && (sg != 2 || sun == 8)) continue;
-          md->tune_split_warps = sw;
-          md->tune_split_nb = snb;
-          md->tune_split_unroll = sun;
-          md->tune_split_sched = sg;
+      md->tune_split_nb = md->tune_split_unroll = md->tune_split_sched = 0;   // the grouped contraction
+      for (int sw : {4, 8}) {
+        md->tune_split_warps = sw;
+        run();
+        if (!md->last_split) continue;
+        float t_min = 0.f;
+        for (int rep = 0; rep < 3; ++rep) {
+          MTP_CUDA(cudaEventRecord(e0, s));
           run();
-          if (!md->last_split || md->last_split_sched != sg) continue;   // placement unavailable
-          float t_min = 0.f;
-          for (int rep = 0; rep < 3; ++rep) {
-            MTP_CUDA(cudaEventRecord(e0, s));
-            run();
-            MTP_CUDA(cudaEventRecord(e1, s));
-            MTP_CUDA(cudaEventSynchronize(e1));
-            float t = 0.f;
-            MTP_CUDA(cudaEventElapsedTime(&t, e0, e1));
-            if (rep == 0 || t < t_min) t_min = t;
-          }
-          if (best_sw == 0 || t_min < best_split) {
-            best_split = t_min; best_sw = sw; best_snb = snb; best_sun = sun; best_sg = sg;
-          }
+          MTP_CUDA(cudaEventRecord(e1, s));
+          MTP_CUDA(cudaEventSynchronize(e1));
+          float t = 0.f;
+          MTP_CUDA(cudaEventElapsedTime(&t, e0, e1));
+          if (rep == 0 || t < t_min) t_min = t;
         }
+        if (best_sw == 0 || t_min < best_split) { best_split = t_min; best_sw = sw; }
+      }
       md->tune_split = keep_split;
     }
     MTP_CUDA(cudaEventDestroy(e0));
@@ -872,9 +941,6 @@ mtp_status mtp_autotune(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mt
     if (fast) md->tune_fwd_global = best_p;
     if (best_sw > 0) {
       md->tune_split_warps = best_sw;
-      md->tune_split_nb = best_snb;
-      md->tune_split_unroll = best_sun;
-      md->tune_split_sched = best_sg;
       const bool split = md->mixed_pass == 2 || best_split < best_ms;
       if (md->mixed_pass == 0) md->tune_split = split ? 1 : 0;
       if (split) best_ms = best_split;

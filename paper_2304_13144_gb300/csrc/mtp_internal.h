@@ -101,6 +101,16 @@ struct DevSchedule {
   const int4* prround;
   const int* prr_val;
   int n_prround, prslab_words;
+  // the same packed rounds for the grouped contraction (site_group.cu), dealt to group_warps warps
+  // (each wave's rounds balanced over them): per warp meta = {first round, forward rounds, reverse
+  // rounds, first row}, round = {L, end_of_wave | butterfly steps << 1}, its 32 lane entries of 16
+  // bits (index | log2(group) << 12 | leader << 15, 0 = idle); a warp's rows follow one another in
+  // gslab in the order of its rounds, kGroupPad rows of padding after them
+  const uint32_t* gslab;
+  const int2* ground;
+  const uint16_t* gent;
+  const int4* gmeta;
+  int n_ground, n_grows, group_warps;
   const double* theta_d;    // [n_params]
   const float* theta_f;
   const double* seed_d;     // [n_vals] sum of xi over basis functions stored at that value
@@ -283,6 +293,13 @@ extern std::atomic<int> g_inject_alloc;
 extern std::atomic<int> g_inject_overflow;
 extern std::atomic<int> g_inject_grade_wait;
 bool take_injected(std::atomic<int>& c);
+// Warps per group of the grouped contraction (site_group.cu), by how many groups' arrays fit an SM:
+// 16 at level 16 and below (a warp each), 6 at level 20, 1 at level 24.  Measured, ms per pass:
+// level 16, 128,000 atoms: 1 warp 0.215, 2 warps 0.238; level 20, 1,048,576 atoms: 1 warp 11.9,
+// 2 warps 8.26, 3 warps 7.37, 4 warps 7.62 (latency hidden against waves of a few rounds only);
+// level 24, 131,072 atoms: 8 warps 6.50, 12 warps 5.72, 16 warps 5.64 (128 registers).
+constexpr int kGroupWarpsSmall = 1, kGroupWarpsMid = 3, kGroupWarpsLarge = 12;
+constexpr int kGroupPad = 4;   // rows of padding after each warp's word stream (grouped contraction)
 // per-neighborhood value slots of the specialised kernel's shared-memory arrays: the values,
 // one always-zero slot (index n_values), padded to a multiple of 4
 inline int padded_nv(int n_values) { return (n_values + 1 + 3) & ~3; }

@@ -29,6 +29,7 @@
 
 #include "mtp_internal.h"
 #include "profiler.h"
+#include "site_group.h"
 #include "site_shape.h"
 
 namespace mtp {
@@ -985,8 +986,8 @@ int num_sms() {
 }
 
 template <int NR, int NU0>
-void launch_split(SplitArgs P, int warps_pair, int nb_contract, int unroll, int sch, bool efs, bool rows,
-                  cudaStream_t s) {
+int launch_split(SplitArgs P, int warps_pair, int nb_contract, int unroll, int sch, bool efs, bool rows,
+                 cudaStream_t s) {
   const int nsm = num_sms();
   const int64_t groups = (P.n_work + GPW - 1) / GPW;
   // ---- moments ----
@@ -1003,7 +1004,9 @@ void launch_split(SplitArgs P, int warps_pair, int nb_contract, int unroll, int 
     MTP_CUDA(cudaGetLastError());
   }
   // ---- contraction ----
-  {
+  if (sch == 0) {
+    sch = run_contract_group(P.d, P.o, P.type, P.n_work, P.mom, P.ldm, P.slot_comp, s);
+  } else {
     const size_t sched = sch == 2 ? ring_bytes() : (sch == 3 ? P.ovf_bytes : P.sched_bytes);
     const int wpb = std::max(1, static_cast<int>((227 * 1024 - P.c_bytes - sched) / P.warp_bytes));
     // the streamed variant is built for <= 256 threads, the tensor-memory one for <= 384
@@ -1068,6 +1071,7 @@ void launch_split(SplitArgs P, int warps_pair, int nb_contract, int unroll, int 
     if (rows) go(k_adjoint<NR, NU0, true>);
     else go(k_adjoint<NR, NU0, false>);
   }
+  return sch;
 }
 
 template <int NR, int NU0>
@@ -1149,26 +1153,30 @@ bool run_sites_split(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, const 
                                      32 * d.n_prround + ((d.n_vals + 3) & ~3)) * 4;   // headers, lane entries, seeds
   const bool fits = P.c_bytes + P.sched_bytes + 4 * P.warp_bytes <= 227 * 1024;
   const int ask = m->tune_split_sched;
-  int sch = fits ? 1 : 2;
+  // 0: the grouped contraction (site_group.cu), unless a shape was asked for
+  int sch = (ask == 0 && m->tune_split_nb == 0 && m->tune_split_unroll == 0 && contract_group_available(d)) ? 0
+                                                                                                          : (fits ? 1 : 2);
   if (ask == 2) sch = 2;
   if (ask == 3 && nr < 6 && P.c_bytes + P.ovf_bytes + 4 * P.warp_bytes <= 227 * 1024) sch = 3;
-  if ((nr >= 6 && sch != 2) || (nr >= 6 && d.coef_inline)) return false;
-  if (sch != 1 && (d.pfslab_words % 32 != 0 || d.prslab_words % 32 != 0)) return false;   // whole rows
-  const size_t sbytes = sch == 2 ? ring_bytes() : (sch == 3 ? P.ovf_bytes : P.sched_bytes);
-  if (P.c_bytes + sbytes + P.warp_bytes > 227 * 1024) return false;
-  P.total = P.c_bytes + sbytes + P.warp_bytes;
+  if (nr >= 6 && d.coef_inline) return false;
+  if (sch != 0) {
+    if (nr >= 6 && sch != 2) return false;
+    if (sch != 1 && (d.pfslab_words % 32 != 0 || d.prslab_words % 32 != 0)) return false;   // whole rows
+    const size_t sbytes = sch == 2 ? ring_bytes() : (sch == 3 ? P.ovf_bytes : P.sched_bytes);
+    if (P.c_bytes + sbytes + P.warp_bytes > 227 * 1024) return false;
+    P.total = P.c_bytes + sbytes + P.warp_bytes;
+  }
   const int wp = m->tune_split_warps > 0 ? m->tune_split_warps : 8;
   m->last_fast = true;
   m->last_split = true;
-  m->last_split_sched = sch;
   m->last_warps = wp;
   if (P.n_work == 0) return true;
   const int unr = m->tune_split_unroll == 4 ? 4 : (m->tune_split_unroll == 8 && nbc == 2 ? 8 : 2);
-  if (nr == 2) launch_split<2, 2>(P, wp, nbc, unr, sch, efs, rows, s);
-  else if (nr == 3) launch_split<3, 4>(P, wp, nbc, unr, sch, efs, rows, s);
-  else if (nr == 4) launch_split<4, 6>(P, wp, nbc, unr, sch, efs, rows, s);
-  else if (nr == 5) launch_split<5, 8>(P, wp, nbc, unr, sch, efs, rows, s);
-  else launch_split<6, 10>(P, wp, nbc, unr, sch, efs, rows, s);
+  if (nr == 2) m->last_split_sched = launch_split<2, 2>(P, wp, nbc, unr, sch, efs, rows, s);
+  else if (nr == 3) m->last_split_sched = launch_split<3, 4>(P, wp, nbc, unr, sch, efs, rows, s);
+  else if (nr == 4) m->last_split_sched = launch_split<4, 6>(P, wp, nbc, unr, sch, efs, rows, s);
+  else if (nr == 5) m->last_split_sched = launch_split<5, 8>(P, wp, nbc, unr, sch, efs, rows, s);
+  else m->last_split_sched = launch_split<6, 10>(P, wp, nbc, unr, sch, efs, rows, s);
 #ifdef MTP_SPLIT_CHECK
   unsigned long long fault = 0;
   MTP_CUDA(cudaStreamSynchronize(s));
