@@ -1388,10 +1388,8 @@ mtp_status mtp_extract_neighborhoods(const mtp_nbr* nb, const mtp_batch* b, cons
   return guarded([&] {
     if (!nb || !b || !off || !total || (n > 0 && !idx)) throw Fail{MTP_ERR_ARG, "null argument"};
     if (n < 0) throw Fail{MTP_ERR_ARG, "negative count"};
-    DevBuf tmp;
-    const int64_t t = run_extract(nb, b, idx, n, off, r, type, j, capacity, tmp, as_stream(stream));
+    const int64_t t = run_extract(nb, b, idx, n, off, r, type, j, capacity, as_stream(stream));
     MTP_CUDA(cudaStreamSynchronize(as_stream(stream)));
-    tmp.release();
     *total = t;
     if (t > capacity) throw Fail{MTP_ERR_CAPACITY, "extraction needs " + std::to_string(t) + " neighbor slots"};
   });

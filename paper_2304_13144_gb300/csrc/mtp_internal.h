@@ -44,6 +44,16 @@ struct DevBuf {
   void release();
   template <class T> T* as() const { return static_cast<T*>(p); }
 };
+// one call's workspace, given back in stream order when the call returns or throws
+struct ScopedBuf : DevBuf {
+  explicit ScopedBuf(cudaStream_t stream) : s(stream) {}
+  ~ScopedBuf() {
+    if (p) cudaFreeAsync(p, s);
+  }
+  ScopedBuf(const ScopedBuf&) = delete;
+  ScopedBuf& operator=(const ScopedBuf&) = delete;
+  cudaStream_t s;
+};
 
 // ------------------------------------------------------------------------------------
 // schedule and parameters on the device (one copy per model)
@@ -317,7 +327,7 @@ void run_grade(mtp_model* m, int64_t N, bool fp64, const double* rows, const flo
 void run_flag(int64_t N, const double* gamma, double threshold, int32_t* flagged, int64_t* n_flagged,
               DevBuf& tmp, cudaStream_t s);
 int64_t run_extract(const mtp_nbr* nb, const mtp_batch* b, const int32_t* idx, int64_t n, int64_t* off,
-                    double* r, int32_t* type, int32_t* j, int64_t capacity, DevBuf& tmp, cudaStream_t s);
+                    double* r, int32_t* type, int32_t* j, int64_t capacity, cudaStream_t s);
 void run_train_prep(const mtp_nbr* nb, int n_cfg, const double* E, const double* F, const double* W,
                     const double* E_ref, const double* F_ref, const double* W_ref, double w_e,
                     double w_f, double w_s, double* coef, double* U, double* Scfg, double* loss,

@@ -147,18 +147,21 @@ __global__ void k_extract_counts(DevNbr nb, const int32_t* idx, int64_t n, long 
   cnt[k] = nb.off[i + 1] - nb.off[i];
 }
 
+// a warp per atom, a lane per pair: 2,000 atoms' pairs by one thread per atom were a serial chain
+// of dependent loads
 __global__ void k_extract_fill(DevNbr nb, const double* pos, const int* type, const double* cell,
                                const int32_t* idx, int64_t n, const long long* off, double* r, int32_t* ty,
                                int32_t* jout) {
-  int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  const int64_t k = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
   if (k >= n) return;
   const int i = idx[k];
   if (i < 0 || i >= nb.n_atoms) return;
   const double* H = cell + 9 * nb.atom_cfg[i];
-  int64_t o = off[k];
-  for (int64_t p = nb.off[i]; p < nb.off[i + 1]; ++p, ++o) {
-    const int j = nb.pj[p];
-    const int img = nb.pimg[p];
+  const int64_t p0 = nb.off[i], np = nb.off[i + 1] - p0;
+  for (int64_t t = threadIdx.x & 31; t < np; t += 32) {
+    const int64_t o = off[k] + t;
+    const int j = nb.pj[p0 + t];
+    const int img = nb.pimg[p0 + t];
     const int n0 = unpack_img(img, 0), n1 = unpack_img(img, 1), n2 = unpack_img(img, 2);
     if (r)
       for (int c = 0; c < 3; ++c) {
@@ -308,30 +311,29 @@ void run_flag(int64_t N, const double* gamma, double threshold, int32_t* flagged
 }
 
 int64_t run_extract(const mtp_nbr* nb, const mtp_batch* b, const int32_t* idx, int64_t n, int64_t* off, double* r,
-                    int32_t* type, int32_t* j, int64_t capacity, DevBuf& tmp, cudaStream_t s) {
-  tmp.ensure((n + 1) * sizeof(long long) + 64, s);
-  long long* cnt = tmp.as<long long>();
+                    int32_t* type, int32_t* j, int64_t capacity, cudaStream_t s) {
+  size_t bytes = 0;
+  long long* offl = reinterpret_cast<long long*>(off);
+  MTP_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, bytes, offl, offl, n + 1, s));
+  ScopedBuf work(s);   // counts, the error flag, the scan's scratch
+  const size_t at = ((n + 1) * sizeof(long long) + 16 + 255) & ~size_t(255);
+  work.ensure(at + bytes, s);
+  long long* cnt = work.as<long long>();
   unsigned* bad = reinterpret_cast<unsigned*>(cnt + n + 1);
   MTP_CUDA(cudaMemsetAsync(bad, 0, sizeof(unsigned), s));
   k_extract_counts<<<nblk(n + 1, 256), 256, 0, s>>>(nb->dn, idx, n, cnt, bad);
   ProfRegion::launched();
   MTP_CUDA(cudaGetLastError());
-  DevBuf scan_tmp;
-  size_t bytes = 0;
-  long long* offl = reinterpret_cast<long long*>(off);
-  MTP_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, bytes, cnt, offl, n + 1, s));
-  scan_tmp.ensure(bytes, s);
-  MTP_CUDA(cub::DeviceScan::ExclusiveSum(scan_tmp.p, bytes, cnt, offl, n + 1, s));
+  MTP_CUDA(cub::DeviceScan::ExclusiveSum(reinterpret_cast<char*>(work.p) + at, bytes, cnt, offl, n + 1, s));
   long long total = 0;
   unsigned badh = 0;
   MTP_CUDA(cudaMemcpyAsync(&total, offl + n, sizeof(long long), cudaMemcpyDeviceToHost, s));
   MTP_CUDA(cudaMemcpyAsync(&badh, bad, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
   MTP_CUDA(cudaStreamSynchronize(s));
-  scan_tmp.release();
   if (badh) throw Fail{MTP_ERR_ARG, "atom index out of range"};
   if (total > capacity) return total;
   if (n > 0) {
-    k_extract_fill<<<nblk(n, 128), 128, 0, s>>>(nb->dn, b->pos, b->type, b->cell, idx, n, offl, r, type, j);
+    k_extract_fill<<<nblk(n * 32, 128), 128, 0, s>>>(nb->dn, b->pos, b->type, b->cell, idx, n, offl, r, type, j);
     ProfRegion::launched();
     MTP_CUDA(cudaGetLastError());
   }

@@ -87,3 +87,14 @@ def test_cut_errors(api):
         api.mtp_cut_clusters(b, torch.tensor([0]), 0.0)
     out = api.mtp_cut_clusters(b, torch.tensor([], dtype=torch.int64), 8.0)
     assert out["off"].cpu().numpy().tolist() == [0] and len(out["src"]) == 0
+
+
+@pytest.mark.parametrize("reps,n_centers,radius", [((2, 12, 2), 1, 8.0), ((9, 5, 4), 7, 5.3), ((1, 1, 1), 2, 8.0), ((12, 9, 2), 200, 6.0)])
+def test_cut_skewed_cells_and_split_ranges(api, reps, n_centers, radius):
+    """Elongated non-orthogonal cells (images far from the center's along the skewed axes) and one
+    to many ranges of atoms per center."""
+    g = synth.rng(71)
+    pos, cell, _ = synth.hcp_supercell(2.55, 2.55 * 1.633, reps)
+    bnp = synth.single(pos + g.normal(0, 0.05, pos.shape), g.integers(0, 3, len(pos)), cell)
+    centers = g.integers(0, len(pos), n_centers)
+    check_against_oracle(api.mtp_cut_clusters(api.Batch(bnp), torch.tensor(centers), radius), bnp, centers, radius)
