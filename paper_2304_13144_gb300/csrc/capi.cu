@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "mtp_internal.h"
+#include "site_wide.h"
 
 namespace mtp {
 
@@ -191,6 +192,12 @@ void upload_schedule(mtp_model* md) {
   std::vector<float> coef_f(coefs.begin(), coefs.end());
   coef_f.push_back(0.0f);   // coefficient of the padding terms
   const uint32_t zero_ci = static_cast<uint32_t>(coef_f.size() - 1);
+  // words of the FP64 / dual-number pass (site_wide.cu): the packed rounds' lists, unit coefficients
+  // last, padded with 1 * 0 * 0 (the always-zero slot n_vals)
+  std::vector<uint32_t> wfslab, wrslab;
+  const auto one = std::find(coefs.begin(), coefs.end(), 1.0);
+  const uint32_t unit_ci = static_cast<uint32_t>(one - coefs.begin());
+  const bool wide_ok = packable && nv + 1 <= 4096 && one != coefs.end();
   std::vector<uint32_t> fslab, rslab;
   std::vector<int> fr_dst, rr_val;
   std::vector<int> fround, rround;   // 4 ints per round
@@ -249,8 +256,8 @@ void upload_schedule(mtp_model* md) {
     // and the L that minimises (32 L + kRoundCost) per term, kRoundCost being the fixed cost of a
     // round in slot units
     auto pack_wave = [&](const std::vector<int>& items, auto&& list_of, std::vector<uint32_t>& slab,
-                         std::vector<int>& lane_item, std::vector<int>& rounds, auto&& bank_a, auto&& bank_b,
-                         auto&& swap) {
+                         std::vector<int>& lane_item, std::vector<int>& rounds, std::vector<uint32_t>& wslab,
+                         auto&& bank_a, auto&& bank_b, auto&& swap) {
       const double kRoundCost = group_warps == kGroupWarpsLarge ? 60.0 : 300.0;   // (more rounds balance better)
       auto np2 = [](int x) { int g = 1; while (g < x) g *= 2; return g; };
       const int n = static_cast<int>(items.size());
@@ -299,6 +306,16 @@ void upload_schedule(mtp_model* md) {
         }
         rounds.insert(rounds.end(), {L, static_cast<int>(slab.size()), j == n ? 1 : 0, grouped ? 1 : 0});
         lane_item.insert(lane_item.end(), entry.begin(), entry.end());
+        if (wide_ok) {
+          const uint32_t wpad = static_cast<uint32_t>(nv) | (static_cast<uint32_t>(nv) << 12) | (unit_ci << 24);
+          const size_t at = wslab.size();
+          wslab.resize(at + 32 * static_cast<size_t>(L), wpad);
+          for (int l = 0; l < 32; ++l) {
+            auto lst = lists[l];
+            std::stable_partition(lst.begin(), lst.end(), [&](uint32_t w) { return (w >> 24) != unit_ci; });
+            for (size_t t = 0; t < lst.size(); ++t) wslab[at + 32 * t + l] = lst[t];
+          }
+        }
         auto ord = bank_order(lists, L, bank_a, bank_b, swap, 8);
         for (int it = 0; it < L; ++it)
           for (int l = 0; l < 32; ++l) slab.push_back(it < static_cast<int>(ord[l].size()) ? ord[l][it] : pad);
@@ -320,13 +337,13 @@ void upload_schedule(mtp_model* md) {
       for (int wv = 0; wv + 1 < static_cast<int>(fwave_ptr.size()); ++wv) {
         std::vector<int> items(fdst.begin() + fwave_ptr[wv], fdst.begin() + fwave_ptr[wv + 1]);
         pack_wave(by_len(flist, items), [&](int x) -> const std::vector<uint32_t>& { return flist[x]; }, pfslab,
-                  pfr_dst, pfround, [](uint32_t w) { return w & 4095u; }, [](uint32_t w) { return (w >> 12) & 4095u; },
+                  pfr_dst, pfround, wfslab, [](uint32_t w) { return w & 4095u; }, [](uint32_t w) { return (w >> 12) & 4095u; },
                   [](uint32_t w) { return (w & 0xff000000u) | ((w & 4095u) << 12) | ((w >> 12) & 4095u); });
       }
       for (int wv = 0; wv + 1 < static_cast<int>(rwave_ptr.size()); ++wv) {
         std::vector<int> items(rval.begin() + rwave_ptr[wv], rval.begin() + rwave_ptr[wv + 1]);
         pack_wave(by_len(rlist, items), [&](int x) -> const std::vector<uint32_t>& { return rlist[x]; }, prslab,
-                  prr_val, prround, [](uint32_t w) { return w & 4095u; },
+                  prr_val, prround, wrslab, [](uint32_t w) { return w & 4095u; },
                   [gofs](uint32_t w) { return gofs + ((w >> 12) & 4095u); }, [](uint32_t w) { return w; });
       }
     }
@@ -374,6 +391,9 @@ void upload_schedule(mtp_model* md) {
         bad(what);
       }
     };
+    for (const auto* ws : {&wfslab, &wrslab})
+      for (uint32_t w : *ws)
+        if ((w & 4095u) > unv || ((w >> 12) & 4095u) > unv || (w >> 24) >= ncf) bad("unit-last slab");
     for (uint32_t w : fslab) check_word(w, "forward slab");
     for (uint32_t w : rslab) check_word(w, "reverse slab");
     for (uint32_t w : pfslab) check_word(w, "packed forward slab");
@@ -476,6 +496,9 @@ void upload_schedule(mtp_model* md) {
   }
   std::vector<char> blob;
   const size_t o_gs = put(blob, gslab), o_gr = put(blob, ground), o_ge = put(blob, gent), o_gm = put(blob, gmeta);
+  std::vector<double> coef_d(coefs);
+  coef_d.push_back(0.0);
+  const size_t o_wf = put(blob, wfslab), o_wr = put(blob, wrslab), o_cd = put(blob, coef_d);
   const size_t o_tpk = put(blob, tri_pk), o_upk = put(blob, use_pk), o_cf = put(blob, coef_f);
   const size_t o_fs = put(blob, fslab), o_fr = put(blob, fround), o_frd = put(blob, fr_dst), o_rs = put(blob, rslab),
                o_rr = put(blob, rround), o_rrv = put(blob, rr_val);
@@ -543,6 +566,14 @@ void upload_schedule(mtp_model* md) {
   D.n_ground = static_cast<int>(ground.size());
   D.n_grows = static_cast<int>(gslab.size() / 32);
   D.group_warps = group_warps;
+  md->wide_words = {};
+  if (wide_ok) {
+    md->wide_words.f = reinterpret_cast<const uint32_t*>(base + o_wf);
+    md->wide_words.r = reinterpret_cast<const uint32_t*>(base + o_wr);
+    md->wide_words.coef = reinterpret_cast<const double*>(base + o_cd);
+    md->wide_words.n_coef = D.n_coef;
+    md->wide_words.unit = static_cast<int>(unit_ci);
+  }
 }
 
 void upload_theta(mtp_model* md) {
@@ -628,6 +659,14 @@ void check_model(const mtp_model* m) {
   if (dev != m->device) throw Fail{MTP_ERR_ARG, "model belongs to another device"};
 }
 
+// the workspace of the FP64 / dual-number pass, where the model has it
+void give_wide(mtp_model* m, int64_t n_work, bool fp64, bool tangent, SiteOutputs& o, cudaStream_t s) {
+  const size_t bytes = wide_workspace(m, n_work, fp64, tangent);
+  if (!bytes) return;
+  m->ws_wide.ensure(bytes, s);
+  o.wide = m->ws_wide.p;
+}
+
 // Shared body of the EFS / grade / step entry points.
 void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec, double* energy,
                    double* site_energy, double* forces, double* virial, double threshold, double* gamma,
@@ -655,6 +694,7 @@ void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_prec
     m->ws_mom.ensure(std::max<int64_t>(N, 1) * split_ldm(m->ds.n_mom) * sizeof(float), s);
     o.mom = m->ws_mom.as<float>();
   }
+  if (fp64) give_wide(m, N, true, false, o, s);
   int64_t ld = 0;
   const bool use_tc = !fp64 && want_grade && grade_tc_available(m);
   if (want_grade) {
@@ -793,6 +833,7 @@ mtp_status mtp_load(const mtp_desc* desc, const double* theta, int64_t m, mtp_mo
       upload_schedule(md);
       upload_theta(md);
       split_prepare(md);
+      wide_prepare(md);
       noalloc_prepare(md->device);
       md->async_err.ensure(sizeof(unsigned), 0);
       MTP_CUDA(cudaMemset(md->async_err.p, 0, sizeof(unsigned)));
@@ -813,7 +854,7 @@ void mtp_free_model(mtp_model* md) {
   cudaDeviceSynchronize();
   for (DevBuf* b : {&md->sched_buf, &md->theta_buf, &md->a_d, &md->ainv_d, &md->ainv_f, &md->ws_pair,
                     &md->ws_atom, &md->ws_rows, &md->ws_grade, &md->ws_sort, &md->ws_misc, &md->ws_red,
-                    &md->err_flag, &md->async_err, &md->split_tab, &md->ws_mom})
+                    &md->err_flag, &md->async_err, &md->split_tab, &md->ws_mom, &md->wide_tab, &md->ws_wide})
     b->release();
   cudaSetDevice(cur);
   delete md;
@@ -1291,6 +1332,7 @@ mtp_status mtp_config_rows(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb,
     SiteOutputs o;
     o.rows = md->ws_rows.as<double>();
     o.rows_ld = m;
+    give_wide(md, N, prec == MTP_FP64, false, o, s);
     run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
     run_config_row_sums(nb, md->ws_rows.as<double>(), m, rows, md->ws_red, s);
   });
@@ -1314,6 +1356,7 @@ mtp_status mtp_energy_vjp(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
       SiteOutputs o;
       o.rows = md->ws_rows.as<double>();
       o.rows_ld = m;
+      give_wide(md, N, prec == MTP_FP64, false, o, s);
       run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
       run_config_row_sums(nb, md->ws_rows.as<double>(), m, R, md->ws_red, s);
     }
@@ -1348,6 +1391,7 @@ mtp_status mtp_config_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb
       SiteOutputs o;
       o.rows = md->ws_rows.as<double>();
       o.rows_ld = m;
+      give_wide(md, N, prec == MTP_FP64, false, o, s);
       run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
       run_config_row_sums(nb, md->ws_rows.as<double>(), m, rc, md->ws_red, s);
       run_grade_simt(md, K, true, rc, nullptr, m, gamma_cfg, am, s);
@@ -1378,6 +1422,7 @@ mtp_status mtp_param_rows(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     o.rows_ld = md->sched.n_params;
     o.atom_list = atoms;
     o.n_list = atoms ? n : nb->n_atoms;
+    give_wide(md, o.n_list, prec == MTP_FP64, false, o, as_stream(stream));
     run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, as_stream(stream));
   });
 }
@@ -1440,6 +1485,12 @@ mtp_status mtp_train_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     double* Sc = coef + n_cfg;
     SiteOutputs o;
     o.V = V; o.Wat = Wat; o.G = md->ws_pair.p;
+    if (fp64) {
+      give_wide(md, N, true, false, o, s);
+    } else if (split_wanted(md)) {
+      md->ws_mom.ensure(std::max<int64_t>(N, 1) * split_ldm(md->ds.n_mom) * sizeof(float), s);
+      o.mom = md->ws_mom.as<float>();
+    }
     run_sites(md, b, nb, fp64, o, false, nullptr, s);
     run_forces(nb, fp64, o.G, F, s);
     run_config_sums(nb, V, Wat, E, W, md->ws_red, s);
@@ -1458,9 +1509,14 @@ mtp_status mtp_train_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     md->ws_rows.ensure(part_bytes, s);
     MTP_CUDA(cudaMemsetAsync(md->ws_rows.p, 0, part_bytes, s));
     t.grad_part = md->ws_rows.as<double>();
-    int used = gmax;
-    run_sites(md, b, nb, fp64, t, true, &used, s);
-    run_sum_rows(t.grad_part, used * rows_per_block, m, grad, s);
+    give_wide(md, N, fp64, true, t, s);
+    int64_t part_rows = 0;
+    if (!run_sites_wide(md, b, nb, fp64, t, true, gmax * rows_per_block, &part_rows, s)) {
+      int used = gmax;
+      run_sites(md, b, nb, fp64, t, true, &used, s);
+      part_rows = static_cast<int64_t>(used) * rows_per_block;
+    }
+    run_sum_rows(t.grad_part, static_cast<int>(part_rows), m, grad, s);
   });
 }
 

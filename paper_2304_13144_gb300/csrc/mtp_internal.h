@@ -228,6 +228,22 @@ struct mtp_model {
                                // memory, 2 = streamed through a shared ring, 3 = tensor memory
   bool last_split = false;
   int last_split_sched = 0;   // where the last three-kernel pass read its schedule (1, 2 or 3 as above)
+  // tables of the FP64 / dual-number pass (site_wide.cu), uploaded by mtp_load; slot_comp is null
+  // for shapes without it
+  struct {
+    const int *slot_comp = nullptr, *slot_mk = nullptr, *mono = nullptr, *ab = nullptr;
+    int n_mono = 0, n_ab = 0;
+    std::vector<int> numax;
+  } wide;
+  // its schedule words: those of the packed rounds as a | b << 12 | coefficient << 24, unit
+  // coefficients last (n_coef = 0: not packable)
+  struct {
+    const uint32_t *f = nullptr, *r = nullptr;
+    const double* coef = nullptr;
+    int n_coef = 0, unit = 0;
+  } wide_words;
+  mtp::DevBuf wide_tab;
+  mtp::DevBuf ws_wide;         // its moments / their adjoints
   mtp::DevBuf split_tab;       // slot -> component table of the split pass (uploaded by mtp_load)
   mtp::DevBuf ws_mom;          // moments / their adjoints of the split pass
 };
@@ -271,6 +287,8 @@ struct SiteOutputs {
   // workspace of the three-kernel mixed pass (moments, then their adjoints; split_ldm(n_mom)
   // floats per atom); null: the single-kernel pass
   float* mom = nullptr;
+  // workspace of the FP64 / dual-number pass (wide_workspace bytes); null: the generic kernel
+  void* wide = nullptr;
   // tangent mode (training)
   const double* U = nullptr;    // per atom 3
   const double* Scfg = nullptr; // per config 9

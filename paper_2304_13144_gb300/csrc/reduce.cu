@@ -222,12 +222,32 @@ __global__ void k_train_cfg(int n_cfg, const double* E, const double* Eref, cons
   }
 }
 
-__global__ void k_sum_rows(const double* part, int nrows, int64_t m, double* out) {
-  int64_t c = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-  if (c >= m) return;
+// column sums of part[nrows x m] in a fixed order: a block takes 32 columns, its 32 warps every
+// 32nd row each (several loads in flight), then the warps' sums are added in order.  One thread per
+// column walked the rows one load after the other (2,432 rows of 383: 0.27 ms).
+__global__ void __launch_bounds__(1024) k_sum_rows(const double* __restrict__ part, int nrows, int64_t m, double* out) {
+  __shared__ double red[32][33];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t c = blockIdx.x * 32LL + lane;
   double acc = 0.0;
-  for (int r = 0; r < nrows; ++r) acc += part[static_cast<int64_t>(r) * m + c];
-  out[c] = acc;
+  if (c < m) {
+    const double* p = part + c;
+    int r = w;
+    for (; r + 7 * 32 < nrows; r += 8 * 32) {
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = p[static_cast<int64_t>(r + 32 * u) * m];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc += v[u];
+    }
+    for (; r < nrows; r += 32) acc += p[static_cast<int64_t>(r) * m];
+  }
+  red[w][lane] = acc;
+  __syncthreads();
+  if (w == 0 && c < m) {
+    for (int k = 1; k < 32; ++k) acc += red[k][lane];
+    out[c] = acc;
+  }
 }
 
 }  // namespace
@@ -356,7 +376,7 @@ void run_train_prep(const mtp_nbr* nb, int n_cfg, const double* E, const double*
 
 void run_sum_rows(const double* part, int nrows, int64_t m, double* out, cudaStream_t s) {
   ProfRegion pr("train_grad_sum", s);
-  k_sum_rows<<<nblk(m, 128), 128, 0, s>>>(part, nrows, m, out);
+  k_sum_rows<<<nblk(m, 32), 1024, 0, s>>>(part, nrows, m, out);
   ProfRegion::launched();
   MTP_CUDA(cudaGetLastError());
 }

@@ -1,4 +1,6 @@
-// Per-neighborhood kernel of the MTP hot path (one warp per atomic neighborhood).
+// Generic per-neighborhood kernel of the MTP hot path (one warp per atomic neighborhood): for the
+// allocation-free entry point in FP64 and for shapes without a specialised pass (n_q != 8, levels
+// above 24, mixed precision with more species than the three-kernel pass takes).
 //
 // For atom i with neighbors j (Section II.A):
 //   radial basis   Q_b(r) = T_b(x) (R_cut - r)^2, x = (2r - R_min - R_cut)/(R_cut - R_min)   (eq. 4)
@@ -15,68 +17,13 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "dual.h"
 #include "mtp_internal.h"
 #include "profiler.h"
+#include "site_wide.h"
 
 namespace mtp {
 namespace {
-
-template <class R>
-struct Dual {
-  R v, d;
-};
-template <class R> __device__ __forceinline__ Dual<R> operator+(Dual<R> a, Dual<R> b) { return {a.v + b.v, a.d + b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator-(Dual<R> a, Dual<R> b) { return {a.v - b.v, a.d - b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator*(Dual<R> a, Dual<R> b) {
-  return {a.v * b.v, a.d * b.v + a.v * b.d};
-}
-template <class R> __device__ __forceinline__ Dual<R> operator*(R s, Dual<R> b) { return {s * b.v, s * b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator*(Dual<R> b, R s) { return {s * b.v, s * b.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator+(Dual<R> a, R s) { return {a.v + s, a.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator-(R s, Dual<R> a) { return {s - a.v, -a.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator-(Dual<R> a, R s) { return {a.v - s, a.d}; }
-template <class R> __device__ __forceinline__ Dual<R> operator/(Dual<R> a, Dual<R> b) {
-  R inv = R(1) / b.v;
-  return {a.v * inv, (a.d - a.v * inv * b.d) * inv};
-}
-template <class R> __device__ __forceinline__ Dual<R>& operator+=(Dual<R>& a, Dual<R> b) { a.v += b.v; a.d += b.d; return a; }
-
-template <class S> struct Traits;
-template <> struct Traits<float> { using R = float; };
-template <> struct Traits<double> { using R = double; };
-template <> struct Traits<Dual<float>> { using R = float; };
-template <> struct Traits<Dual<double>> { using R = double; };
-
-template <class S> __device__ __forceinline__ S mk(typename Traits<S>::R v) {
-  if constexpr (std::is_same<S, typename Traits<S>::R>::value) return v;
-  else return S{v, typename Traits<S>::R(0)};
-}
-template <class S> __device__ __forceinline__ S mk2(typename Traits<S>::R v, typename Traits<S>::R d) {
-  if constexpr (std::is_same<S, typename Traits<S>::R>::value) return v;
-  else return S{v, d};
-}
-template <class S> __device__ __forceinline__ typename Traits<S>::R vpart(S x) {
-  if constexpr (std::is_same<S, typename Traits<S>::R>::value) return x;
-  else return x.v;
-}
-template <class S> __device__ __forceinline__ typename Traits<S>::R dpart(S x) {
-  if constexpr (std::is_same<S, typename Traits<S>::R>::value) return typename Traits<S>::R(0);
-  else return x.d;
-}
-__device__ __forceinline__ float ssqrt(float x) { return sqrtf(x); }
-__device__ __forceinline__ double ssqrt(double x) { return sqrt(x); }
-template <class R> __device__ __forceinline__ Dual<R> ssqrt(Dual<R> x) {
-  R s = ssqrt(x.v);
-  return {s, x.d / (R(2) * s)};
-}
-template <class S> __device__ __forceinline__ S shfl_xor(S x, int m) {
-  if constexpr (std::is_same<S, typename Traits<S>::R>::value) return __shfl_xor_sync(0xffffffffu, x, m);
-  else return S{__shfl_xor_sync(0xffffffffu, x.v, m), __shfl_xor_sync(0xffffffffu, x.d, m)};
-}
-template <class S> __device__ __forceinline__ S warp_sum(S x) {
-  for (int m = 16; m; m >>= 1) x = x + shfl_xor(x, m);
-  return x;
-}
 
 constexpr int kWarps = 4;
 
@@ -500,6 +447,7 @@ void run_sites(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, bool fp64, c
   m->last_split = false;
   if (!fp64 && !tangent && !m->force_generic && run_sites_split(m, b, nb, o, s)) return;
   if (!fp64 && !tangent && !m->force_generic && run_sites_fast(m, b, nb, o, s)) return;
+  if (!tangent && !m->force_generic && run_sites_wide(m, b, nb, fp64, o, false, 0, nullptr, s)) return;
   SiteParams P{};
   P.warps_hint = m->tune_warps_generic;
   m->last_fast = false;
