@@ -1347,7 +1347,7 @@ mtp_status mtp_energy_vjp(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     if (g_pos && !forces) throw Fail{MTP_ERR_ARG, "g_pos needs the forces of the forward pass"};
     cudaStream_t s = as_stream(stream);
     const int64_t m = md->sched.n_params, N = nb->n_atoms, K = nb->n_cfg;
-    DevBuf work;
+    ScopedBuf work(s);
     double* R = nullptr;
     if (g_theta) {
       work.ensure(std::max<int64_t>(K, 1) * m * sizeof(double), s);
@@ -1361,7 +1361,7 @@ mtp_status mtp_energy_vjp(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
       run_config_row_sums(nb, md->ws_rows.as<double>(), m, R, md->ws_red, s);
     }
     run_energy_vjp(nb, R, gE, m, forces, g_pos, g_theta, s);
-    MTP_CUDA(cudaStreamSynchronize(s));   // `work` is released on return
+    MTP_CUDA(cudaStreamSynchronize(s));
   });
 }
 
@@ -1375,7 +1375,7 @@ mtp_status mtp_config_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb
     if (!md->have_ainv) throw Fail{MTP_ERR_ARG, "no active set (call mtp_set_active_set)"};
     cudaStream_t s = as_stream(stream);
     const int64_t m = md->sched.n_params, K = nb->n_cfg;
-    DevBuf work;
+    ScopedBuf work(s);
     if (mode == MTP_GRADE_NEIGHBORHOOD) {
       work.ensure(std::max<int64_t>(nb->n_atoms, 1) * sizeof(double), s);
       efs_and_grade(md, b, nb, prec, nullptr, nullptr, nullptr, nullptr, 0.0, work.as<double>(), nullptr, nullptr,

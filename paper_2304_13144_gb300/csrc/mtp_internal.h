@@ -165,6 +165,28 @@ inline __host__ __device__ float tf32_rn(float x) {
 #endif
 }
 
+#ifdef __CUDACC__
+// |v| as an integer with the order of the absolute values (FP64 comparisons take the slow pipe);
+// NaN sorts below everything
+__device__ __forceinline__ long long abs_key(double v) {
+  const long long k = __double_as_longlong(v) & 0x7fffffffffffffffLL;
+  return k > 0x7ff0000000000000LL ? -1 : k;
+}
+// the warp's largest key, the lowest index on ties (keys >= -1, 0 <= idx < 2^63); every lane gets it
+__device__ __forceinline__ void warp_best(long long& key, long long& idx) {
+  const unsigned full = 0xffffffffu;
+  const int hi = __reduce_max_sync(full, static_cast<int>(key >> 32));
+  bool in = static_cast<int>(key >> 32) == hi;
+  const unsigned lo = __reduce_max_sync(full, in ? static_cast<unsigned>(key) : 0u);
+  in = in && static_cast<unsigned>(key) == lo;
+  const unsigned ih = __reduce_min_sync(full, in ? static_cast<unsigned>(idx >> 32) : 0xffffffffu);
+  in = in && static_cast<unsigned>(idx >> 32) == ih;
+  const unsigned il = __reduce_min_sync(full, in ? static_cast<unsigned>(idx) : 0xffffffffu);
+  key = (static_cast<long long>(hi) << 32) | lo;
+  idx = (static_cast<long long>(ih) << 32) | il;
+}
+#endif
+
 inline __host__ __device__ int pack_img(int a, int b, int c) {
   return (a & 1023) | ((b & 1023) << 10) | ((c & 1023) << 20);
 }

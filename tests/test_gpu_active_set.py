@@ -102,3 +102,36 @@ def test_maxvol_edge_cases(api):
         api.mtp_maxvol(model, torch.zeros((4, m)), eps=-1.0)
     src, ns = api.mtp_maxvol(model, torch.tensor(A0 * 3.0), max_swaps=2)
     assert ns == 2
+
+
+@pytest.mark.parametrize("types,n_q", [(1, 1), (1, 13), (1, 14), (1, 15), (2, 32), (4, 32), (8, 16), (8, 31), (8, 32)])
+def test_active_inverse_at_panel_edges(api, types, n_q):
+    """A^-1 around the edges of the panels and of the rows a thread holds (m = 3, 15, 16, 17, 131, 517,
+    1033, 1993 and, column by column, 2057): random matrices whose every pivot is off the diagonal."""
+    desc = api.make_desc(types, 2, n_q)
+    m = api.mtp_describe(desc)["n_params"]
+    model = api.mtp_load(desc, np.zeros(m))
+    g = synth.rng(m)
+    A = g.normal(size=(m, m)) + np.roll(np.diag(g.uniform(2.0, 3.0, m) * np.sqrt(m)), 1 + m // 3, axis=1)
+    api.mtp_set_active_set(model, torch.tensor(A, device="cuda"))
+    ref = np.linalg.inv(A)
+    err = np.abs(api.mtp_get_active_inverse(model).cpu().numpy() - ref).max() / np.abs(ref).max()
+    # both inverses: a few m eps cond(A); the condition number of these is a few tens at most
+    assert err <= 4 * m * np.finfo(float).eps * np.linalg.cond(A, 1)
+
+
+@pytest.mark.parametrize("n,max_swaps", [(5, 100), (40, 3), (700, 1_000_000)])
+def test_maxvol_fewer_and_more_candidates_than_parameters(api, n, max_swaps):
+    """Candidates fewer than parameters, a limit on the swaps, several blocks' worth of entries."""
+    desc = api.make_desc(2, 2, 24)
+    m = api.mtp_describe(desc)["n_params"]
+    model = api.mtp_load(desc, np.zeros(m))
+    g = synth.rng(23)
+    A0 = synth.diag_dominant(24, m)
+    B = g.normal(size=(n, m)) * np.abs(A0).max()
+    api.mtp_set_active_set(model, torch.tensor(A0, device="cuda"))
+    src, ns = api.mtp_maxvol(model, torch.tensor(B), eps=1e-3, max_swaps=max_swaps)
+    A_ref, src_ref, ns_ref = AS.maxvol(A0, B, 1e-3, max_swaps)
+    assert ns == ns_ref and 0 < ns <= max_swaps
+    np.testing.assert_array_equal(src.cpu().numpy(), src_ref)
+    np.testing.assert_array_equal(api.mtp_get_active_set(model).cpu().numpy(), A_ref)
