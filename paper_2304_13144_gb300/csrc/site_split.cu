@@ -27,6 +27,7 @@
 #include <string>
 #include <vector>
 
+#include "f32x2.h"
 #include "mtp_internal.h"
 #include "profiler.h"
 #include "site_group.h"
@@ -40,8 +41,8 @@ constexpr int kNQs = 8;      // radial polynomials of the specialised kernels
 constexpr int LPN = 8;       // lanes per neighborhood in the per-pair kernels
 constexpr int GPW = 32 / LPN;
 constexpr int BATCH = 64;    // pairs staged per neighborhood at a time (moments)
-constexpr int BATCH_A = 32;  // pairs staged per neighborhood at a time (pair adjoint)
-constexpr int GS = 17;       // floats staged per pair for the radial block: g_mu, Q_b, species (odd)
+constexpr int BATCH_A = 2 * LPN;   // pairs per neighborhood at a time (pair adjoint: two per lane)
+constexpr int GS = 20;       // floats staged per pair for the radial block: g_mu (8), Q_b (8), species; 16-byte aligned
 
 // float4 arrays staged per pair by the moment kernel: (x, y, z, f_0), then f_1.. four at a time
 __host__ __device__ constexpr int stage_f4(int nr) { return 1 + (nr - 1 + 3) / 4; }
@@ -50,13 +51,14 @@ __host__ __device__ constexpr int stage_f4(int nr) { return 1 + (nr - 1 + 3) / 4
 __host__ __device__ constexpr int pre_of(int nr) { return nr <= 5 ? 10 : 19; }
 __host__ __device__ constexpr int tmax_of(int nr) { return nr <= 5 ? 3 : 4; }
 
-// shared-memory floats per neighborhood group of the pair-adjoint kernel: dV/dM (ldm rounded up
-// to 32, plus 8) then the radial-block staging; the stride is 8 mod 32 banks, so the four groups'
-// broadcast reads of one component hit four different banks, and with the odd per-pair stride
-// the 32 lanes' staging stores hit 32 different banks
+// shared-memory floats per neighborhood group of the pair-adjoint kernel: dV/dM (ldm rounded up to
+// 32) then the radial-block staging, plus 8: the stride is 8 mod 32 banks, so the four groups'
+// broadcast reads of one component hit different banks
 __host__ __device__ inline int adj_region(int ldm, bool rows) {
   return ((ldm + 31) & ~31) + 8 + (rows ? BATCH_A * GS : 0);
 }
+// its blocks per SM (128 registers for two; level 24 is faster with more registers: 1.99 against 2.31 ms)
+constexpr int adj_blocks(int nr) { return nr <= 5 ? 2 : 1; }
 
 struct SplitArgs {
   DevSchedule d;
@@ -67,7 +69,8 @@ struct SplitArgs {
   float* mom;   // [n_work x ldm]: moments (k_moments), overwritten by dV/dM (k_contract), both in
                 // slot order (monomial-major, the order of the moment pass's chunks)
   int ldm;
-  const int* slot_comp;   // slot -> value index of the moment component
+  const int* slot_comp;     // slot -> value index of the moment component
+  const int* slot_horner;   // slot -> place in the pair adjoint's order
   int T, CBN, NC, NV;
   // contraction kernel: shared-memory layout (word offsets of the schedule arrays)
   size_t c_bytes, sched_bytes, warp_bytes, total;
@@ -813,11 +816,99 @@ __global__ void __launch_bounds__(SCH == 1 ? 256 : (SCH == 2 ? 384 : 512), 1) k_
 // ------------------------------------------------------------------------------------
 // pair adjoint: per-pair gradients, the neighborhood's virial, the radial block of b_i
 // ------------------------------------------------------------------------------------
+// dV/dM of a neighborhood in the order the nested Horner schemes read it: mu, then descending
+// powers a of x, b of y, c of z
+template <int NR, int NU0>
+struct HornerOrder {
+  using Sh = Shape<NR, NU0>;
+  // position of (mu, a, b) with the highest power of z
+  static constexpr int at(int mu, int a, int b) {
+    int p = 0;
+    for (int m = 0; m < mu; ++m) p += nmono_upto(Sh::numax(m));
+    const int n = Sh::numax(mu);
+    for (int x = n; x > a; --x) p += (n - x + 1) * (n - x + 2) / 2;
+    for (int y = n - a; y > b; --y) p += n - a - y + 1;
+    return p;
+  }
+  static std::vector<int> of_slots() {
+    constexpr auto S = make_slots<NR, NU0>();
+    constexpr auto M = make_mono<NU0>();
+    std::vector<int> t(Sh::NCOMP);
+    for (int s = 0; s < Sh::NCOMP; ++s) {
+      const int k = S.k[s], mu = S.mu[s], top = Sh::numax(mu) - M.a[k] - M.b[k];
+      t[s] = at(mu, M.a[k], M.b[k]) + (top - M.c[k]);
+    }
+    return t;
+  }
+};
+
+// Values P_mu(r) = sum_k (dV/dM_mu,k) x^a y^b z^c of two pairs at once (packed), and their
+// gradients through `use(mu, P, dP/dx, dP/dy, dP/dz)`.  Per component two packed FMAs and, four at a
+// time, a broadcast load; per (a, b) three more.  G: Horner order, 16-byte aligned.
+template <int NR, int NU0, class Use>
+__device__ __forceinline__ void horner_pass(const float* G, u64 x, u64 y, u64 z, Use&& use) {
+  using Sh = Shape<NR, NU0>;
+  using HO = HornerOrder<NR, NU0>;
+  float4 cur = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto get = [&](auto I) -> u64 {   // component I (called in ascending order)
+    constexpr int i = decltype(I)::value;
+    if constexpr (i % 4 == 0) cur = *reinterpret_cast<const float4*>(G + i);
+    const float v = i % 4 == 0 ? cur.x : (i % 4 == 1 ? cur.y : (i % 4 == 2 ? cur.z : cur.w));
+    return pack2(v, v);
+  };
+  static_for<0, NR>([&](auto Mu) {
+    constexpr int mu = decltype(Mu)::value, n = Sh::numax(mu);
+    u64 pv = 0, px = 0, py = 0, pz = 0;
+    static_for<0, n + 1>([&](auto A) {
+      constexpr int a = n - decltype(A)::value, na = n - a;
+      u64 av = 0, ay = 0, az = 0;
+      static_for<0, na + 1>([&](auto B) {
+        constexpr int b = na - decltype(B)::value, nc = na - b, i0 = HO::at(mu, a, b);
+        u64 t = get(std::integral_constant<int, i0>{}), u = 0;
+        static_for<1, nc + 1>([&](auto C) {
+          constexpr int c = decltype(C)::value;
+          u = c == 1 ? t : fma2(u, z, t);
+          t = fma2(t, z, get(std::integral_constant<int, i0 + c>{}));
+        });
+        if constexpr (b == na) {
+          av = t;
+          az = u;
+        } else {
+          ay = b == na - 1 ? av : fma2(ay, y, av);
+          az = fma2(az, y, u);
+          av = fma2(av, y, t);
+        }
+      });
+      if constexpr (a == n) {
+        pv = av;
+        py = ay;
+        pz = az;
+      } else {
+        px = a == n - 1 ? pv : fma2(px, x, pv);
+        py = fma2(py, x, ay);
+        pz = fma2(pz, x, az);
+        pv = fma2(pv, x, av);
+      }
+      // keeps the loads of later components from being hoisted wholesale
+      if constexpr (na >= 3) asm volatile("" ::: "memory");
+    });
+    use(Mu, pv, px, py, pz);
+  });
+}
+
+// What bounds it: issue and the latency of dependent FMAs (9,300 warp instructions per four
+// neighborhoods at level 20, half an instruction per clock and scheduler; a third of them moves
+// that double a loaded component for the packed FMAs: loading it doubled from shared memory was
+// slower, 5.70 ms).  A lane takes two pairs, packed (fma.rn.f32x2), and walks nested Horner schemes:
+// at level 20 785 packed FMAs per two pairs instead of about 1,400 scalar operations per pair over a
+// register array of 165 monomials.  Rows are written by whole warps, their zero blocks without a
+// division per entry.  Level 20, 1,048,576 atoms (with rows): 5.33 -> 4.09 ms; level 16, 128,000
+// atoms 0.281 -> 0.220; level 24, 131,072 atoms 3.68 -> 1.99.
 template <int NR, int NU0, bool ROWS>
-__global__ void __launch_bounds__(256) k_adjoint(SplitArgs P) {
+__global__ void __launch_bounds__(256, adj_blocks(NR)) k_adjoint(SplitArgs P) {
   using Sh = Shape<NR, NU0>;
   constexpr int NQ = kNQs;
-  static_assert(NR + NQ + 1 <= GS, "radial-block staging");
+  static_assert(NR <= 8 && 8 + NQ + 1 <= GS, "radial-block staging");
   extern __shared__ __align__(16) unsigned char smem[];
   const DevSchedule& d = P.d;
   const int T = P.T;
@@ -827,9 +918,12 @@ __global__ void __launch_bounds__(256) k_adjoint(SplitArgs P) {
   const int nwarps = blockDim.x >> 5;
   const int gstride = adj_region(P.ldm, ROWS);
   float* gM = reinterpret_cast<float*>(smem + P.c_bytes) + (static_cast<size_t>(warp) * GPW + grp) * gstride;
-  float* rstg = gM + ((P.ldm + 31) & ~31) + 8;
+  float* rstg = gM + ((P.ldm + 31) & ~31);
+  float* rblk = gM;   // radial block of the row on its way out (at most T NR NQ floats)
   __syncthreads();
   const float rmin = static_cast<float>(d.r_min), rcut = static_cast<float>(d.r_cut);
+  const float sc = 1.f / (rcut - rmin);
+  const u64 one2 = pack2(1.f, 1.f);
   for (int64_t w0 = (static_cast<int64_t>(blockIdx.x) * nwarps + warp) * GPW; w0 < P.n_work;
        w0 += static_cast<int64_t>(gridDim.x) * nwarps * GPW) {
     const int64_t wk = w0 + grp;
@@ -849,121 +943,195 @@ __global__ void __launch_bounds__(256) k_adjoint(SplitArgs P) {
     if (live) {
       const float* src = P.mom + wk * P.ldm;
       for (int k = q; k < Sh::NCOMP; k += LPN)
-        if (OK(P.slot_comp[k], P.ldm, 43) && OK(wk * P.ldm + k, P.n_work * P.ldm, 44)) gM[P.slot_comp[k]] = __ldcs(src + k);
+        if (OK(P.slot_horner[k], P.ldm, 43) && OK(wk * P.ldm + k, P.n_work * P.ldm, 44)) gM[P.slot_horner[k]] = __ldcs(src + k);
     }
     __syncwarp();
     const float* czi = ctab + static_cast<size_t>(zi) * T * NR * NQ;
-    float Wl[9];
+    u64 Wl[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) Wl[k] = 0.f;
-    // radial block accumulators: lane q owns beta = q for every (species, mu)
-    constexpr int TM = tmax_of(NR);
-    float cb[TM][NR];
+    for (int k = 0; k < 9; ++k) Wl[k] = 0;
+    // radial block accumulators: lane q owns beta = q for every (species, mu), mu in packed pairs
+    constexpr int TM = tmax_of(NR), MP = (NR + 1) / 2;
+    u64 cb[TM][MP];
 #pragma unroll
     for (int z = 0; z < TM; ++z)
 #pragma unroll
-      for (int mu = 0; mu < NR; ++mu) cb[z][mu] = 0.f;
+      for (int k = 0; k < MP; ++k) cb[z][k] = 0;
     float* Gout = static_cast<float*>(P.o.G);
     for (int base = 0; base < np_max; base += BATCH_A) {
-      const int nbt = min(BATCH_A, np - base);
-      // every lane of the warp runs the same number of iterations (adjoint_pass has warp-wide
-      // __syncwarp fences); lanes without a pair of their own work on a dummy one
-      const int nbt_w = min(BATCH_A, np_max - base);
-      for (int t0 = 0; t0 < nbt_w; t0 += LPN) {
-        const int t = t0 + q;
-        const int64_t p = p0 + base + t;
-        bool act = t < nbt;
-        if (act && (!OK(p, P.nb.n_pairs, 45) || (ROWS && !OK(t * GS + GS - 1, BATCH_A * GS, 46)))) act = false;
-        float4 r = make_float4(1.f, 0.f, 0.f, 1.f);
-        int zj = 0;
-        if (act) {
-          r = P.nb.pr32[p];
-          const int jj = P.nb.pj[p];
-          if (OK(jj, P.nb.n_atoms, 47)) zj = P.type[jj];
-          if (!OK(zj, T, 48)) zj = 0;
-        }
-        float f[NR], df[NR], g[NR];
-        radial<NR, NQ>(r.w, czi + zj * NR * NQ, rmin, rcut, f, df, (ROWS && act) ? rstg + t * GS + NR : nullptr);
+      // lane q: pairs base + q and base + LPN + q; lanes without a pair work on a dummy one
+      float4 r[2];
+      int zj[2];
+      bool act[2];
+      int64_t p[2];
 #pragma unroll
-        for (int mu = 0; mu < NR; ++mu) g[mu] = 0.f;
-        float gx = 0.f, gy = 0.f, gz = 0.f;
-        adjoint_pass<NR, NU0>(r.x, r.y, r.z, f, gM, g, gx, gy, gz);
-        if (!act) continue;
-        float rad = 0.f;
-#pragma unroll
-        for (int mu = 0; mu < NR; ++mu) rad = fmaf(g[mu], df[mu], rad);
-        const float sc = rad / r.w;
-        gx = fmaf(sc, r.x, gx);
-        gy = fmaf(sc, r.y, gy);
-        gz = fmaf(sc, r.z, gz);
-        if (Gout && OK(3 * p + 2, 3 * P.nb.n_pairs, 53)) {
-          __stcs(Gout + 3 * p + 0, gx);
-          __stcs(Gout + 3 * p + 1, gy);
-          __stcs(Gout + 3 * p + 2, gz);
-        }
-        const float g3[3] = {gx, gy, gz}, r3[3] = {r.x, r.y, r.z};
-#pragma unroll
-        for (int a2 = 0; a2 < 3; ++a2)
-#pragma unroll
-          for (int b2 = 0; b2 < 3; ++b2) Wl[3 * a2 + b2] = fmaf(-g3[a2], r3[b2], Wl[3 * a2 + b2]);
-        if (ROWS) {
-          float* e = rstg + t * GS;
-#pragma unroll
-          for (int mu = 0; mu < NR; ++mu) e[mu] = g[mu];
-          e[NR + NQ] = __int_as_float(zj);
+      for (int h = 0; h < 2; ++h) {
+        const int t = base + h * LPN + q;
+        p[h] = p0 + t;
+        act[h] = t < np && OK(p[h], P.nb.n_pairs, 45);
+        r[h] = make_float4(1.f, 0.f, 0.f, 1.f);
+        zj[h] = 0;
+        if (act[h]) {
+          r[h] = P.nb.pr32[p[h]];
+          const int jj = P.nb.pj[p[h]];
+          if (OK(jj, P.nb.n_atoms, 47)) zj[h] = P.type[jj];
+          if (!OK(zj[h], T, 48)) zj[h] = 0;
         }
       }
+      const u64 x = pack2(r[0].x, r[1].x), y = pack2(r[0].y, r[1].y), z = pack2(r[0].z, r[1].z), d2 = pack2(r[0].w, r[1].w);
+      // T_b and b U_(b-1) = T_b' of both distances, w = R_cut - r
+      const u64 t1 = mul2(add2(add2(d2, d2), pack2(-(rmin + rcut), -(rmin + rcut))), pack2(sc, sc)), tt = add2(t1, t1);
+      const u64 w = fma2(d2, pack2(-1.f, -1.f), pack2(rcut, rcut)), w2 = mul2(w, w);
+      const u64 dxw2 = mul2(pack2(2.f * sc, 2.f * sc), w2), mw = mul2(pack2(-2.f, -2.f), w);
+      u64 Tb[NQ], Ub[NQ];
+      Tb[0] = one2;
+      Tb[1] = t1;
+      Ub[0] = one2;
+      Ub[1] = tt;
+#pragma unroll
+      for (int b = 2; b < NQ; ++b) {
+        Tb[b] = fma2(tt, Tb[b - 1], Tb[b - 2] ^ 0x8000000080000000ull);
+        Ub[b] = fma2(tt, Ub[b - 1], Ub[b - 2] ^ 0x8000000080000000ull);
+      }
+#pragma unroll
+      for (int b = NQ - 1; b >= 1; --b) Ub[b] = mul2(pack2(static_cast<float>(b), static_cast<float>(b)), Ub[b - 1]);
+      if (ROWS) {
+#pragma unroll
+        for (int b = 0; b < NQ; ++b) {
+          float q0, q1;
+          unpack2(mul2(Tb[b], w2), q0, q1);
+          rstg[q * GS + 8 + b] = q0;
+          rstg[(LPN + q) * GS + 8 + b] = q1;
+        }
+      }
+      const float *c0 = czi + zj[0] * NR * NQ, *c1 = czi + zj[1] * NR * NQ;
+      u64 gx = 0, gy = 0, gz = 0, rad = 0;
+      horner_pass<NR, NU0>(gM, x, y, z, [&](auto Mu, u64 pv, u64 px, u64 py, u64 pz) {
+        constexpr int mu = decltype(Mu)::value;
+        // f_mu = w^2 sum c T_b, f_mu' = (dx/dr) w^2 sum c T_b' - 2 w sum c T_b
+        u64 F = pack2(c0[mu * NQ], c1[mu * NQ]), D = 0;
+#pragma unroll
+        for (int b = 1; b < NQ; ++b) {
+          const u64 cc = pack2(c0[mu * NQ + b], c1[mu * NQ + b]);
+          F = fma2(cc, Tb[b], F);
+          D = b == 1 ? mul2(cc, Ub[1]) : fma2(cc, Ub[b], D);
+        }
+        const u64 f = mul2(F, w2);
+        gx = fma2(f, px, gx);
+        gy = fma2(f, py, gy);
+        gz = fma2(f, pz, gz);
+        rad = fma2(pv, fma2(dxw2, D, mul2(mw, F)), rad);
+        if (ROWS) {
+          float g0, g1;
+          unpack2(pv, g0, g1);
+          rstg[q * GS + mu] = g0;
+          rstg[(LPN + q) * GS + mu] = g1;
+        }
+      });
+      float rd[2];
+      unpack2(rad, rd[0], rd[1]);
+      const u64 s2 = pack2(rd[0] / r[0].w, rd[1] / r[1].w);
+      gx = fma2(s2, x, gx);
+      gy = fma2(s2, y, gy);
+      gz = fma2(s2, z, gz);
+      float g3[2][3];
+      unpack2(gx, g3[0][0], g3[1][0]);
+      unpack2(gy, g3[0][1], g3[1][1]);
+      unpack2(gz, g3[0][2], g3[1][2]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (act[h] && Gout && OK(3 * p[h] + 2, 3 * P.nb.n_pairs, 53)) {
+          __stcs(Gout + 3 * p[h] + 0, g3[h][0]);
+          __stcs(Gout + 3 * p[h] + 1, g3[h][1]);
+          __stcs(Gout + 3 * p[h] + 2, g3[h][2]);
+        }
+        if (!act[h]) g3[h][0] = g3[h][1] = g3[h][2] = 0.f;   // a dummy pair adds nothing to the virial
+        if (ROWS) rstg[(h * LPN + q) * GS + 8 + NQ] = __int_as_float(zj[h]);
+      }
+      const u64 n3[3] = {pack2(-g3[0][0], -g3[1][0]), pack2(-g3[0][1], -g3[1][1]), pack2(-g3[0][2], -g3[1][2])};
+      const u64 r3[3] = {x, y, z};
+#pragma unroll
+      for (int a2 = 0; a2 < 3; ++a2)
+#pragma unroll
+        for (int b2 = 0; b2 < 3; ++b2) Wl[3 * a2 + b2] = fma2(n3[a2], r3[b2], Wl[3 * a2 + b2]);
       if (ROWS) {
         __syncwarp();
         // sum_j g_mu(j) Q_b(r_ij) per neighbor species: lane q takes b = q over the staged pairs
+        const int nbt = min(BATCH_A, np - base);
         for (int t = 0; t < nbt; ++t) {
-          if (!OK(t * GS + GS - 1, BATCH_A * GS, 49)) continue;
           const float* e = rstg + t * GS;
-          const float qb = e[NR + q];
-          const int zj = __float_as_int(e[NR + NQ]);
+          const float qb = e[8 + q];
+          const int zt = __float_as_int(e[8 + NQ]);
+          u64 em[MP];
+          if constexpr (MP >= 2) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(e);
+            em[0] = v.x;
+            em[1] = v.y;
+          } else {
+            em[0] = *reinterpret_cast<const u64*>(e);
+          }
+          if constexpr (MP >= 3) em[2] = *reinterpret_cast<const u64*>(e + 4);
+          // (an odd NR's last half sums what the slot past g holds: never written out)
 #pragma unroll
-          for (int mu = 0; mu < NR; ++mu) {
-            const float pr = e[mu] * qb;
+          for (int zz = 0; zz < TM; ++zz) {
+            if (zz >= T) break;
+            const float qz = zt == zz ? qb : 0.f;
+            const u64 q2 = pack2(qz, qz);
 #pragma unroll
-            for (int z = 0; z < TM; ++z) cb[z][mu] += (zj == z) ? pr : 0.f;
+            for (int k = 0; k < MP; ++k) cb[zz][k] = fma2(em[k], q2, cb[zz][k]);
           }
         }
         __syncwarp();
       }
     }
     // the neighborhood's virial (FP32 over its pairs, like its forces; sums over atoms are FP64)
+    float Ws[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) Wl[k] = group_sum(Wl[k]);
+    for (int k = 0; k < 9; ++k) {
+      float lo, hi;
+      unpack2(Wl[k], lo, hi);
+      Ws[k] = group_sum(lo + hi);
+    }
     if (live && P.o.Wat && q == 0 && OK(9 * i + 8, 9 * P.nb.n_atoms, 50)) {
 #pragma unroll
-      for (int k = 0; k < 9; ++k) P.o.Wat[9 * i + k] = static_cast<double>(Wl[k]);
+      for (int k = 0; k < 9; ++k) P.o.Wat[9 * i + k] = static_cast<double>(Ws[k]);
     }
-    if (ROWS && live && P.o.rows_hi) {
-      const int64_t rw = P.o.row_pos ? P.o.row_pos[i] : wk;
-      const int64_t ld = P.o.rows_ld;
-      const int off_c = T + d.n_lin;
-      float* hi = P.o.rows_hi + rw * ld;
-      float* lo = P.o.rows_lo ? P.o.rows_lo + rw * ld : nullptr;
-      auto put = [&](int64_t k, float val) {
-        if (!OK(rw * ld + k, P.nb.n_atoms * ld, 51) || !OK(k, ld, 52)) return;
-        if (lo) {
-          const float h = tf32_rn(val);
-          __stcs(hi + k, h);
-          __stcs(lo + k, tf32_rn(val - h));
-        } else {
-          __stcs(hi + k, val);
+    if (ROWS && P.o.rows_hi) {
+      // the sums through shared memory (over the group's dV/dM, which is done with), then whole rows:
+      // block zi holds them; the other species' blocks and the padding past m are zero
+      __syncwarp();
+#pragma unroll
+      for (int zz = 0; zz < TM; ++zz) {
+        if (zz >= T) break;
+#pragma unroll
+        for (int mu = 0; mu < NR; ++mu) {
+          float lo2, hi2;
+          unpack2(cb[zz][mu / 2], lo2, hi2);
+          rblk[(zz * NR + mu) * NQ + q] = mu % 2 ? hi2 : lo2;
         }
-      };
-      // block zi holds the sums; the other species' blocks and the padding past m are zero
-      for (int k = off_c + q; k < ld; k += LPN) {
-        const int e = k - off_c;
-        if (e / P.CBN != zi || k >= d.n_params) put(k, 0.f);
       }
+      __syncwarp();
+      const int off_c = T + d.n_lin, ld = static_cast<int>(P.o.rows_ld);
+      const long long at = live ? (P.o.row_pos ? P.o.row_pos[i] : wk) * static_cast<long long>(ld) : -1;
 #pragma unroll
-      for (int z = 0; z < TM; ++z) {
-        if (z < T) {
-#pragma unroll
-          for (int mu = 0; mu < NR; ++mu) put(off_c + static_cast<int64_t>(zi) * P.CBN + (z * NR + mu) * NQ + q, cb[z][mu]);
+      for (int g = 0; g < GPW; ++g) {
+        const long long ro = __shfl_sync(0xffffffffu, at, g * LPN);
+        const int z0 = __shfl_sync(0xffffffffu, zi, g * LPN) * P.CBN;
+        if (ro < 0) continue;
+        const float* blk = rblk + (g - grp) * gstride;
+        float* hi = P.o.rows_hi + ro + off_c;
+        float* lo = P.o.rows_lo ? P.o.rows_lo + ro + off_c : nullptr;
+        for (int e = lane; e < ld - off_c; e += 32) {
+          if (!OK(ro + off_c + e, P.nb.n_atoms * P.o.rows_ld, 51)) continue;
+          const unsigned rel = static_cast<unsigned>(e - z0);
+          const float v = rel < static_cast<unsigned>(P.CBN) ? blk[rel] : 0.f;
+          if (lo) {
+            const float h = tf32_rn(v);
+            __stcs(hi + e, h);
+            __stcs(lo + e, tf32_rn(v - h));
+          } else {
+            __stcs(hi + e, v);
+          }
         }
       }
     }
@@ -1078,12 +1246,15 @@ template <int NR, int NU0>
 std::vector<int> slot_table() {
   using Sh = Shape<NR, NU0>;
   constexpr auto S = make_slots<NR, NU0>();
-  return std::vector<int>(S.comp, S.comp + Sh::NCOMP);
+  std::vector<int> t(S.comp, S.comp + Sh::NCOMP);
+  const std::vector<int> h = HornerOrder<NR, NU0>::of_slots();   // then slot -> Horner order
+  t.insert(t.end(), h.begin(), h.end());
+  return t;
 }
 
 }  // namespace
 
-// Uploads the slot -> component table of the model's shape (at load time, so that the split
+// Uploads the slot -> component and slot -> Horner-order tables of the model's shape (at load time, so that the split
 // pass allocates nothing when it runs); leaves it empty for shapes without a split kernel.
 void split_prepare(mtp_model* m) {
   const DevSchedule& d = m->ds;
@@ -1095,7 +1266,7 @@ void split_prepare(mtp_model* m) {
     else if (d.n_rad == 5 && d.nu_max == 8) t = slot_table<5, 8>();
     else if (d.n_rad == 6 && d.nu_max == 10) t = slot_table<6, 10>();
   }
-  if (t.empty() || static_cast<int>(t.size()) != d.n_mom) return;
+  if (t.empty() || static_cast<int>(t.size()) != 2 * d.n_mom) return;
   m->split_tab.ensure(t.size() * sizeof(int), 0);
   MTP_CUDA(cudaMemcpy(m->split_tab.p, t.data(), t.size() * sizeof(int), cudaMemcpyHostToDevice));
 }
@@ -1125,6 +1296,7 @@ bool run_sites_split(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, const 
   P.mom = mom_ws;
   P.ldm = split_ldm(d.n_mom);
   P.slot_comp = m->split_tab.as<int>();
+  P.slot_horner = P.slot_comp + d.n_mom;
   P.T = d.n_types;
   P.CBN = d.n_types * d.n_rad * d.n_q;
   P.NC = d.n_types * P.CBN;
