@@ -835,6 +835,7 @@ mtp_status mtp_load(const mtp_desc* desc, const double* theta, int64_t m, mtp_mo
       split_prepare(md);
       wide_prepare(md);
       noalloc_prepare(md->device);
+      MTP_CUDA(cudaMallocHost(&md->pin, kPinBytes));
       md->async_err.ensure(sizeof(unsigned), 0);
       MTP_CUDA(cudaMemset(md->async_err.p, 0, sizeof(unsigned)));
       MTP_CUDA(cudaDeviceSynchronize());
@@ -856,6 +857,7 @@ void mtp_free_model(mtp_model* md) {
                     &md->ws_atom, &md->ws_rows, &md->ws_grade, &md->ws_sort, &md->ws_misc, &md->ws_red,
                     &md->err_flag, &md->async_err, &md->split_tab, &md->ws_mom, &md->wide_tab, &md->ws_wide})
     b->release();
+  if (md->pin) cudaFreeHost(md->pin);
   cudaSetDevice(cur);
   delete md;
 }

@@ -130,16 +130,6 @@ struct DevSchedule {
 // ------------------------------------------------------------------------------------
 // neighbor list on the device
 // ------------------------------------------------------------------------------------
-struct CfgPlan {
-  double H[9];        // rows = lattice vectors
-  double Hinv[9];     // s = x Hinv
-  int nb[3], kb[3], pbc[3];
-  int K;              // image table half-width: nrel in [-K, K]^3
-  int64_t bin_base;
-  int64_t shift_base; // offset into the shift table ((2K+1)^3 entries)
-  double rc2;
-};
-
 struct DevNbr {
   int64_t n_atoms, n_pairs;
   const int64_t* off;   // [n_atoms+1]
@@ -198,7 +188,7 @@ inline __host__ __device__ int unpack_img(int v, int k) {
 // ------------------------------------------------------------------------------------
 // handles
 // ------------------------------------------------------------------------------------
-struct ModelHost;
+constexpr size_t kPinBytes = 16384;
 }  // namespace mtp
 
 struct mtp_model {
@@ -225,6 +215,7 @@ struct mtp_model {
   mtp::DevBuf ws_misc;
   mtp::DevBuf ws_red;          // reductions
   mtp::DevBuf err_flag;        // unsigned
+  void* pin = nullptr;         // kPinBytes of pinned host memory for read-backs (mtp_load)
   // errors of asynchronous kernels (bit 1: a bounded wait of the tensor-core grade expired),
   // allocated and zeroed by mtp_load, OR-ed by the kernels, read and cleared by mtp_sync
   mtp::DevBuf async_err;
@@ -278,8 +269,14 @@ struct mtp_nbr {
   mtp::DevBuf segs;   // per scanned bin and atom: accepted slots and pairs before the bin (neighbors.cu)
   mtp::DevBuf masks;  // per-atom accepted-candidate bits of the count pass (neighbors.cu)
   mtp::DevBuf bins, plan, shifts, wrap, scratch, counts;
-  std::vector<mtp::CfgPlan> plans;
   std::vector<int64_t> atom_offset;   // host copy
+  // the device plan (bins, shifts, segments) belongs to these values
+  bool plan_valid = false;
+  double plan_rc = 0.0;
+  std::vector<double> plan_cell;
+  std::vector<uint8_t> plan_pbc;
+  size_t plan_shifts = 0;
+  int plan_max_scan = 0;
   int64_t n_bins_total = 0;
   // segments for deterministic per-config reductions: [cfg, atom_begin, atom_end]
   std::vector<int64_t> seg_host;

@@ -20,6 +20,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "mtp_internal.h"
@@ -205,18 +206,19 @@ __device__ __forceinline__ int decide(const NbrArgs& A, const DevCfg& C, int64_t
   return 1;
 }
 
+// atoms from which the count pass takes a thread per atom instead of a warp (binning and count, ms,
+// warp against thread: 4,000 atoms 0.055, 0.171; 32,000 0.166, 0.224; 62,500 0.249, 0.259; 65,536
+// 0.267, 0.273; 131,072 0.424, 0.328; 500,000 1.40, 0.90)
+constexpr int64_t kCountThreads = 65536;
 constexpr int kWarpScan = 32;    // the warp fill and the reverse record: at most 32 scanned bins
 constexpr int kMaskWords = 16;   // accepted-candidate bits per atom recorded by the count pass
 constexpr int kMaskBits = 32 * kMaskWords;
 
+// Count pass with a thread per atom (bin order), for lists large enough to fill the GPU that way.
 // (at most 64 registers, 8 CTAs of 128 threads per SM: with the per-bin reverse record the
 // count pass measured 1.77 ms at 1M atoms against 1.91 ms at 48 registers / 10 CTAs and at
-// 80 registers / 6 CTAs; a warp-per-atom count pass with ballots measured 2.86 ms)
-#ifndef MTP_NB_MINB
-#define MTP_NB_MINB 8
-#endif
-template <bool FILL>
-__global__ void __launch_bounds__(128, MTP_NB_MINB) k_pairs(NbrArgs A) {
+// 80 registers / 6 CTAs; the warp-per-atom pass below measured 2.86 ms)
+__global__ void __launch_bounds__(128, 8) k_count(NbrArgs A) {
   // threads take the atoms in bin order, so that a warp's atoms scan the same or adjacent bins
   const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (t >= A.n_atoms) return;
@@ -226,11 +228,9 @@ __global__ void __launch_bounds__(128, MTP_NB_MINB) k_pairs(NbrArgs A) {
   const int bc = A.bcoord[i];
   const int b0 = bc & 1023, b1 = (bc >> 10) & 1023, b2 = (bc >> 20) & 1023;
   const float4 xi_h = A.ph[i], xi_l = A.pl[i];
-  long long out = FILL ? A.off[i] : 0;
-  const long long out_end = FILL ? A.off[i + 1] : 0;
-  long long count = 0;
+  int count = 0;
   int cand = 0;          // candidate index in scan order (the self candidate included)
-  uint32_t mword = 0;    // count pass: accepted bits of the current mask word
+  uint32_t mword = 0;    // accepted bits of the current mask word
   // bins are scanned in increasing q = ((d0 + kb0) w1 + (d1 + kb1)) w2 + (d2 + kb2)
   const int w1 = 2 * C.kb[1] + 1, w2 = 2 * C.kb[2] + 1;
   for (int d0 = -C.kb[0]; d0 <= C.kb[0]; ++d0) {
@@ -257,64 +257,211 @@ __global__ void __launch_bounds__(128, MTP_NB_MINB) k_pairs(NbrArgs A) {
         const int q = ((d0 + C.kb[0]) * w1 + (d1 + C.kb[1])) * w2 + (d2 + C.kb[2]);
         const long long tb = C.bin_base + (static_cast<long long>(t0) * C.nb[1] + t1) * C.nb[2] + t2;
         const long long s0 = A.bin_start[tb], s1 = A.bin_start[tb + 1];
-        // candidate s of this bin: 1 if (i -> j, n) is a pair (written out in the fill pass)
-        auto test = [&](long long s) -> int {
+        const unsigned before = static_cast<unsigned>(count);
+        uint32_t slots = 0;   // accepted bits of this bin's first 32 slots
+        for (long long s = s0; s < s1; ++s, ++cand) {
           const float4 xj_h = A.bph[s];
           const int j = __float_as_int(xj_h.w);
-          if (j == static_cast<int>(i) && n0 == 0 && n1 == 0 && n2 == 0) return 0;
-          float4 r;
-          int img;
-          if (!decide(A, C, i, j, xi_h, xi_l, xj_h, A.bpl[s], n0, n1, n2, r, img)) return 0;
-          if (FILL && out < out_end) {
-            A.pj[out] = j;
-            A.pimg[out] = img;
-            A.pr32[out] = r;
-            ++out;
+          int acc = 0;
+          if (!(j == static_cast<int>(i) && n0 == 0 && n1 == 0 && n2 == 0)) {
+            float4 r;
+            int img;
+            acc = decide(A, C, i, j, xi_h, xi_l, xj_h, A.bpl[s], n0, n1, n2, r, img);
           }
-          ++count;
-          return 1;
-        };
-        long long s = s0;
-        if (FILL && A.mask) {
-          // replay the count pass's decisions: only its accepted candidates are formed again
-          while (s < s1 && cand < kMaskBits) {
-            const int wb = cand & 31;
-            const int span = static_cast<int>(min(static_cast<long long>(32 - wb), s1 - s));
-            uint32_t word = A.mask[static_cast<long long>(cand >> 5) * A.n_atoms + t] >> wb;
-            if (span < 32) word &= (1u << span) - 1u;
-            while (word) {
-              const int b = __ffs(word) - 1;
-              word &= word - 1u;
-              test(s + b);
-            }
-            s += span;
-            cand += span;
-          }
-        }
-        const unsigned before = static_cast<unsigned>(count);
-        uint32_t slots = 0;   // count pass: accepted bits of this bin's first 32 slots
-        for (; s < s1; ++s, ++cand) {
-          const int acc = test(s);
-          if (!FILL && A.mask && cand < kMaskBits) {
+          count += acc;
+          if (cand < kMaskBits) {
             mword |= static_cast<uint32_t>(acc) << (cand & 31);
             if ((cand & 31) == 31) {
               A.mask[static_cast<long long>(cand >> 5) * A.n_atoms + t] = mword;
               mword = 0;
             }
           }
-          if (!FILL && s - s0 < 32) slots |= static_cast<uint32_t>(acc) << (s - s0);
+          if (s - s0 < 32) slots |= static_cast<uint32_t>(acc) << (s - s0);
         }
-        if (!FILL && A.rv) A.rv[static_cast<long long>(q) * A.n_atoms + t] = make_uint2(slots, before);
+        A.rv[static_cast<long long>(q) * A.n_atoms + t] = make_uint2(slots, before);
       }
     }
   }
-  if (!FILL && A.mask && cand < kMaskBits && (cand & 31) != 0)
-    A.mask[static_cast<long long>(cand >> 5) * A.n_atoms + t] = mword;
-  if (!FILL) A.cnt[i] = count;
-  else if (count != out_end - A.off[i]) atomicOr(A.err, ERRF_CAPACITY);
+  if (cand < kMaskBits && (cand & 31) != 0) A.mask[static_cast<long long>(cand >> 5) * A.n_atoms + t] = mword;
+  A.cnt[i] = count;
 }
 
-// Fill pass with one warp per atom (bin order), for configurations that scan at most 32 bins:
+// A warp per atom (bin order), any number of scanned bins: 32 bins at a time, a lane per bin (its
+// first binned atom, size and image), their candidates 32 at a time.  The count pass of small lists
+// (a thread per atom walks its few hundred candidates one after the other: 137 us for 108 atoms) and
+// of cells that scan more than 32 bins, whose fill pass it is too (candidates decided again, written
+// in scan order).  Same candidates, decisions and order as k_count.
+template <bool FILL>
+__global__ void __launch_bounds__(128) k_scan_warp(NbrArgs A) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int64_t t = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
+  if (t >= A.n_atoms) return;   // whole warps leave together
+  const int64_t i = A.bin_atoms[t];
+  const DevCfg& C = A.cfg[A.atom_cfg[i]];
+  const int bc = A.bcoord[i];
+  const int b[3] = {bc & 1023, (bc >> 10) & 1023, (bc >> 20) & 1023};
+  const float4 xi_h = A.ph[i], xi_l = A.pl[i];
+  const int w1 = 2 * C.kb[1] + 1, w2 = 2 * C.kb[2] + 1;
+  const int n_scan = (2 * C.kb[0] + 1) * w1 * w2;
+  const long long out0 = FILL ? A.off[i] : 0, out1 = FILL ? A.off[i + 1] : 0;
+  int total = 0;   // pairs so far
+  for (int q0 = 0; q0 < n_scan; q0 += 32) {
+    const int q = q0 + lane;
+    int n[3] = {0, 0, 0};
+    long long s0 = 0;
+    int sz = 0;
+    if (q < n_scan) {
+      const int d[3] = {q / (w1 * w2) - C.kb[0], (q / w2) % w1 - C.kb[1], q % w2 - C.kb[2]};
+      int tt[3];
+      bool ok = true;
+      for (int a = 0; a < 3; ++a) {
+        tt[a] = b[a] + d[a];
+        if (C.pbc[a]) {
+          if (tt[a] < 0 || tt[a] >= C.nb[a]) {
+            n[a] = (tt[a] >= 0) ? tt[a] / C.nb[a] : -((-tt[a] + C.nb[a] - 1) / C.nb[a]);
+            tt[a] -= n[a] * C.nb[a];
+          }
+        } else if (tt[a] < 0 || tt[a] >= C.nb[a]) {
+          ok = false;
+        }
+      }
+      if (ok) {
+        const long long tb = C.bin_base + (static_cast<long long>(tt[0]) * C.nb[1] + tt[1]) * C.nb[2] + tt[2];
+        s0 = A.bin_start[tb];
+        sz = static_cast<int>(A.bin_start[tb + 1] - s0);
+      }
+    }
+    int cst = sz;   // first candidate of each bin: exclusive prefix of the sizes
+    for (int m = 1; m < 32; m <<= 1) {
+      const int v = __shfl_up_sync(full, cst, m);
+      if (lane >= m) cst += v;
+    }
+    const int ctot = __shfl_sync(full, cst, 31);
+    cst -= sz;
+    unsigned before = static_cast<unsigned>(total);   // pairs before this lane's bin
+    uint32_t slots = 0;                               // accepted bits of its first 32 slots
+    for (int c0 = 0; c0 < ctot; c0 += 32) {
+      const int c = c0 + lane;
+      int lo = 0, hi = 31;   // the last bin that starts at or before candidate c
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (__shfl_sync(full, cst, mid) <= c) lo = mid; else hi = mid - 1;
+      }
+      const long long sb = __shfl_sync(full, s0, lo);
+      const int cq = __shfl_sync(full, cst, lo);
+      const int n0 = __shfl_sync(full, n[0], lo), n1 = __shfl_sync(full, n[1], lo), n2 = __shfl_sync(full, n[2], lo);
+      int acc = 0, j = 0, img = 0;
+      float4 r;
+      if (c < ctot) {
+        const long long s = sb + (c - cq);
+        const float4 xj_h = A.bph[s];
+        j = __float_as_int(xj_h.w);
+        if (!(j == static_cast<int>(i) && n0 == 0 && n1 == 0 && n2 == 0))
+          acc = decide(A, C, i, j, xi_h, xi_l, xj_h, A.bpl[s], n0, n1, n2, r, img);
+      }
+      const uint32_t bal = __ballot_sync(full, acc != 0);
+      if (FILL) {
+        const long long o = out0 + total + __popc(bal & ((1u << lane) - 1u));
+        if (acc && o < out1) {
+          A.pj[o] = j;
+          A.pimg[o] = img;
+          A.pr32[o] = r;
+        }
+      } else {
+        if (n_scan <= 32 && (c0 >> 5) < kMaskWords && lane == 0)
+          A.mask[static_cast<long long>(c0 >> 5) * A.n_atoms + t] = bal;
+        // candidates of this word below the lane's bin, and in its first 32 slots
+        const int rel = cst - c0;
+        if (rel > 0) before += __popc(rel >= 32 ? bal : bal & ((1u << rel) - 1u));
+        if (rel >= 0 && rel < 32) slots |= bal >> rel;
+        else if (rel < 0 && rel > -32) slots |= bal << -rel;
+      }
+      total += __popc(bal);
+    }
+    if (!FILL && A.rv && q < n_scan)
+      A.rv[static_cast<long long>(q) * A.n_atoms + t] = make_uint2(sz < 32 ? slots & ((1u << sz) - 1u) : slots, before);
+  }
+  if (lane == 0) {
+    if (!FILL) A.cnt[i] = total;
+    else if (total != out1 - out0) atomicOr(A.err, ERRF_CAPACITY);
+  }
+}
+
+// Bin starts, scatter, sort by atom index and binned copies of a small list by one block (instead of
+// a two-kernel scan, a scatter and a sort).
+constexpr int kSmallAtoms = 8192, kSmallBins = 8192;
+__global__ void __launch_bounds__(1024, 1) k_bin_small(NbrArgs A, int n_bins) {
+  extern __shared__ int sm[];
+  int* start = sm;                // [n_bins + 1]
+  int* fill = start + n_bins + 1; // [n_bins]
+  int* atoms = fill + n_bins;     // [n_atoms]
+  __shared__ int warp_sum[32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, N = static_cast<int>(A.n_atoms);
+  const int per = (n_bins + 1023) / 1024, b0 = min(n_bins, tid * per), b1 = min(n_bins, b0 + per);
+  int mine = 0;
+  for (int k = b0; k < b1; ++k) mine += A.bin_count[k];
+  int incl = mine;
+  for (int m = 1; m < 32; m <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, m);
+    if (lane >= m) incl += v;
+  }
+  if (lane == 31) warp_sum[w] = incl;
+  __syncthreads();
+  int at = incl - mine;
+  for (int k = 0; k < w; ++k) at += warp_sum[k];
+  for (int k = b0; k < b1; ++k) {
+    start[k] = at;
+    fill[k] = at;
+    A.bin_start[k] = at;
+    at += A.bin_count[k];
+  }
+  if (tid == 0) { start[n_bins] = N; A.bin_start[n_bins] = N; }
+  __syncthreads();
+  for (int i = tid; i < N; i += 1024) atoms[atomicAdd(&fill[A.atom_bin[i]], 1)] = i;
+  __syncthreads();
+  for (int k = tid; k < n_bins; k += 1024) {
+    const int s0 = start[k], s1 = start[k + 1];
+    for (int a = s0 + 1; a < s1; ++a) {
+      const int v = atoms[a];
+      int b = a - 1;
+      while (b >= s0 && atoms[b] > v) { atoms[b + 1] = atoms[b]; --b; }
+      atoms[b + 1] = v;
+    }
+  }
+  __syncthreads();
+  for (int a = tid; a < N; a += 1024) {
+    const int v = atoms[a];
+    A.bin_atoms[a] = v;
+    A.bph[a] = A.ph[v];
+    A.bpl[a] = A.pl[v];
+  }
+}
+
+// off = exclusive sums of the counts (off[n] = their total), by one block
+__global__ void __launch_bounds__(1024, 1) k_offsets_small(const long long* cnt, long long* off, int n) {
+  __shared__ int warp_sum[32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int per = (n + 1023) / 1024, b0 = min(n, tid * per), b1 = min(n, b0 + per);
+  int mine = 0;
+  for (int k = b0; k < b1; ++k) mine += static_cast<int>(cnt[k]);
+  int incl = mine;
+  for (int m = 1; m < 32; m <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, m);
+    if (lane >= m) incl += v;
+  }
+  if (lane == 31) warp_sum[w] = incl;
+  __syncthreads();
+  long long at = incl - mine;
+  for (int k = 0; k < w; ++k) at += warp_sum[k];
+  for (int k = b0; k < b1; ++k) {
+    off[k] = at;
+    at += cnt[k];
+  }
+  if (b0 < n && b1 == n) off[n] = at;
+}
+
+// Fill pass with one warp per atom (bin order), for cells that scan at most 32 bins:
 // lane q owns scanned bin q (its first binned atom, size, image and first candidate index), the
 // count pass's accepted bits are located by prefix popcounts, and lane k forms the atom's k-th
 // pair, so consecutive lanes write consecutive slots.  Candidates past the recorded bits are
@@ -348,7 +495,7 @@ __global__ void __launch_bounds__(256, 4) k_fill_warp(NbrArgs A) {
   const int w1 = 2 * C.kb[1] + 1, w2 = 2 * C.kb[2] + 1;
   const int n_scan = (2 * C.kb[0] + 1) * w1 * w2;
   const int slot_i = static_cast<int>(t - A.bin_start[A.atom_bin[i]]);   // i's slot in its bin
-  // scanned bin of this lane (same order as k_pairs): first binned atom, size, image
+  // scanned bin of this lane (same order as k_count): first binned atom, size, image
   int n[3] = {0, 0, 0};
   long long s0 = 0;
   int sz = 0;
@@ -520,10 +667,23 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   std::vector<int64_t> ao(n_cfg + 1);
   std::vector<double> cell(9 * static_cast<size_t>(n_cfg));
   std::vector<uint8_t> pbc(3 * static_cast<size_t>(n_cfg));
-  MTP_CUDA(cudaMemcpyAsync(ao.data(), b->atom_offset, ao.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  MTP_CUDA(cudaMemcpyAsync(cell.data(), b->cell, cell.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
-  MTP_CUDA(cudaMemcpyAsync(pbc.data(), b->pbc, pbc.size(), cudaMemcpyDeviceToHost, s));
-  MTP_CUDA(cudaStreamSynchronize(s));
+  {
+    // through the model's pinned buffer where they fit (a copy into pageable memory waits by itself)
+    const size_t n0 = ao.size() * sizeof(int64_t), n1 = cell.size() * sizeof(double), n2 = pbc.size();
+    const bool pin = n0 + n1 + n2 <= kPinBytes;
+    char* h0 = pin ? static_cast<char*>(m->pin) : reinterpret_cast<char*>(ao.data());
+    char* h1 = pin ? h0 + n0 : reinterpret_cast<char*>(cell.data());
+    char* h2 = pin ? h1 + n1 : reinterpret_cast<char*>(pbc.data());
+    MTP_CUDA(cudaMemcpyAsync(h0, b->atom_offset, n0, cudaMemcpyDeviceToHost, s));
+    MTP_CUDA(cudaMemcpyAsync(h1, b->cell, n1, cudaMemcpyDeviceToHost, s));
+    MTP_CUDA(cudaMemcpyAsync(h2, b->pbc, n2, cudaMemcpyDeviceToHost, s));
+    MTP_CUDA(cudaStreamSynchronize(s));
+    if (pin) {
+      std::memcpy(ao.data(), h0, n0);
+      std::memcpy(cell.data(), h1, n1);
+      std::memcpy(pbc.data(), h2, n2);
+    }
+  }
   if (ao[0] != 0) throw Fail{MTP_ERR_ARG, "atom_offset[0] must be 0"};
   for (int k = 0; k < n_cfg; ++k)
     if (ao[k + 1] < ao[k]) throw Fail{MTP_ERR_ARG, "atom_offset must be non-decreasing"};
@@ -531,9 +691,17 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   if (N <= 0) throw Fail{MTP_ERR_ARG, "empty batch"};
   if (N >= (int64_t(1) << 31)) throw Fail{MTP_ERR_UNSUPPORTED, "more than 2^31 atoms"};
   const double rc = m->desc.r_cut;
+  // the plan of these cells, kept in the list while offsets, cells and periodicity stay the same
+  // values (a constant-volume run): a comparison instead of the loop below and four uploads
+  const bool same = nb->plan_valid && nb->plan_rc == rc && nb->atom_offset == ao && nb->plan_cell == cell && nb->plan_pbc == pbc;
+  long long bins = nb->n_bins_total;
+  size_t n_shift = nb->plan_shifts;
+  int max_scan = nb->plan_max_scan;
+  if (!same) {
+  nb->plan_valid = false;
   std::vector<DevCfg> cfgs(n_cfg);
   std::vector<float4> shi, slo;
-  long long bins = 0;
+  bins = 0;
   nb->seg_host.clear();
   for (int k = 0; k < n_cfg; ++k) {
     DevCfg& C = cfgs[k];
@@ -590,7 +758,6 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
       nb->seg_host.push_back(std::min<int64_t>(a0 + 4096, ao[k + 1]));
     }
   }
-  nb->n_atoms = N;
   nb->n_cfg = n_cfg;
   nb->atom_offset = ao;
   nb->n_bins_total = bins;
@@ -606,6 +773,20 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   nb->seg.ensure(nb->seg_host.size() * sizeof(int64_t), s);
   MTP_CUDA(cudaMemcpyAsync(nb->seg.p, nb->seg_host.data(), nb->seg_host.size() * sizeof(int64_t),
                            cudaMemcpyHostToDevice, s));
+  max_scan = 0;
+  for (const DevCfg& C : cfgs) max_scan = std::max(max_scan, (2 * C.kb[0] + 1) * (2 * C.kb[1] + 1) * (2 * C.kb[2] + 1));
+  n_shift = shi.size();
+  nb->plan_shifts = n_shift;
+  nb->plan_max_scan = max_scan;
+  nb->plan_rc = rc;
+  nb->plan_cell = cell;
+  nb->plan_pbc = pbc;
+  nb->plan_valid = true;
+  }
+  nb->n_atoms = N;
+  DevCfg* d_cfg = nb->plan.as<DevCfg>();
+  float4* d_shi = reinterpret_cast<float4*>(reinterpret_cast<char*>(d_cfg) + ((n_cfg * sizeof(DevCfg) + 15) & ~size_t(15)));
+  float4* d_slo = d_shi + n_shift;
   nb->atom_cfg.ensure(N * sizeof(int), s);
   nb->wrap.ensure(N * sizeof(int) + N * sizeof(long long) + 2 * N * sizeof(float4) + N * sizeof(int) + 64, s);
   int* d_wrap = nb->wrap.as<int>();
@@ -626,8 +807,9 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   nb->off.ensure((N + 1) * sizeof(long long), s);
   m->err_flag.ensure(sizeof(unsigned), s);
   MTP_CUDA(cudaMemsetAsync(m->err_flag.p, 0, sizeof(unsigned), s));
-  MTP_CUDA(cudaMemsetAsync(d_bcount, 0, 2 * (bins + 1) * sizeof(int), s));
-  MTP_CUDA(cudaMemsetAsync(nb->counts.p, 0, (N + 1) * sizeof(long long), s));
+  MTP_CUDA(cudaMemsetAsync(d_bcount, 0, 2 * (bins + 1) * sizeof(int), s));   // counts and fill counters
+  const bool small = N <= kSmallAtoms && bins <= kSmallBins;
+  if (!small) MTP_CUDA(cudaMemsetAsync(nb->counts.as<long long>() + N, 0, sizeof(long long), s));
 
   NbrArgs A{};
   A.n_atoms = N;
@@ -656,10 +838,10 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   A.err = m->err_flag.as<unsigned>();
   nb->masks.ensure(static_cast<size_t>(N) * kMaskWords * sizeof(uint32_t), s);
   A.mask = nb->masks.as<uint32_t>();
-  // the warp fill and the reverse record, when every configuration scans at most 32 bins
-  int max_scan = 0;
-  for (const DevCfg& C : cfgs) max_scan = std::max(max_scan, (2 * C.kb[0] + 1) * (2 * C.kb[1] + 1) * (2 * C.kb[2] + 1));
+  // the replaying fill and the reverse record, when every configuration scans at most 32 bins; the
+  // count pass by threads there from kCountThreads atoms on
   const bool warp_fill = max_scan <= kWarpScan;
+  const bool warp_count = !warp_fill || N < kCountThreads;
   A.rv = nullptr;
   if (warp_fill) {
     nb->segs.ensure(static_cast<size_t>(max_scan) * N * sizeof(uint2), s);
@@ -671,30 +853,50 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
     k_prep<<<blocks_for(N, TB), TB, 0, s>>>(A);
     ProfRegion::launched();
     MTP_CUDA(cudaGetLastError());
-    // bin_count has bins+1 entries (last = 0) -> bin_start[bins] = N
-    {
-      // scan int counts into long long starts
+    if (small) {
+      const size_t smem = (2 * static_cast<size_t>(bins) + 1 + N) * sizeof(int);
+      if (smem > 48 * 1024)
+        MTP_CUDA(cudaFuncSetAttribute(k_bin_small, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+      k_bin_small<<<1, 1024, smem, s>>>(A, static_cast<int>(bins));
+      ProfRegion::launched();
+      MTP_CUDA(cudaGetLastError());
+    } else {
+      // bin_count has bins+1 entries (last = 0) -> bin_start[bins] = N; int counts into long long starts
       size_t bytes = 0;
       MTP_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, bytes, d_bcount, d_bstart, bins + 1, s));
       nb->scratch.ensure(bytes, s);
       MTP_CUDA(cub::DeviceScan::ExclusiveSum(nb->scratch.p, bytes, d_bcount, d_bstart, bins + 1, s));
+      k_scatter<<<blocks_for(N, TB), TB, 0, s>>>(A);
+      ProfRegion::launched();
+      MTP_CUDA(cudaGetLastError());
+      k_sort_bins<<<blocks_for(bins, TB), TB, 0, s>>>(A, bins);
+      ProfRegion::launched();
+      MTP_CUDA(cudaGetLastError());
     }
-    k_scatter<<<blocks_for(N, TB), TB, 0, s>>>(A);
+    if (warp_count) k_scan_warp<false><<<blocks_for(N * 32, 128), 128, 0, s>>>(A);
+    else k_count<<<blocks_for(N, 128), 128, 0, s>>>(A);
     ProfRegion::launched();
     MTP_CUDA(cudaGetLastError());
-    k_sort_bins<<<blocks_for(bins, TB), TB, 0, s>>>(A, bins);
-    ProfRegion::launched();
-    MTP_CUDA(cudaGetLastError());
-    k_pairs<false><<<blocks_for(N, 128), 128, 0, s>>>(A);
-    ProfRegion::launched();
-    MTP_CUDA(cudaGetLastError());
-    scan_exclusive<long long>(nb->counts.as<long long>(), nb->off.as<long long>(), N + 1, nb->scratch, s);
+    if (small) {
+      k_offsets_small<<<1, 1024, 0, s>>>(A.cnt, nb->off.as<long long>(), static_cast<int>(N));
+      ProfRegion::launched();
+      MTP_CUDA(cudaGetLastError());
+    } else {
+      scan_exclusive<long long>(nb->counts.as<long long>(), nb->off.as<long long>(), N + 1, nb->scratch, s);
+    }
   }
-  long long total = 0;
+  volatile long long* h_total = static_cast<long long*>(m->pin);
+  volatile unsigned* h_flag = reinterpret_cast<unsigned*>(static_cast<char*>(m->pin) + 16);
   unsigned flag = 0;
-  MTP_CUDA(cudaMemcpyAsync(&total, nb->off.as<long long>() + N, sizeof(long long), cudaMemcpyDeviceToHost, s));
-  MTP_CUDA(cudaMemcpyAsync(&flag, m->err_flag.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-  MTP_CUDA(cudaStreamSynchronize(s));
+  auto read_flag = [&] {
+    MTP_CUDA(cudaMemcpyAsync(const_cast<unsigned*>(h_flag), m->err_flag.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+    MTP_CUDA(cudaStreamSynchronize(s));
+    flag = *h_flag;
+  };
+  MTP_CUDA(cudaMemcpyAsync(const_cast<long long*>(h_total), nb->off.as<long long>() + N, sizeof(long long),
+                           cudaMemcpyDeviceToHost, s));
+  read_flag();
+  const long long total = *h_total;
   if (flag & ERRF_SPECIES) throw Fail{MTP_ERR_ARG, "species outside [0, n_types)"};
   if (flag & ERRF_NONFINITE) throw Fail{MTP_ERR_NUMERIC, "non-finite position"};
   if (flag & ERRF_GEOMETRY) throw Fail{MTP_ERR_GEOMETRY, "coincident atoms (|r_ij| < 1e-8 A)"};
@@ -718,7 +920,7 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
         k_fill_warp<<<blocks_for(N * 32, 256), 256, 0, s>>>(A);
         ProfRegion::launched();
       } else {
-        k_pairs<true><<<blocks_for(N, 128), 128, 0, s>>>(A);
+        k_scan_warp<true><<<blocks_for(N * 32, 128), 128, 0, s>>>(A);
         ProfRegion::launched();
       }
       MTP_CUDA(cudaGetLastError());
@@ -729,8 +931,7 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
       ProfRegion::launched();
       MTP_CUDA(cudaGetLastError());
     }
-    MTP_CUDA(cudaMemcpyAsync(&flag, m->err_flag.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-    MTP_CUDA(cudaStreamSynchronize(s));
+    read_flag();
     if (take_injected(g_inject_overflow)) flag |= ERRF_CAPACITY;
     if (flag & ERRF_GEOMETRY) throw Fail{MTP_ERR_GEOMETRY, "coincident atoms (|r_ij| < 1e-8 A)"};
     if (!(flag & ERRF_CAPACITY)) break;
@@ -745,8 +946,7 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
       ProfRegion::launched();
       MTP_CUDA(cudaGetLastError());
     }
-    MTP_CUDA(cudaMemcpyAsync(&flag, m->err_flag.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-    MTP_CUDA(cudaStreamSynchronize(s));
+    read_flag();
   }
   if (flag & ERRF_REVERSE) throw Fail{MTP_ERR_NUMERIC, "inconsistent neighbor list (reverse-pair mismatch)"};
   DevNbr& D = nb->dn;
