@@ -596,7 +596,8 @@ void upload_theta(mtp_model* md) {
 }
 
 void run_grade_simt(mtp_model* md, int64_t N, bool fp64, const double* rows, const float* rows_f, int64_t ld,
-                    double* gamma, int32_t* argmax, cudaStream_t s);
+                    double* gamma, int32_t* argmax, const unsigned char* only, cudaStream_t s);
+void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, double* gamma, int32_t* argmax, cudaStream_t s);
 bool grade_tc_available(const mtp_model* md);
 void run_grade_tc(mtp_model* md, int64_t N, const float* hi, const float* lo, int64_t ld, double* gamma,
                   int32_t* argmax, const int32_t* zrow, const int64_t* row_atom, cudaStream_t s);
@@ -735,7 +736,8 @@ void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_prec
   }
   if (want_grade) {
     if (use_tc) run_grade_tc(m, N, o.rows_hi, o.rows_lo, ld, gamma, argmax, zrow, row_atom, s);
-    else run_grade_simt(m, N, fp64, o.rows, o.rows_hi, ld, gamma, argmax, s);
+    else if (fp64) run_grade_fp64(m, N, o.rows, ld, gamma, argmax, s);
+    else run_grade_simt(m, N, false, nullptr, o.rows_hi, ld, gamma, argmax, nullptr, s);
     if (flagged || n_flagged) {
       int64_t* cnt = n_flagged;
       int32_t* fl = flagged;
@@ -853,7 +855,7 @@ void mtp_free_model(mtp_model* md) {
   cudaGetDevice(&cur);
   cudaSetDevice(md->device);
   cudaDeviceSynchronize();
-  for (DevBuf* b : {&md->sched_buf, &md->theta_buf, &md->a_d, &md->ainv_d, &md->ainv_f, &md->ws_pair,
+  for (DevBuf* b : {&md->sched_buf, &md->theta_buf, &md->a_d, &md->ainv_d, &md->ainv_f, &md->ainv_s, &md->ws_pair,
                     &md->ws_atom, &md->ws_rows, &md->ws_grade, &md->ws_sort, &md->ws_misc, &md->ws_red,
                     &md->err_flag, &md->async_err, &md->split_tab, &md->ws_mom, &md->wide_tab, &md->ws_wide})
     b->release();
@@ -1396,7 +1398,7 @@ mtp_status mtp_config_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb
       give_wide(md, N, prec == MTP_FP64, false, o, s);
       run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
       run_config_row_sums(nb, md->ws_rows.as<double>(), m, rc, md->ws_red, s);
-      run_grade_simt(md, K, true, rc, nullptr, m, gamma_cfg, am, s);
+      run_grade_fp64(md, K, rc, m, gamma_cfg, am, s);
       if (worst) run_widen_argmax(am, K, worst, s);
     }
     if (cls) run_classify(gamma_cfg, K, gamma_save, gamma_break, cls, s);

@@ -206,6 +206,7 @@ struct mtp_model {
   mtp::DevBuf ainv_d;          // m x m FP64
   mtp::DevBuf ainv_f;          // padded FP32 (hi) and (lo) for the mixed grade
   int64_t ainv_ld = 0;
+  mtp::DevBuf ainv_s;          // slices of A^-1 for the FP64 grade (grade_fp64.cu)
   // workspaces
   mtp::DevBuf ws_pair;         // per-pair gradients
   mtp::DevBuf ws_atom;         // per-atom V, W
