@@ -138,18 +138,36 @@ __global__ void k_scatter(NbrArgs A) {
   A.bin_atoms[A.bin_start[bin] + slot] = static_cast<int>(i);
 }
 
-__global__ void k_sort_bins(NbrArgs A, long long n_bins) {
-  long long bn = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
+// Sorts each bin by atom index and makes the binned copies, a warp per bin: a lane per atom ranks it
+// among the bin's (bins of more than 32 atoms: insertion by one lane).  A thread per bin moved
+// entries in global memory one by one (16,384 atoms: 44 -> 4.5 us).
+__global__ void __launch_bounds__(256) k_sort_bins(NbrArgs A, long long n_bins) {
+  const long long bn = (blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x) >> 5;
   if (bn >= n_bins) return;
-  long long s0 = A.bin_start[bn], s1 = A.bin_start[bn + 1];
-  for (long long a = s0 + 1; a < s1; ++a) {
-    int v = A.bin_atoms[a];
-    long long b = a - 1;
-    while (b >= s0 && A.bin_atoms[b] > v) { A.bin_atoms[b + 1] = A.bin_atoms[b]; --b; }
-    A.bin_atoms[b + 1] = v;
+  const int lane = threadIdx.x & 31;
+  const long long s0 = A.bin_start[bn], s1 = A.bin_start[bn + 1];
+  const int sz = static_cast<int>(s1 - s0);
+  if (sz <= 32) {
+    const int v = lane < sz ? A.bin_atoms[s0 + lane] : 0x7fffffff;
+    int rank = 0;
+    for (int k = 0; k < sz; ++k) rank += __shfl_sync(0xffffffffu, v, k) < v ? 1 : 0;
+    if (lane < sz) {
+      A.bin_atoms[s0 + rank] = v;
+      A.bph[s0 + rank] = A.ph[v];
+      A.bpl[s0 + rank] = A.pl[v];
+    }
+    return;
   }
-  for (long long a = s0; a < s1; ++a) {
-    int v = A.bin_atoms[a];
+  if (lane == 0)
+    for (long long a = s0 + 1; a < s1; ++a) {
+      int v = A.bin_atoms[a];
+      long long b = a - 1;
+      while (b >= s0 && A.bin_atoms[b] > v) { A.bin_atoms[b + 1] = A.bin_atoms[b]; --b; }
+      A.bin_atoms[b + 1] = v;
+    }
+  __syncwarp();
+  for (long long a = s0 + lane; a < s1; a += 32) {
+    const int v = A.bin_atoms[a];
     A.bph[a] = A.ph[v];
     A.bpl[a] = A.pl[v];
   }
@@ -869,7 +887,7 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
       k_scatter<<<blocks_for(N, TB), TB, 0, s>>>(A);
       ProfRegion::launched();
       MTP_CUDA(cudaGetLastError());
-      k_sort_bins<<<blocks_for(bins, TB), TB, 0, s>>>(A, bins);
+      k_sort_bins<<<blocks_for(bins * 32, TB), TB, 0, s>>>(A, bins);
       ProfRegion::launched();
       MTP_CUDA(cudaGetLastError());
     }
