@@ -6,14 +6,14 @@
 //               32-component chunk of the moment set each lane sums f_mu x^a y^b z^c over its
 //               own pairs in registers and one 3-stage butterfly over the 8 lanes leaves each
 //               lane with 4 component sums.  Output: the moments, FP32, [work x ldm].
-//   k_contract  (eqs. 2, 5-6 and their adjoint)  one or two neighborhoods per warp carried
-//               through the contraction schedule (32-lane slabs of packed triples in shared
-//               memory, as in site_fast.cu), V_i = s_z + sum_a xi_a B_a, the reverse pass seeded
-//               with xi, and the adjoints dV/dM written over the moments.  The basis part of
-//               the parameter row b_i (eq. 9) is written here.
+//   contraction (eqs. 2, 5-6 and their adjoint)  V_i = s_z + sum_a xi_a B_a, the reverse pass
+//               seeded with xi, the adjoints dV/dM written over the moments, the basis part of the
+//               parameter row b_i (eq. 9): k_contract_group (site_group.cu), or, where
+//               mtp_set_split_shape asks for a shape, k_contract here (one or two neighborhoods
+//               per warp carried through 32-lane slabs of packed triples).
 //   k_adjoint   (forces and virial; the radial block of eq. 9)  8 lanes per neighborhood: per
-//               pair dV_i/dr_ij from dV/dM (monomials regenerated in registers), the per-pair
-//               gradients for the force gather, the neighborhood's virial, and
+//               pair dV_i/dr_ij from dV/dM (nested Horner schemes over packed slices of the
+//               polynomials in x, y, z), the per-pair gradients for the force gather, the neighborhood's virial, and
 //               sum_j g_mu(j) Q_b(r_ij) per neighbor species for b_i.
 //
 // Splitting frees each phase from the others' resources: the contraction runs without the
@@ -41,7 +41,7 @@ constexpr int kNQs = 8;      // radial polynomials of the specialised kernels
 constexpr int LPN = 8;       // lanes per neighborhood in the per-pair kernels
 constexpr int GPW = 32 / LPN;
 constexpr int BATCH = 64;    // pairs staged per neighborhood at a time (moments)
-constexpr int BATCH_A = 2 * LPN;   // pairs per neighborhood at a time (pair adjoint: two per lane)
+constexpr int BATCH_A = LPN;   // pairs per neighborhood at a time (pair adjoint: one per lane)
 constexpr int GS = 20;       // floats staged per pair for the radial block: g_mu (8), Q_b (8), species; 16-byte aligned
 
 // float4 arrays staged per pair by the moment kernel: (x, y, z, f_0), then f_1.. four at a time
@@ -51,13 +51,15 @@ __host__ __device__ constexpr int stage_f4(int nr) { return 1 + (nr - 1 + 3) / 4
 __host__ __device__ constexpr int pre_of(int nr) { return nr <= 5 ? 10 : 19; }
 __host__ __device__ constexpr int tmax_of(int nr) { return nr <= 5 ? 3 : 4; }
 
-// shared-memory floats per neighborhood group of the pair-adjoint kernel: dV/dM (ldm rounded up to
-// 32) then the radial-block staging, plus 8: the stride is 8 mod 32 banks, so the four groups'
-// broadcast reads of one component hit different banks
-__host__ __device__ inline int adj_region(int ldm, bool rows) {
-  return ((ldm + 31) & ~31) + 8 + (rows ? BATCH_A * GS : 0);
+// shared-memory floats per neighborhood group of the pair-adjoint kernel: dV/dM in `packed` floats
+// (rounded up to 32), then the radial-block staging or the row's block on its way out (at most 192),
+// plus 8: the stride is 8 mod 32 banks, so the four groups' broadcast reads of one component hit
+// different banks
+__host__ __device__ constexpr int adj_region(int packed, bool rows) {
+  return ((packed + 31) & ~31) + 8 + (rows ? 192 : 0);
 }
-// its blocks per SM (128 registers for two; level 24 is faster with more registers: 1.99 against 2.31 ms)
+static_assert(BATCH_A * GS <= 192, "radial-block staging");
+// its blocks per SM (128 registers for two; level 24 takes 167)
 constexpr int adj_blocks(int nr) { return nr <= 5 ? 2 : 1; }
 
 struct SplitArgs {
@@ -70,7 +72,7 @@ struct SplitArgs {
                 // slot order (monomial-major, the order of the moment pass's chunks)
   int ldm;
   const int* slot_comp;     // slot -> value index of the moment component
-  const int* slot_horner;   // slot -> place in the pair adjoint's order
+  const int* slot_horner;   // slot -> place among the pair adjoint's slices
   int T, CBN, NC, NV;
   // contraction kernel: shared-memory layout (word offsets of the schedule arrays)
   size_t c_bytes, sched_bytes, warp_bytes, total;
@@ -816,99 +818,107 @@ __global__ void __launch_bounds__(SCH == 1 ? 256 : (SCH == 2 ? 384 : 512), 1) k_
 // ------------------------------------------------------------------------------------
 // pair adjoint: per-pair gradients, the neighborhood's virial, the radial block of b_i
 // ------------------------------------------------------------------------------------
-// dV/dM of a neighborhood in the order the nested Horner schemes read it: mu, then descending
-// powers a of x, b of y, c of z
+// dV/dM of a neighborhood as the pair adjoint reads it.  P_mu(r) = sum_k (dV/dM_mu,k) x^a y^b z^c is a
+// sum over a of x^a times a polynomial in y and z, the slice (mu, a) of degree numax(mu) - a.  Slices
+// are sorted by degree and taken two by two, side by side in packed FP32: per pair of slices the
+// coefficients by descending powers b of y, then c of z, of the larger degree (zeros where the
+// smaller slice has none).
 template <int NR, int NU0>
-struct HornerOrder {
+struct Slices {
   using Sh = Shape<NR, NU0>;
-  // position of (mu, a, b) with the highest power of z
-  static constexpr int at(int mu, int a, int b) {
-    int p = 0;
-    for (int m = 0; m < mu; ++m) p += nmono_upto(Sh::numax(m));
-    const int n = Sh::numax(mu);
-    for (int x = n; x > a; --x) p += (n - x + 1) * (n - x + 2) / 2;
-    for (int y = n - a; y > b; --y) p += n - a - y + 1;
-    return p;
+  static constexpr int count() {
+    int n = 0;
+    for (int mu = 0; mu < NR; ++mu) n += Sh::numax(mu) + 1;
+    return n;
   }
-  static std::vector<int> of_slots() {
+  static constexpr int N = count(), NP = (N + 1) / 2;
+  struct Table {
+    int mu[2 * NP], a[2 * NP], deg[2 * NP], first[NP + 1];   // first: packed index of a pair's coefficients
+  };
+  static constexpr Table make() {
+    Table t{};
+    int n = 0;
+    for (int d = NU0; d >= 0; --d)
+      for (int mu = 0; mu < NR; ++mu) {
+        const int a = Sh::numax(mu) - d;
+        if (a >= 0) { t.mu[n] = mu; t.a[n] = a; t.deg[n] = d; ++n; }
+      }
+    if (n < 2 * NP) { t.mu[n] = -1; t.a[n] = 0; t.deg[n] = -1; }
+    for (int p = 0; p < NP; ++p) t.first[p + 1] = t.first[p] + (t.deg[2 * p] + 1) * (t.deg[2 * p] + 2) / 2;
+    return t;
+  }
+  static constexpr Table T = make();
+  static constexpr int FLOATS = 2 * ((T.first[NP] + 1) & ~1);   // whole 16-byte loads
+  // coefficient (b, c) of slice pair p in packed units
+  static constexpr int at(int p, int b, int c) {
+    int i = T.first[p];
+    for (int y = T.deg[2 * p]; y > b; --y) i += T.deg[2 * p] - y + 1;
+    return i + (T.deg[2 * p] - b - c);
+  }
+  static std::vector<int> of_slots() {   // slot -> float
     constexpr auto S = make_slots<NR, NU0>();
     constexpr auto M = make_mono<NU0>();
-    std::vector<int> t(Sh::NCOMP);
-    for (int s = 0; s < Sh::NCOMP; ++s) {
-      const int k = S.k[s], mu = S.mu[s], top = Sh::numax(mu) - M.a[k] - M.b[k];
-      t[s] = at(mu, M.a[k], M.b[k]) + (top - M.c[k]);
-    }
+    std::vector<int> t(Sh::NCOMP, 0);
+    for (int s = 0; s < Sh::NCOMP; ++s)
+      for (int n = 0; n < N; ++n)
+        if (T.mu[n] == S.mu[s] && T.a[n] == M.a[S.k[s]]) t[s] = 2 * at(n / 2, M.b[S.k[s]], M.c[S.k[s]]) + n % 2;
     return t;
   }
 };
 
-// Values P_mu(r) = sum_k (dV/dM_mu,k) x^a y^b z^c of two pairs at once (packed), and their
-// gradients through `use(mu, P, dP/dx, dP/dy, dP/dz)`.  Per component two packed FMAs and, four at a
-// time, a broadcast load; per (a, b) three more.  G: Horner order, 16-byte aligned.
+// Values of the slice pairs and their derivatives in y and z at one (y, z) through
+// `use(pair, S, dS/dy, dS/dz)` (packed).  Per packed coefficient two FMAs by nested Horner schemes
+// and half a 128-bit broadcast load, per (slice, b) three more.  G: 16-byte aligned.
 template <int NR, int NU0, class Use>
-__device__ __forceinline__ void horner_pass(const float* G, u64 x, u64 y, u64 z, Use&& use) {
-  using Sh = Shape<NR, NU0>;
-  using HO = HornerOrder<NR, NU0>;
-  float4 cur = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto get = [&](auto I) -> u64 {   // component I (called in ascending order)
+__device__ __forceinline__ void slice_pass(const float* G, float y, float z, Use&& use) {
+  using Sl = Slices<NR, NU0>;
+  const u64 y2 = pack2(y, y), z2 = pack2(z, z);
+  ulonglong2 cur = make_ulonglong2(0, 0);
+  auto get = [&](auto I) -> u64 {   // packed coefficient I (called in ascending order)
     constexpr int i = decltype(I)::value;
-    if constexpr (i % 4 == 0) cur = *reinterpret_cast<const float4*>(G + i);
-    const float v = i % 4 == 0 ? cur.x : (i % 4 == 1 ? cur.y : (i % 4 == 2 ? cur.z : cur.w));
-    return pack2(v, v);
+    if constexpr (i % 2 == 0) cur = *reinterpret_cast<const ulonglong2*>(G + 2 * i);
+    return i % 2 == 0 ? cur.x : cur.y;
   };
-  static_for<0, NR>([&](auto Mu) {
-    constexpr int mu = decltype(Mu)::value, n = Sh::numax(mu);
-    u64 pv = 0, px = 0, py = 0, pz = 0;
-    static_for<0, n + 1>([&](auto A) {
-      constexpr int a = n - decltype(A)::value, na = n - a;
-      u64 av = 0, ay = 0, az = 0;
-      static_for<0, na + 1>([&](auto B) {
-        constexpr int b = na - decltype(B)::value, nc = na - b, i0 = HO::at(mu, a, b);
-        u64 t = get(std::integral_constant<int, i0>{}), u = 0;
-        static_for<1, nc + 1>([&](auto C) {
-          constexpr int c = decltype(C)::value;
-          u = c == 1 ? t : fma2(u, z, t);
-          t = fma2(t, z, get(std::integral_constant<int, i0 + c>{}));
-        });
-        if constexpr (b == na) {
-          av = t;
-          az = u;
-        } else {
-          ay = b == na - 1 ? av : fma2(ay, y, av);
-          az = fma2(az, y, u);
-          av = fma2(av, y, t);
-        }
+  static_for<0, Sl::NP>([&](auto Pp) {
+    constexpr int p = decltype(Pp)::value, n = Sl::T.deg[2 * p];
+    u64 av = 0, ay = 0, az = 0;
+    static_for<0, n + 1>([&](auto B) {
+      constexpr int b = n - decltype(B)::value, nc = n - b, i0 = Sl::at(p, b, nc);
+      u64 t = get(std::integral_constant<int, i0>{}), u = 0;
+      static_for<1, nc + 1>([&](auto C) {
+        constexpr int c = decltype(C)::value;
+        u = c == 1 ? t : fma2(u, z2, t);
+        t = fma2(t, z2, get(std::integral_constant<int, i0 + c>{}));
       });
-      if constexpr (a == n) {
-        pv = av;
-        py = ay;
-        pz = az;
+      if constexpr (b == n) {
+        av = t;
+        az = u;
       } else {
-        px = a == n - 1 ? pv : fma2(px, x, pv);
-        py = fma2(py, x, ay);
-        pz = fma2(pz, x, az);
-        pv = fma2(pv, x, av);
+        ay = b == n - 1 ? av : fma2(ay, y2, av);
+        az = fma2(az, y2, u);
+        av = fma2(av, y2, t);
       }
-      // keeps the loads of later components from being hoisted wholesale
-      if constexpr (na >= 3) asm volatile("" ::: "memory");
     });
-    use(Mu, pv, px, py, pz);
+    use(Pp, av, ay, az);
+    // keeps the loads of later slices from being hoisted wholesale
+    if constexpr (n >= 3) asm volatile("" ::: "memory");
   });
 }
 
-// What bounds it: issue and the latency of dependent FMAs (9,300 warp instructions per four
-// neighborhoods at level 20, half an instruction per clock and scheduler; a third of them moves
-// that double a loaded component for the packed FMAs: loading it doubled from shared memory was
-// slower, 5.70 ms).  A lane takes two pairs, packed (fma.rn.f32x2), and walks nested Horner schemes:
-// at level 20 785 packed FMAs per two pairs instead of about 1,400 scalar operations per pair over a
-// register array of 165 monomials.  Rows are written by whole warps, their zero blocks without a
-// division per entry.  Level 20, 1,048,576 atoms (with rows): 5.33 -> 4.09 ms; level 16, 128,000
-// atoms 0.281 -> 0.220; level 24, 131,072 atoms 3.68 -> 1.99.
+// What bounds it: issue and the latency of dependent FMAs.  A lane takes a pair; the coefficients of
+// two slices lie side by side in shared memory, so that a 128-bit broadcast load feeds two packed
+// FMAs without a move (packing two pairs instead, with each coefficient doubled by moves: 4.09 ms at
+// level 20; loaded doubled: 5.70).  The pairs' loads run one and two passes ahead.  Rows are written by
+// whole warps, their zero blocks without a division per entry.  Before (scalar recursion over a
+// register array of 165 monomials, 1,400 operations per pair) and now: level 20, 1,048,576 atoms, with
+// rows 5.33 -> 3.16 ms; level 16, 128,000 atoms 0.281 -> 0.178; level 24, 131,072 atoms 3.68 -> 1.30.
 template <int NR, int NU0, bool ROWS>
 __global__ void __launch_bounds__(256, adj_blocks(NR)) k_adjoint(SplitArgs P) {
   using Sh = Shape<NR, NU0>;
-  constexpr int NQ = kNQs;
+  using Sl = Slices<NR, NU0>;
+  constexpr int NQ = kNQs, GF = (Sl::FLOATS + 31) & ~31;
   static_assert(NR <= 8 && 8 + NQ + 1 <= GS, "radial-block staging");
+  static_assert(tmax_of(NR) * NR * NQ <= 192, "the row's radial block goes out through the staging");
   extern __shared__ __align__(16) unsigned char smem[];
   const DevSchedule& d = P.d;
   const int T = P.T;
@@ -916,14 +926,14 @@ __global__ void __launch_bounds__(256, adj_blocks(NR)) k_adjoint(SplitArgs P) {
   for (int k = threadIdx.x; k < P.NC; k += blockDim.x) ctab[k] = d.theta_f[T + d.n_lin + k];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = lane / LPN, q = lane % LPN;
   const int nwarps = blockDim.x >> 5;
-  const int gstride = adj_region(P.ldm, ROWS);
+  constexpr int gstride = adj_region(Sl::FLOATS, ROWS);
   float* gM = reinterpret_cast<float*>(smem + P.c_bytes) + (static_cast<size_t>(warp) * GPW + grp) * gstride;
-  float* rstg = gM + ((P.ldm + 31) & ~31);
-  float* rblk = gM;   // radial block of the row on its way out (at most T NR NQ floats)
+  float* rstg = gM + GF;
+  float* rblk = rstg;   // radial block of the row on its way out
+  for (int k = q; k < GF; k += LPN) gM[k] = 0.f;   // the padding of the smaller slices stays 0
   __syncthreads();
   const float rmin = static_cast<float>(d.r_min), rcut = static_cast<float>(d.r_cut);
   const float sc = 1.f / (rcut - rmin);
-  const u64 one2 = pack2(1.f, 1.f);
   for (int64_t w0 = (static_cast<int64_t>(blockIdx.x) * nwarps + warp) * GPW; w0 < P.n_work;
        w0 += static_cast<int64_t>(gridDim.x) * nwarps * GPW) {
     const int64_t wk = w0 + grp;
@@ -937,19 +947,38 @@ __global__ void __launch_bounds__(256, adj_blocks(NR)) k_adjoint(SplitArgs P) {
       np = static_cast<int>(P.nb.off[i + 1] - p0);
       if (!OK(zi, T, 41) || !OK(p0 + np - 1 + (np == 0), P.nb.n_pairs + 1, 42)) { zi = 0; np = 0; }
     }
+    // the pairs' loads run ahead of the arithmetic: r_ij and the species by one pass, the neighbor by two
+    auto load_j = [&](int t) {
+      int j = -1;
+      if (t < np && OK(p0 + t, P.nb.n_pairs, 45)) j = P.nb.pj[p0 + t];
+      if (j >= 0 && !OK(j, P.nb.n_atoms, 47)) j = -1;
+      return j;
+    };
+    auto load_r = [&](int t, int j, float4& r, int& zj) {   // lanes without a pair work on a dummy one
+      r = make_float4(1.f, 0.f, 0.f, 1.f);
+      zj = 0;
+      if (j >= 0) {
+        r = P.nb.pr32[p0 + t];
+        zj = P.type[j];
+        if (!OK(zj, T, 48)) zj = 0;
+      }
+    };
+    int j_n = load_j(q), j_nn = load_j(LPN + q), zj_n;
+    float4 r_n;
     int np_max = np;
     for (int m = 16; m; m >>= 1) np_max = max(np_max, __shfl_xor_sync(0xffffffffu, np_max, m));
     __syncwarp();
     if (live) {
       const float* src = P.mom + wk * P.ldm;
       for (int k = q; k < Sh::NCOMP; k += LPN)
-        if (OK(P.slot_horner[k], P.ldm, 43) && OK(wk * P.ldm + k, P.n_work * P.ldm, 44)) gM[P.slot_horner[k]] = __ldcs(src + k);
+        if (OK(P.slot_horner[k], GF, 43) && OK(wk * P.ldm + k, P.n_work * P.ldm, 44)) gM[P.slot_horner[k]] = __ldcs(src + k);
     }
+    load_r(q, j_n, r_n, zj_n);
     __syncwarp();
     const float* czi = ctab + static_cast<size_t>(zi) * T * NR * NQ;
-    u64 Wl[9];
+    float Wl[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) Wl[k] = 0;
+    for (int k = 0; k < 9; ++k) Wl[k] = 0.f;
     // radial block accumulators: lane q owns beta = q for every (species, mu), mu in packed pairs
     constexpr int TM = tmax_of(NR), MP = (NR + 1) / 2;
     u64 cb[TM][MP];
@@ -958,106 +987,109 @@ __global__ void __launch_bounds__(256, adj_blocks(NR)) k_adjoint(SplitArgs P) {
 #pragma unroll
       for (int k = 0; k < MP; ++k) cb[z][k] = 0;
     float* Gout = static_cast<float*>(P.o.G);
-    for (int base = 0; base < np_max; base += BATCH_A) {
-      // lane q: pairs base + q and base + LPN + q; lanes without a pair work on a dummy one
-      float4 r[2];
-      int zj[2];
-      bool act[2];
-      int64_t p[2];
+    for (int base = 0; base < np_max; base += LPN) {
+      const float4 r = r_n;
+      const int zj = zj_n;
+      const bool act = j_n >= 0;
+      const int64_t p = p0 + base + q;
+      j_n = j_nn;
+      load_r(base + LPN + q, j_n, r_n, zj_n);
+      j_nn = load_j(base + 2 * LPN + q);
+      // T_b and b U_(b-1) = T_b', w = R_cut - r; f_mu = w^2 sum c T_b,
+      // f_mu' = (dx/dr) w^2 sum c T_b' - 2 w sum c T_b
+      const float t1 = (2.f * r.w - (rmin + rcut)) * sc, tt = t1 + t1, w = rcut - r.w, w2 = w * w;
+      float f[NR], df[NR], g[NR];
+      {
+        float Tb[NQ], Ub[NQ];
+        Tb[0] = Ub[0] = 1.f;
+        Tb[1] = t1;
+        Ub[1] = tt;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int t = base + h * LPN + q;
-        p[h] = p0 + t;
-        act[h] = t < np && OK(p[h], P.nb.n_pairs, 45);
-        r[h] = make_float4(1.f, 0.f, 0.f, 1.f);
-        zj[h] = 0;
-        if (act[h]) {
-          r[h] = P.nb.pr32[p[h]];
-          const int jj = P.nb.pj[p[h]];
-          if (OK(jj, P.nb.n_atoms, 47)) zj[h] = P.type[jj];
-          if (!OK(zj[h], T, 48)) zj[h] = 0;
+        for (int b = 2; b < NQ; ++b) {
+          Tb[b] = fmaf(tt, Tb[b - 1], -Tb[b - 2]);
+          Ub[b] = fmaf(tt, Ub[b - 1], -Ub[b - 2]);
         }
-      }
-      const u64 x = pack2(r[0].x, r[1].x), y = pack2(r[0].y, r[1].y), z = pack2(r[0].z, r[1].z), d2 = pack2(r[0].w, r[1].w);
-      // T_b and b U_(b-1) = T_b' of both distances, w = R_cut - r
-      const u64 t1 = mul2(add2(add2(d2, d2), pack2(-(rmin + rcut), -(rmin + rcut))), pack2(sc, sc)), tt = add2(t1, t1);
-      const u64 w = fma2(d2, pack2(-1.f, -1.f), pack2(rcut, rcut)), w2 = mul2(w, w);
-      const u64 dxw2 = mul2(pack2(2.f * sc, 2.f * sc), w2), mw = mul2(pack2(-2.f, -2.f), w);
-      u64 Tb[NQ], Ub[NQ];
-      Tb[0] = one2;
-      Tb[1] = t1;
-      Ub[0] = one2;
-      Ub[1] = tt;
-#pragma unroll
-      for (int b = 2; b < NQ; ++b) {
-        Tb[b] = fma2(tt, Tb[b - 1], Tb[b - 2] ^ 0x8000000080000000ull);
-        Ub[b] = fma2(tt, Ub[b - 1], Ub[b - 2] ^ 0x8000000080000000ull);
-      }
-#pragma unroll
-      for (int b = NQ - 1; b >= 1; --b) Ub[b] = mul2(pack2(static_cast<float>(b), static_cast<float>(b)), Ub[b - 1]);
-      if (ROWS) {
-#pragma unroll
-        for (int b = 0; b < NQ; ++b) {
-          float q0, q1;
-          unpack2(mul2(Tb[b], w2), q0, q1);
-          rstg[q * GS + 8 + b] = q0;
-          rstg[(LPN + q) * GS + 8 + b] = q1;
-        }
-      }
-      const float *c0 = czi + zj[0] * NR * NQ, *c1 = czi + zj[1] * NR * NQ;
-      u64 gx = 0, gy = 0, gz = 0, rad = 0;
-      horner_pass<NR, NU0>(gM, x, y, z, [&](auto Mu, u64 pv, u64 px, u64 py, u64 pz) {
-        constexpr int mu = decltype(Mu)::value;
-        // f_mu = w^2 sum c T_b, f_mu' = (dx/dr) w^2 sum c T_b' - 2 w sum c T_b
-        u64 F = pack2(c0[mu * NQ], c1[mu * NQ]), D = 0;
-#pragma unroll
-        for (int b = 1; b < NQ; ++b) {
-          const u64 cc = pack2(c0[mu * NQ + b], c1[mu * NQ + b]);
-          F = fma2(cc, Tb[b], F);
-          D = b == 1 ? mul2(cc, Ub[1]) : fma2(cc, Ub[b], D);
-        }
-        const u64 f = mul2(F, w2);
-        gx = fma2(f, px, gx);
-        gy = fma2(f, py, gy);
-        gz = fma2(f, pz, gz);
-        rad = fma2(pv, fma2(dxw2, D, mul2(mw, F)), rad);
         if (ROWS) {
-          float g0, g1;
-          unpack2(pv, g0, g1);
-          rstg[q * GS + mu] = g0;
-          rstg[(LPN + q) * GS + mu] = g1;
-        }
-      });
-      float rd[2];
-      unpack2(rad, rd[0], rd[1]);
-      const u64 s2 = pack2(rd[0] / r[0].w, rd[1] / r[1].w);
-      gx = fma2(s2, x, gx);
-      gy = fma2(s2, y, gy);
-      gz = fma2(s2, z, gz);
-      float g3[2][3];
-      unpack2(gx, g3[0][0], g3[1][0]);
-      unpack2(gy, g3[0][1], g3[1][1]);
-      unpack2(gz, g3[0][2], g3[1][2]);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (act[h] && Gout && OK(3 * p[h] + 2, 3 * P.nb.n_pairs, 53)) {
-          __stcs(Gout + 3 * p[h] + 0, g3[h][0]);
-          __stcs(Gout + 3 * p[h] + 1, g3[h][1]);
-          __stcs(Gout + 3 * p[h] + 2, g3[h][2]);
+          for (int b = 0; b < NQ; ++b) rstg[q * GS + 8 + b] = Tb[b] * w2;
         }
-        if (!act[h]) g3[h][0] = g3[h][1] = g3[h][2] = 0.f;   // a dummy pair adds nothing to the virial
-        if (ROWS) rstg[(h * LPN + q) * GS + 8 + NQ] = __int_as_float(zj[h]);
+#pragma unroll
+        for (int b = NQ - 1; b >= 1; --b) Ub[b] = static_cast<float>(b) * Ub[b - 1];
+        const float4* c4 = reinterpret_cast<const float4*>(czi + zj * NR * NQ);
+        static_assert(NQ == 8, "two 128-bit loads per radial function");
+#pragma unroll
+        for (int mu = 0; mu < NR; ++mu) {
+          const float4 ca = c4[2 * mu], cc = c4[2 * mu + 1];
+          const float c[NQ] = {ca.x, ca.y, ca.z, ca.w, cc.x, cc.y, cc.z, cc.w};
+          float F = c[0], D = c[1] * Ub[1];
+#pragma unroll
+          for (int b = 1; b < NQ; ++b) {
+            F = fmaf(c[b], Tb[b], F);
+            if (b > 1) D = fmaf(c[b], Ub[b], D);
+          }
+          f[mu] = F * w2;
+          df[mu] = fmaf(2.f * sc * w2, D, -2.f * w * F);
+          g[mu] = 0.f;
+        }
       }
-      const u64 n3[3] = {pack2(-g3[0][0], -g3[1][0]), pack2(-g3[0][1], -g3[1][1]), pack2(-g3[0][2], -g3[1][2])};
-      const u64 r3[3] = {x, y, z};
+      // powers of x, and a x^(a-1)
+      float X[NU0 + 1], DX[NU0 + 1];
+      X[0] = 1.f;
+      DX[0] = 0.f;
 #pragma unroll
-      for (int a2 = 0; a2 < 3; ++a2)
+      for (int a = 1; a <= NU0; ++a) {
+        X[a] = a == 1 ? r.x : X[a - 1] * r.x;
+        DX[a] = static_cast<float>(a) * X[a - 1];
+      }
+      u64 gx2 = 0, gy2 = 0, gz2 = 0;
+      slice_pass<NR, NU0>(gM, r.y, r.z, [&](auto Pp, u64 av, u64 ay, u64 az) {
+        constexpr int n = 2 * decltype(Pp)::value;
+        constexpr int m0 = Sl::T.mu[n], a0 = Sl::T.a[n], m1 = Sl::T.mu[n + 1], a1 = Sl::T.a[n + 1];
+        const float f0 = f[m0], f1 = m1 >= 0 ? f[m1 >= 0 ? m1 : 0] : 0.f;
+        const u64 fx = pack2(f0 * X[a0], f1 * X[a1]);
+        gx2 = fma2(pack2(f0 * DX[a0], f1 * DX[a1]), av, gx2);
+        if constexpr (Sl::T.deg[n] > 0) {
+          gy2 = fma2(fx, ay, gy2);
+          gz2 = fma2(fx, az, gz2);
+        }
+        float v0, v1;
+        unpack2(av, v0, v1);
+        g[m0] = fmaf(X[a0], v0, g[m0]);
+        if constexpr (m1 >= 0) g[m1] = fmaf(X[a1], v1, g[m1]);
+      });
+      float g3[3], hi;
+      unpack2(gx2, g3[0], hi);
+      g3[0] += hi;
+      unpack2(gy2, g3[1], hi);
+      g3[1] += hi;
+      unpack2(gz2, g3[2], hi);
+      g3[2] += hi;
+      float rad = 0.f;
 #pragma unroll
-        for (int b2 = 0; b2 < 3; ++b2) Wl[3 * a2 + b2] = fma2(n3[a2], r3[b2], Wl[3 * a2 + b2]);
+      for (int mu = 0; mu < NR; ++mu) {
+        rad = fmaf(g[mu], df[mu], rad);
+        if (ROWS) rstg[q * GS + mu] = g[mu];
+      }
+      if (ROWS) rstg[q * GS + 8 + NQ] = __int_as_float(zj);
+      const float s = rad / r.w;
+      const float r3[3] = {r.x, r.y, r.z};
+#pragma unroll
+      for (int a2 = 0; a2 < 3; ++a2) g3[a2] = fmaf(s, r3[a2], g3[a2]);
+      if (act) {
+        if (Gout && OK(3 * p + 2, 3 * P.nb.n_pairs, 53)) {
+          __stcs(Gout + 3 * p + 0, g3[0]);
+          __stcs(Gout + 3 * p + 1, g3[1]);
+          __stcs(Gout + 3 * p + 2, g3[2]);
+        }
+#pragma unroll
+        for (int a2 = 0; a2 < 3; ++a2)
+#pragma unroll
+          for (int b2 = 0; b2 < 3; ++b2) Wl[3 * a2 + b2] = fmaf(-g3[a2], r3[b2], Wl[3 * a2 + b2]);
+      }
       if (ROWS) {
         __syncwarp();
         // sum_j g_mu(j) Q_b(r_ij) per neighbor species: lane q takes b = q over the staged pairs
-        const int nbt = min(BATCH_A, np - base);
+        const int nbt = min(LPN, np - base);
         for (int t = 0; t < nbt; ++t) {
           const float* e = rstg + t * GS;
           const float qb = e[8 + q];
@@ -1087,17 +1119,13 @@ __global__ void __launch_bounds__(256, adj_blocks(NR)) k_adjoint(SplitArgs P) {
     // the neighborhood's virial (FP32 over its pairs, like its forces; sums over atoms are FP64)
     float Ws[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      float lo, hi;
-      unpack2(Wl[k], lo, hi);
-      Ws[k] = group_sum(lo + hi);
-    }
+    for (int k = 0; k < 9; ++k) Ws[k] = group_sum(Wl[k]);
     if (live && P.o.Wat && q == 0 && OK(9 * i + 8, 9 * P.nb.n_atoms, 50)) {
 #pragma unroll
       for (int k = 0; k < 9; ++k) P.o.Wat[9 * i + k] = static_cast<double>(Ws[k]);
     }
     if (ROWS && P.o.rows_hi) {
-      // the sums through shared memory (over the group's dV/dM, which is done with), then whole rows:
+      // the sums through shared memory (over the staging, which is done with), then whole rows:
       // block zi holds them; the other species' blocks and the padding past m are zero
       __syncwarp();
 #pragma unroll
@@ -1224,7 +1252,7 @@ int launch_split(SplitArgs P, int warps_pair, int nb_contract, int unroll, int s
   }
   // ---- pair adjoint ----
   if (efs || rows) {
-    const size_t gstride = static_cast<size_t>(adj_region(P.ldm, rows));
+    const size_t gstride = static_cast<size_t>(adj_region(Slices<NR, NU0>::FLOATS, rows));
     const size_t smem = P.c_bytes + static_cast<size_t>(warps_pair) * GPW * gstride * sizeof(float);
     auto go = [&](auto kern) {
       MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
@@ -1247,14 +1275,14 @@ std::vector<int> slot_table() {
   using Sh = Shape<NR, NU0>;
   constexpr auto S = make_slots<NR, NU0>();
   std::vector<int> t(S.comp, S.comp + Sh::NCOMP);
-  const std::vector<int> h = HornerOrder<NR, NU0>::of_slots();   // then slot -> Horner order
+  const std::vector<int> h = Slices<NR, NU0>::of_slots();   // then slot -> place among the slices
   t.insert(t.end(), h.begin(), h.end());
   return t;
 }
 
 }  // namespace
 
-// Uploads the slot -> component and slot -> Horner-order tables of the model's shape (at load time, so that the split
+// Uploads the slot -> component and slot -> slice-coefficient tables of the model's shape (at load time, so that the split
 // pass allocates nothing when it runs); leaves it empty for shapes without a split kernel.
 void split_prepare(mtp_model* m) {
   const DevSchedule& d = m->ds;
