@@ -12,9 +12,9 @@
 // own.  Back substitution goes by kBack rows, two launches each, with the diagonal blocks of U inverted
 // beforehand (all at once).
 //   What bounded it: three launches per column (1,955 at m = 651) and a thread per column of the
-// inverse walking m^2 dependent steps.  Now the panels (1.4 of 3.2 ms: a pivot chain of about 2 us
+// inverse walking m^2 dependent steps.  Now the panels (1.3 of 3.2 ms: a pivot chain of about 2 us
 // per column, and FP64 at 2 FMAs per clock in the one SM; pivots are compared as integers, FP64
-// comparisons alone took twice that) and 123 dependent launches.  A^-1 at m = 651: 45.3 -> 3.24 ms,
+// comparisons alone took twice that) and 123 dependent launches.  A^-1 at m = 651: 45.3 -> 3.18 ms,
 // m = 222: 6.3 -> 0.9, m = 1,636: 271 -> 18.5.
 // The grade product C = B A^-1 is fused with its row epilogue (max |C_ip| and the lowest p
 // attaining it), so C is never written.  This SIMT kernel serves small active sets and rows with
@@ -43,7 +43,7 @@ __global__ void k_maxabs(const double* A, int64_t n, unsigned long long* out) {
 
 constexpr int kPanel = 16;   // columns per panel (m = 651: 8 columns 3.31 ms, 16 3.24; m = 222: 0.56, 0.52)
 constexpr int kBack = 32;    // rows per step of the back substitution
-constexpr int kPanelThreads = 512;
+constexpr int kPanelRows = 2048;   // rows a panel's block holds in registers
 
 // what one panel's exchanges do to the other columns: row to[e] takes the old row from[e]; the
 // first kPanel entries are the panel's own rows
@@ -61,10 +61,10 @@ __global__ void k_lu_init(int* perm, int64_t m) {
 // panel in registers and their current positions (exchanges move positions, not data).  Writes the
 // panel's U and unit L blocks to M, the multipliers of the rows below to Lp[position][kPanel], the
 // exchanges to *mv and to perm (position -> row of A); a pivot below 1e-13 max|A| sets *flag.
-template <int R>
-__global__ void __launch_bounds__(kPanelThreads, 1) k_panel(double* M, int64_t m, int k0, int nb, double* Lp, PanelMoves* mv,
+template <int R, int NT>
+__global__ void __launch_bounds__(NT, 1) k_panel(double* M, int64_t m, int k0, int nb, double* Lp, PanelMoves* mv,
                                                             int* perm, const unsigned long long* maxabs, unsigned* flag) {
-  constexpr int NW = kPanelThreads / 32;
+  constexpr int NW = NT / 32;
   __shared__ long long s_v[2][NW];
   __shared__ int s_p[2][NW];
   __shared__ double s_row[2][kPanel];
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel(double* M, int64_t m
   int pos[R];
 #pragma unroll
   for (int q = 0; q < R; ++q) {
-    const int64_t r = k0 + tid + static_cast<int64_t>(q) * kPanelThreads;
+    const int64_t r = k0 + tid + static_cast<int64_t>(q) * NT;
     pos[q] = r < m ? static_cast<int>(r) : -1;
 #pragma unroll
     for (int c = 0; c < kPanel; ++c) a[q][c] = (r < m && c < nb) ? M[r * m + k0 + c] : 0.0;
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel(double* M, int64_t m
         s_inv[ph] = d != 0.0 ? 1.0 / d : 0.0;
 #pragma unroll
         for (int c = 0; c < kPanel; ++c) s_row[ph][c] = a[q][c];
-        s_src[j] = k0 + tid + q * kPanelThreads;
+        s_src[j] = k0 + tid + q * NT;
         s_from[j] = bp;
         if (!(fabs(d) > tiny)) atomicOr(flag, 1u);
       }
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel(double* M, int64_t m
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < R; ++q) {
-    const int r = k0 + tid + q * kPanelThreads;
+    const int r = k0 + tid + q * NT;
     if (pos[q] >= k0 + nb && pos[q] != r) {   // a row displaced from the panel's positions (or twice)
       const int e = atomicAdd(&s_n, 1);
       mv->to[e] = pos[q];
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_panel(double* M, int64_t m
 // The panel's exchanges in the other columns and the solve with its unit lower block, a thread per
 // column: M[panel rows][c] = L11^-1 (P M)[panel rows][c]; for the panel's own columns L11^-1 itself
 // goes to Tp (the other blocks still read the panel's block of M).
-__global__ void __launch_bounds__(32) k_swap_solve(double* M, int64_t m, int k0, int nb, const PanelMoves* mv, double* Tp) {
+__global__ void __launch_bounds__(128) k_swap_solve(double* M, int64_t m, int k0, int nb, const PanelMoves* mv, double* Tp) {
   __shared__ double L[kPanel][kPanel + 1];
   __shared__ PanelMoves s;
   for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
@@ -525,10 +525,11 @@ void invert_by_panels(double* M, double* W, double* D, double* Lp, double* Tp, P
   for (int k0 = 0; k0 < m; k0 += kPanel) {
     const int nb = static_cast<int>(std::min<int64_t>(kPanel, m - k0));
     const int64_t rows = m - k0;
-    auto panel = rows <= kPanelThreads ? k_panel<1> : (rows <= 2 * kPanelThreads ? k_panel<2> : k_panel<4>);
-    panel<<<1, kPanelThreads, 0, s>>>(M, m, k0, nb, Lp, mv, perm, maxabs, flag);
+    // a row per thread up to 1,024 rows (two rows in 512 threads: 51 us per panel at 651 rows), then four
+    auto panel = rows <= 512 ? k_panel<1, 512> : (rows <= 1024 ? k_panel<1, 1024> : k_panel<4, 512>);
+    panel<<<1, rows <= 512 || rows > 1024 ? 512 : 1024, 0, s>>>(M, m, k0, nb, Lp, mv, perm, maxabs, flag);
     ProfRegion::launched();
-    k_swap_solve<<<blocks(m, 32), 32, 0, s>>>(M, m, k0, nb, mv, Tp);
+    k_swap_solve<<<blocks(m, 128), 128, 0, s>>>(M, m, k0, nb, mv, Tp);
     ProfRegion::launched();
     const dim3 g(blocks(m, 32), std::max(1u, blocks(rows - nb, 32)));
     k_panel_update<<<g, 256, 0, s>>>(M, m, k0, nb, Lp, Tp);
@@ -599,7 +600,7 @@ void run_lu_inverse(mtp_model* md, const double* A, int64_t m, cudaStream_t s) {
   md->ainv_d.ensure(mm * sizeof(double), s);
   double* inv = md->ainv_d.as<double>();
   unsigned* flag_d = md->err_flag.as<unsigned>();
-  if (m <= 4 * kPanelThreads) invert_by_panels(M, W, D, Lp, Tp, mv, perm, m, maxabs, flag_d, inv, s);
+  if (m <= kPanelRows) invert_by_panels(M, W, D, Lp, Tp, mv, perm, m, maxabs, flag_d, inv, s);
   else invert_by_columns(M, perm, m, maxabs, flag_d, inv, s);
   // mixed-path copies: K-major padded split (tensor cores) and plain FP32 (SIMT)
   const int64_t ld = grade_tc_ld(m);

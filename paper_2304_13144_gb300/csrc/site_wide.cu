@@ -672,9 +672,12 @@ void launch_wide(const mtp_model* m, WideArgs P, int64_t max_part, int64_t* n_pa
   P.c_bytes = coef_bytes<R>(d);
   // ---- moments ----
   {
-    // pairs per monomial batch: 16 where eight warps' tables fit shared memory
+    // pairs per monomial batch: 16 where eight warps' tables fit shared memory; in FP32, which is
+    // bound by latency and not by its pipe, where two such blocks fit (level 16 tangent of 34,968
+    // atoms: 1.16 -> 0.72 ms; FP64 gains nothing at that size)
+    const size_t room = sizeof(R) == 4 ? kSmem / 2 : kSmem;
     P.pb = 16;
-    while (P.pb > 1 && P.c_bytes + WPB * moments_bytes<S>(d, P.n_mono, P.n_ab, P.pb) > kSmem) P.pb /= 2;
+    while (P.pb > 1 && P.c_bytes + WPB * moments_bytes<S>(d, P.n_mono, P.n_ab, P.pb) > room) P.pb /= 2;
     const size_t wb = moments_bytes<S>(d, P.n_mono, P.n_ab, P.pb);
     const int64_t tasks = (P.n_work + P.nbw - 1) / P.nbw;
     auto go = [&](auto kern) { launch_warps(kern, P, wb, tasks, 0, "wide_moments", s); };
