@@ -803,7 +803,6 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   nb->plan_rc = rc;
   nb->plan_cell = cell;
   nb->plan_pbc = pbc;
-  nb->plan_valid = true;
   }
   nb->n_atoms = N;
   DevCfg* d_cfg = nb->plan.as<DevCfg>();
@@ -918,6 +917,7 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   MTP_CUDA(cudaMemcpyAsync(const_cast<long long*>(h_total), nb->off.as<long long>() + N, sizeof(long long),
                            cudaMemcpyDeviceToHost, s));
   read_flag();
+  nb->plan_valid = true;   // (only now: the uploads above are done, so another stream may use them)
   const long long total = *h_total;
   if (flag & ERRF_SPECIES) throw Fail{MTP_ERR_ARG, "species outside [0, n_types)"};
   if (flag & ERRF_NONFINITE) throw Fail{MTP_ERR_NUMERIC, "non-finite position"};
