@@ -40,6 +40,24 @@ void DevBuf::ensure(size_t need, cudaStream_t s) {
   MTP_CUDA(cudaMallocAsync(&p, cap, s));
   bytes = cap;
 }
+bool DevBuf::try_ensure(size_t need, cudaStream_t s) {
+  if (need == 0) need = 16;
+  if (bytes >= need) return true;
+  if (take_injected(g_inject_alloc)) return false;
+  if (p) MTP_CUDA(cudaFreeAsync(p, s));
+  p = nullptr;
+  bytes = 0;
+  const size_t cap = need + need / 8;
+  const cudaError_t e = cudaMallocAsync(&p, cap, s);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    p = nullptr;
+    return false;
+  }
+  MTP_CUDA(e);
+  bytes = cap;
+  return true;
+}
 void DevBuf::release() {
   if (p) cudaFree(p);
   p = nullptr;
@@ -660,12 +678,13 @@ void check_model(const mtp_model* m) {
   if (dev != m->device) throw Fail{MTP_ERR_ARG, "model belongs to another device"};
 }
 
-// the workspace of the FP64 / dual-number pass, where the model has it
+// the workspace of the FP64 / dual-number pass, where the model has it; without the memory for it (a
+// value per moment and neighborhood, two in the tangent) the call runs on the generic kernel, which
+// has none
 void give_wide(mtp_model* m, int64_t n_work, bool fp64, bool tangent, SiteOutputs& o, cudaStream_t s) {
   const size_t bytes = wide_workspace(m, n_work, fp64, tangent);
   if (!bytes) return;
-  m->ws_wide.ensure(bytes, s);
-  o.wide = m->ws_wide.p;
+  if (m->ws_wide.try_ensure(bytes, s)) o.wide = m->ws_wide.p;
 }
 
 // Shared body of the EFS / grade / step entry points.
@@ -695,7 +714,6 @@ void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_prec
     m->ws_mom.ensure(std::max<int64_t>(N, 1) * split_ldm(m->ds.n_mom) * sizeof(float), s);
     o.mom = m->ws_mom.as<float>();
   }
-  if (fp64) give_wide(m, N, true, false, o, s);
   int64_t ld = 0;
   const bool use_tc = !fp64 && want_grade && grade_tc_available(m);
   if (want_grade) {
@@ -729,6 +747,7 @@ void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_prec
     row_atom = order;
     zrow = z;
   }
+  if (fp64) give_wide(m, N, true, false, o, s);   // (last: what the call cannot do without comes first)
   run_sites(m, b, nb, fp64, o, false, nullptr, s);
   if (want_efs) {
     if (forces) run_forces(nb, fp64, o.G, forces, s);
@@ -1492,8 +1511,9 @@ mtp_status mtp_train_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     if (fp64) {
       give_wide(md, N, true, false, o, s);
     } else if (split_wanted(md)) {
-      md->ws_mom.ensure(std::max<int64_t>(N, 1) * split_ldm(md->ds.n_mom) * sizeof(float), s);
-      o.mom = md->ws_mom.as<float>();
+      // (without the memory for it: the single kernel)
+      if (md->ws_mom.try_ensure(std::max<int64_t>(N, 1) * split_ldm(md->ds.n_mom) * sizeof(float), s))
+        o.mom = md->ws_mom.as<float>();
     }
     run_sites(md, b, nb, fp64, o, false, nullptr, s);
     run_forces(nb, fp64, o.G, F, s);

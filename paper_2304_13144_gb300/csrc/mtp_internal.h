@@ -41,6 +41,7 @@ struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
   void ensure(size_t need, cudaStream_t s);
+  bool try_ensure(size_t need, cudaStream_t s);   // false (and empty) where device memory does not suffice
   void release();
   template <class T> T* as() const { return static_cast<T*>(p); }
 };

@@ -62,3 +62,18 @@ def test_train_step_matches_oracle(native_lib, types, lev, prec):
     tol = 1e-10 if prec == "fp64" else 1e-5
     assert abs(loss.item() - L) <= tol * abs(L)
     assert rel(got.cpu().numpy(), grad) <= tol
+
+
+def test_without_memory_for_the_workspace_the_generic_kernel_answers(native_lib):
+    """Its moments cost a value per moment and neighborhood: a call that cannot have them still runs."""
+    from paper_2304_13144_gb300 import api
+    md, theta, bnp = setup(2, 12, 2, 97)
+    model = api.mtp_load(api.make_desc(2, 12), theta)
+    b = api.Batch(bnp)
+    nb = api.mtp_build_neighbors(model, b)
+    try:
+        api.mtp_debug_inject(api.MTP_FAULT_DEVICE_ALLOC, 1)
+        plain = api.mtp_param_rows(model, b, nb, "fp64").cpu().numpy()
+    finally:
+        api.mtp_debug_inject(api.MTP_FAULT_DEVICE_ALLOC, 0)
+    assert rel(plain, api.mtp_param_rows(model, b, nb, "fp64").cpu().numpy()) <= 1e-10
