@@ -14,7 +14,7 @@
 //   What bounded it: three launches per column (1,955 at m = 651) and a thread per column of the
 // inverse walking m^2 dependent steps.  Now the panels (1.3 of 3.2 ms: a pivot chain of about 2 us
 // per column, and FP64 at 2 FMAs per clock in the one SM; pivots are compared as integers, FP64
-// comparisons alone took twice that) and 123 dependent launches.  A^-1 at m = 651: 45.3 -> 3.18 ms,
+// comparisons alone took twice that) and 123 dependent launches.  A^-1 at m = 651: 44.2 -> 3.26 ms,
 // m = 222: 6.3 -> 0.9, m = 1,636: 271 -> 18.5.
 // The grade product C = B A^-1 is fused with its row epilogue (max |C_ip| and the lowest p
 // attaining it), so C is never written.  This SIMT kernel serves small active sets and rows with

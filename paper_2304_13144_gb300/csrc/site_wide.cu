@@ -22,7 +22,7 @@
 //   FP64 energies and forces, level 8, 256,000 atoms         17.3 -> 6.60
 //   the same, level 24, 16,384 atoms of the liquid           83.9 -> 14.7
 //   FP64 training step, level 16, 34,968 atoms (both passes) 34.6 -> 11.1
-//   FP32 tangent of the same step                            3.19 -> 1.82
+//   mixed training step of the same size (FP32 tangent)      3.58 -> 1.66
 // At level 20 the FP64 pipe would take 2.8 ms for the operations that remain.
 //
 // The order of every sum is fixed by the neighbor list, so the results do not depend on the launch
