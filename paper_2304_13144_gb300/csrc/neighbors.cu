@@ -232,10 +232,15 @@ constexpr int kWarpScan = 32;    // the warp fill and the reverse record: at mos
 constexpr int kMaskWords = 16;   // accepted-candidate bits per atom recorded by the count pass
 constexpr int kMaskBits = 32 * kMaskWords;
 
-// Count pass with a thread per atom (bin order), for lists large enough to fill the GPU that way.
+// Count pass with a thread per atom (bin order), for lists large enough to fill the GPU that way, and
+// (FILL) the fill pass of such lists in cells that scan more than 32 bins: it replays the count
+// pass's recorded decisions and forms only the accepted pairs again.  Rebuild of 1,048,576 atoms in
+// a cell one lattice constant thick (45 scanned bins): 5.1 ms, 8.7 with k_scan_warp; 65,536 atoms 0.70
+// and 0.64.
 // (at most 64 registers, 8 CTAs of 128 threads per SM: with the per-bin reverse record the
 // count pass measured 1.77 ms at 1M atoms against 1.91 ms at 48 registers / 10 CTAs and at
 // 80 registers / 6 CTAs; the warp-per-atom pass below measured 2.86 ms)
+template <bool FILL>
 __global__ void __launch_bounds__(128, 8) k_count(NbrArgs A) {
   // threads take the atoms in bin order, so that a warp's atoms scan the same or adjacent bins
   const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
@@ -246,6 +251,8 @@ __global__ void __launch_bounds__(128, 8) k_count(NbrArgs A) {
   const int bc = A.bcoord[i];
   const int b0 = bc & 1023, b1 = (bc >> 10) & 1023, b2 = (bc >> 20) & 1023;
   const float4 xi_h = A.ph[i], xi_l = A.pl[i];
+  long long out = FILL ? A.off[i] : 0;
+  const long long out_end = FILL ? A.off[i + 1] : 0;
   int count = 0;
   int cand = 0;          // candidate index in scan order (the self candidate included)
   uint32_t mword = 0;    // accepted bits of the current mask word
@@ -277,38 +284,63 @@ __global__ void __launch_bounds__(128, 8) k_count(NbrArgs A) {
         const long long s0 = A.bin_start[tb], s1 = A.bin_start[tb + 1];
         const unsigned before = static_cast<unsigned>(count);
         uint32_t slots = 0;   // accepted bits of this bin's first 32 slots
-        for (long long s = s0; s < s1; ++s, ++cand) {
+        // candidate s of this bin: 1 if (i -> j, n) is a pair (written out in the fill pass)
+        auto test = [&](long long s) -> int {
           const float4 xj_h = A.bph[s];
           const int j = __float_as_int(xj_h.w);
-          int acc = 0;
-          if (!(j == static_cast<int>(i) && n0 == 0 && n1 == 0 && n2 == 0)) {
-            float4 r;
-            int img;
-            acc = decide(A, C, i, j, xi_h, xi_l, xj_h, A.bpl[s], n0, n1, n2, r, img);
+          if (j == static_cast<int>(i) && n0 == 0 && n1 == 0 && n2 == 0) return 0;
+          float4 r;
+          int img;
+          if (!decide(A, C, i, j, xi_h, xi_l, xj_h, A.bpl[s], n0, n1, n2, r, img)) return 0;
+          if (FILL && out < out_end) {
+            A.pj[out] = j;
+            A.pimg[out] = img;
+            A.pr32[out] = r;
+            ++out;
           }
-          count += acc;
-          if (cand < kMaskBits) {
+          ++count;
+          return 1;
+        };
+        long long s = s0;
+        while (FILL && s < s1 && cand < kMaskBits) {
+          const int wb = cand & 31;
+          const int span = static_cast<int>(min(static_cast<long long>(32 - wb), s1 - s));
+          uint32_t word = A.mask[static_cast<long long>(cand >> 5) * A.n_atoms + t] >> wb;
+          if (span < 32) word &= (1u << span) - 1u;
+          while (word) {
+            const int bit = __ffs(word) - 1;
+            word &= word - 1u;
+            test(s + bit);
+          }
+          s += span;
+          cand += span;
+        }
+        for (; s < s1; ++s, ++cand) {
+          const int acc = test(s);
+          if (!FILL && cand < kMaskBits) {
             mword |= static_cast<uint32_t>(acc) << (cand & 31);
             if ((cand & 31) == 31) {
               A.mask[static_cast<long long>(cand >> 5) * A.n_atoms + t] = mword;
               mword = 0;
             }
           }
-          if (s - s0 < 32) slots |= static_cast<uint32_t>(acc) << (s - s0);
+          if (!FILL && s - s0 < 32) slots |= static_cast<uint32_t>(acc) << (s - s0);
         }
-        A.rv[static_cast<long long>(q) * A.n_atoms + t] = make_uint2(slots, before);
+        if (!FILL && A.rv) A.rv[static_cast<long long>(q) * A.n_atoms + t] = make_uint2(slots, before);
       }
     }
   }
-  if (cand < kMaskBits && (cand & 31) != 0) A.mask[static_cast<long long>(cand >> 5) * A.n_atoms + t] = mword;
-  A.cnt[i] = count;
+  if (!FILL && cand < kMaskBits && (cand & 31) != 0)
+    A.mask[static_cast<long long>(cand >> 5) * A.n_atoms + t] = mword;
+  if (!FILL) A.cnt[i] = count;
+  else if (count != out_end - A.off[i]) atomicOr(A.err, ERRF_CAPACITY);
 }
 
 // A warp per atom (bin order), any number of scanned bins: 32 bins at a time, a lane per bin (its
 // first binned atom, size and image), their candidates 32 at a time.  The count pass of small lists
-// (a thread per atom walks its few hundred candidates one after the other: 137 us for 108 atoms) and
-// of cells that scan more than 32 bins, whose fill pass it is too (candidates decided again, written
-// in scan order).  Same candidates, decisions and order as k_count.
+// (a thread per atom walks its few hundred candidates one after the other: 137 us for 108 atoms), and
+// the fill pass of those among them whose cells scan more than 32 bins (candidates decided again,
+// written in scan order).  Same candidates, decisions and order as k_count.
 template <bool FILL>
 __global__ void __launch_bounds__(128) k_scan_warp(NbrArgs A) {
   const unsigned full = 0xffffffffu;
@@ -860,9 +892,9 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   nb->masks.ensure(static_cast<size_t>(N) * kMaskWords * sizeof(uint32_t), s);
   A.mask = nb->masks.as<uint32_t>();
   // the replaying fill and the reverse record, when every configuration scans at most 32 bins; the
-  // count pass by threads there from kCountThreads atoms on
+  // count pass by threads from kCountThreads atoms on
   const bool warp_fill = max_scan <= kWarpScan;
-  const bool warp_count = !warp_fill || N < kCountThreads;
+  const bool warp_count = N < kCountThreads;
   A.rv = nullptr;
   if (warp_fill) {
     nb->segs.ensure(static_cast<size_t>(max_scan) * N * sizeof(uint2), s);
@@ -895,7 +927,7 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
       MTP_CUDA(cudaGetLastError());
     }
     if (warp_count) k_scan_warp<false><<<blocks_for(N * 32, 128), 128, 0, s>>>(A);
-    else k_count<<<blocks_for(N, 128), 128, 0, s>>>(A);
+    else k_count<false><<<blocks_for(N, 128), 128, 0, s>>>(A);
     ProfRegion::launched();
     MTP_CUDA(cudaGetLastError());
     if (small) {
@@ -943,7 +975,8 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
         else k_fill_warp<8><<<blocks_for(N * 32, 256), 256, 0, s>>>(A);
         ProfRegion::launched();
       } else {
-        k_scan_warp<true><<<blocks_for(N * 32, 128), 128, 0, s>>>(A);
+        if (warp_count) k_scan_warp<true><<<blocks_for(N * 32, 128), 128, 0, s>>>(A);
+        else k_count<true><<<blocks_for(N, 128), 128, 0, s>>>(A);
         ProfRegion::launched();
       }
       MTP_CUDA(cudaGetLastError());

@@ -33,7 +33,7 @@ def in_order(a):
 
 
 @pytest.mark.parametrize("reps,cut", [((16, 16, 16), 0), ((16, 16, 16), 1), ((16, 16, 17), 0), ((32, 32, 32), 1), ((32, 32, 32), 0),
-                                      ((1, 2, 7), 0), ((2, 2, 2), 3)])
+                                      ((1, 2, 7), 0), ((2, 2, 2), 3), ((1, 182, 182), 0)])
 def test_list_matches_oracle_around_the_rules(api, reps, cut):
     g = synth.rng(sum(reps) + cut)
     pos, cell, _ = synth.cubic_supercell(synth._BCC, 2.87, reps)
