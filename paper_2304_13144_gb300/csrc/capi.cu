@@ -63,6 +63,32 @@ void DevBuf::release() {
   p = nullptr;
   bytes = 0;
 }
+void* PinPool::take() {
+  {
+    std::lock_guard<std::mutex> lk(mu_);
+    if (!free_.empty()) {
+      void* p = free_.back();
+      free_.pop_back();
+      return p;
+    }
+  }
+  void* p = nullptr;
+  MTP_CUDA(cudaMallocHost(&p, kPinBytes));
+  return p;
+}
+void PinPool::give(void* p) noexcept {
+  {
+    std::lock_guard<std::mutex> lk(mu_);
+    if (free_.size() < kKept) {
+      free_.push_back(p);
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+PinPool::~PinPool() {
+  for (void* p : free_) cudaFreeHost(p);
+}
 
 namespace {
 
@@ -856,7 +882,7 @@ mtp_status mtp_load(const mtp_desc* desc, const double* theta, int64_t m, mtp_mo
       split_prepare(md);
       wide_prepare(md);
       noalloc_prepare(md->device);
-      MTP_CUDA(cudaMallocHost(&md->pin, kPinBytes));
+      { PinBlock warm(md->pins, 0); }   // (here, not in the first list build)
       md->async_err.ensure(sizeof(unsigned), 0);
       MTP_CUDA(cudaMemset(md->async_err.p, 0, sizeof(unsigned)));
       MTP_CUDA(cudaDeviceSynchronize());
@@ -878,9 +904,8 @@ void mtp_free_model(mtp_model* md) {
                     &md->ws_atom, &md->ws_rows, &md->ws_grade, &md->ws_sort, &md->ws_misc, &md->ws_red,
                     &md->err_flag, &md->async_err, &md->split_tab, &md->ws_mom, &md->wide_tab, &md->ws_wide})
     b->release();
-  if (md->pin) cudaFreeHost(md->pin);
-  cudaSetDevice(cur);
   delete md;
+  cudaSetDevice(cur);
 }
 
 int64_t mtp_num_params(const mtp_model* md) { return md ? md->sched.n_params : -1; }

@@ -7,6 +7,8 @@
 
 #include <cstdint>
 #include <cstring>
+#include <exception>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -190,6 +192,37 @@ inline __host__ __device__ int unpack_img(int v, int k) {
 // handles
 // ------------------------------------------------------------------------------------
 constexpr size_t kPinBytes = 16384;
+// pinned host memory for the read-backs of a list build, a block of kPinBytes per build in progress:
+// builds of different lists with one model may run in several threads at once, each with a block of
+// its own.  Blocks are kept for the next build (kKept at most) and freed with the model.
+class PinPool {
+ public:
+  PinPool() { free_.reserve(kKept); }
+  ~PinPool();
+  void* take();
+  void give(void* p) noexcept;
+
+ private:
+  static constexpr size_t kKept = 8;
+  std::mutex mu_;
+  std::vector<void*> free_;
+};
+// one build's block, for copies on one stream; the build waits for them itself unless it throws
+struct PinBlock {
+  PinBlock(PinPool& pool, cudaStream_t s) : p(pool.take()), pool(pool), s(s), thrown(std::uncaught_exceptions()) {}
+  ~PinBlock() {
+    if (std::uncaught_exceptions() > thrown) cudaStreamSynchronize(s);
+    pool.give(p);
+  }
+  PinBlock(const PinBlock&) = delete;
+  PinBlock& operator=(const PinBlock&) = delete;
+  void* const p;
+
+ private:
+  PinPool& pool;
+  cudaStream_t s;
+  int thrown;
+};
 }  // namespace mtp
 
 struct mtp_model {
@@ -217,7 +250,7 @@ struct mtp_model {
   mtp::DevBuf ws_misc;
   mtp::DevBuf ws_red;          // reductions
   mtp::DevBuf err_flag;        // unsigned
-  void* pin = nullptr;         // kPinBytes of pinned host memory for read-backs (mtp_load)
+  mtp::PinPool pins;           // pinned host memory of the list builds
   // errors of asynchronous kernels (bit 1: a bounded wait of the tensor-core grade expired),
   // allocated and zeroed by mtp_load, OR-ed by the kernels, read and cleared by mtp_sync
   mtp::DevBuf async_err;

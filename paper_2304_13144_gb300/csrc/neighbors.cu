@@ -721,11 +721,12 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   std::vector<int64_t> ao(n_cfg + 1);
   std::vector<double> cell(9 * static_cast<size_t>(n_cfg));
   std::vector<uint8_t> pbc(3 * static_cast<size_t>(n_cfg));
+  PinBlock pinned(m->pins, s);
   {
-    // through the model's pinned buffer where they fit (a copy into pageable memory waits by itself)
+    // through pinned memory where they fit (a copy into pageable memory waits by itself)
     const size_t n0 = ao.size() * sizeof(int64_t), n1 = cell.size() * sizeof(double), n2 = pbc.size();
     const bool pin = n0 + n1 + n2 <= kPinBytes;
-    char* h0 = pin ? static_cast<char*>(m->pin) : reinterpret_cast<char*>(ao.data());
+    char* h0 = pin ? static_cast<char*>(pinned.p) : reinterpret_cast<char*>(ao.data());
     char* h1 = pin ? h0 + n0 : reinterpret_cast<char*>(cell.data());
     char* h2 = pin ? h1 + n1 : reinterpret_cast<char*>(pbc.data());
     MTP_CUDA(cudaMemcpyAsync(h0, b->atom_offset, n0, cudaMemcpyDeviceToHost, s));
@@ -856,10 +857,10 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   int* d_batoms = d_bfill + (bins + 1);
   float4* d_bph = reinterpret_cast<float4*>((reinterpret_cast<uintptr_t>(d_batoms + N) + 15) & ~uintptr_t(15));
   float4* d_bpl = d_bph + N;
-  nb->counts.ensure((N + 1) * sizeof(long long), s);
+  nb->counts.ensure((N + 2) * sizeof(long long), s);   // N + 1 counts, then the error flag
+  unsigned* const d_err = reinterpret_cast<unsigned*>(nb->counts.as<long long>() + N + 1);
   nb->off.ensure((N + 1) * sizeof(long long), s);
-  m->err_flag.ensure(sizeof(unsigned), s);
-  MTP_CUDA(cudaMemsetAsync(m->err_flag.p, 0, sizeof(unsigned), s));
+  MTP_CUDA(cudaMemsetAsync(d_err, 0, sizeof(unsigned), s));
   MTP_CUDA(cudaMemsetAsync(d_bcount, 0, 2 * (bins + 1) * sizeof(int), s));   // counts and fill counters
   const bool small = N <= kSmallAtoms && bins <= kSmallBins;
   if (!small) MTP_CUDA(cudaMemsetAsync(nb->counts.as<long long>() + N, 0, sizeof(long long), s));
@@ -888,7 +889,7 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   A.bpl = d_bpl;
   A.cnt = nb->counts.as<long long>();
   A.off = nb->off.as<long long>();
-  A.err = m->err_flag.as<unsigned>();
+  A.err = d_err;
   nb->masks.ensure(static_cast<size_t>(N) * kMaskWords * sizeof(uint32_t), s);
   A.mask = nb->masks.as<uint32_t>();
   // the replaying fill and the reverse record, when every configuration scans at most 32 bins; the
@@ -938,11 +939,11 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
       scan_exclusive<long long>(nb->counts.as<long long>(), nb->off.as<long long>(), N + 1, nb->scratch, s);
     }
   }
-  volatile long long* h_total = static_cast<long long*>(m->pin);
-  volatile unsigned* h_flag = reinterpret_cast<unsigned*>(static_cast<char*>(m->pin) + 16);
+  volatile long long* h_total = static_cast<long long*>(pinned.p);
+  volatile unsigned* h_flag = reinterpret_cast<unsigned*>(static_cast<char*>(pinned.p) + 16);
   unsigned flag = 0;
   auto read_flag = [&] {
-    MTP_CUDA(cudaMemcpyAsync(const_cast<unsigned*>(h_flag), m->err_flag.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+    MTP_CUDA(cudaMemcpyAsync(const_cast<unsigned*>(h_flag), d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
     MTP_CUDA(cudaStreamSynchronize(s));
     flag = *h_flag;
   };
@@ -992,7 +993,7 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
     if (flag & ERRF_GEOMETRY) throw Fail{MTP_ERR_GEOMETRY, "coincident atoms (|r_ij| < 1e-8 A)"};
     if (!(flag & ERRF_CAPACITY)) break;
     if (attempt == 1) throw Fail{MTP_ERR_CAPACITY, "neighbor fill overflowed its counted capacity twice"};
-    MTP_CUDA(cudaMemsetAsync(m->err_flag.p, 0, sizeof(unsigned), s));
+    MTP_CUDA(cudaMemsetAsync(d_err, 0, sizeof(unsigned), s));
   }
   if ((flag & ERRF_REVPEND) && !(flag & ERRF_REVERSE)) {
     // atoms past slot 31 of their bin: their pairs' reverses by search

@@ -1,0 +1,71 @@
+"""Neighbor lists of different batches built at once, in several threads and streams, with one model."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2304_13144_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+BUILDS = 40
+
+
+def test_lists_built_at_once_with_one_model(native_lib):
+    """Each thread rebuilds its own list for cells of its own size, and of another size and back, so
+    that offsets, cells and pair counts differ between the builds in flight; every list must be the one
+    that a build alone gives.  One thread's positions are not finite: only its builds fail."""
+    from paper_2304_13144_gb300 import api
+    model = api.mtp_load(api.make_desc(1, 4), np.zeros(api.mtp_describe(api.make_desc(1, 4))["n_params"]))
+    g = synth.rng(77)
+
+    def batch(n, sigma=0.1):
+        pos, cell, _ = synth.cubic_supercell(synth._FCC, 3.6, n)
+        return api.Batch(synth.single(pos + g.normal(0, sigma, pos.shape), np.zeros(len(pos), int), cell))
+
+    work = [[batch(2), batch(3)], [batch(5), batch(4)], [batch(12), batch(9)], [batch(3), batch(14)]]
+    bad = batch(4)
+    bad.pos[7, 1] = float("nan")
+    ref = [[api.mtp_nbr_export(api.mtp_build_neighbors(model, b), b) for b in w] for w in work]
+    torch.cuda.synchronize()
+    errors, got = [], [[None, None] for _ in work]
+    start = threading.Barrier(len(work) + 1)
+
+    def build(t):
+        try:
+            s = torch.cuda.Stream()
+            lists = [None, None]
+            start.wait()
+            for k in range(BUILDS):
+                for e, b in enumerate(work[t]):
+                    lists[e] = api.mtp_build_neighbors(model, b, lists[e], stream=s)
+                    n, pairs = lists[e].size()
+                    assert n == b.n_atoms and pairs == ref[t][e]["j"].numel()
+            got[t] = lists
+        except Exception as e:   # reported by the test below
+            errors.append(f"thread {t}: {e!r}")
+
+    def fail():
+        s = torch.cuda.Stream()
+        start.wait()
+        for k in range(BUILDS):
+            try:
+                api.mtp_build_neighbors(model, bad, stream=s)
+                errors.append("non-finite positions accepted")
+            except api.MtpError as e:
+                if e.name != "MTP_ERR_NUMERIC":
+                    errors.append(repr(e))
+
+    threads = [threading.Thread(target=build, args=(t,)) for t in range(len(work))] + [threading.Thread(target=fail)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
+    for t, w in enumerate(work):
+        for e, b in enumerate(w):
+            ex = api.mtp_nbr_export(got[t][e], b)
+            for k in ("off", "j", "img", "r"):
+                assert torch.equal(ex[k], ref[t][e][k]), (t, e, k)
