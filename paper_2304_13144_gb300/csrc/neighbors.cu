@@ -488,16 +488,18 @@ __global__ void __launch_bounds__(1024, 1) k_bin_small(NbrArgs A, int n_bins) {
   }
 }
 
-// off = exclusive sums of the counts (off[n] = their total), by one block
+// off = exclusive sums of the counts (off[n] = their total), by one block.  In 64 bits throughout: a
+// few hundred atoms of a cell much smaller than the cut-off have more than 2^31 pairs, which the
+// build refuses by this total.
 __global__ void __launch_bounds__(1024, 1) k_offsets_small(const long long* cnt, long long* off, int n) {
-  __shared__ int warp_sum[32];
+  __shared__ long long warp_sum[32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int per = (n + 1023) / 1024, b0 = min(n, tid * per), b1 = min(n, b0 + per);
-  int mine = 0;
-  for (int k = b0; k < b1; ++k) mine += static_cast<int>(cnt[k]);
-  int incl = mine;
+  long long mine = 0;
+  for (int k = b0; k < b1; ++k) mine += cnt[k];
+  long long incl = mine;
   for (int m = 1; m < 32; m <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, m);
+    const long long v = __shfl_up_sync(0xffffffffu, incl, m);
     if (lane >= m) incl += v;
   }
   if (lane == 31) warp_sum[w] = incl;

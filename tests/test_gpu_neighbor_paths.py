@@ -63,3 +63,17 @@ def test_reused_list_follows_cells_offsets_and_periodicity(api):
         new, ex2 = listed(api, api.mtp_build_neighbors(m, b), b)
         np.testing.assert_array_equal(got, new)
         np.testing.assert_array_equal(ex["r"], ex2["r"])
+
+
+def test_more_pairs_than_an_index_holds_are_refused(api):
+    """256 atoms of a cell of 256 A^3 with a cut-off of 130 A have 2.4e9 pairs (9.2 million each);
+    with 7,936 atoms beyond each other's reach the list is one of the largest that one block sums."""
+    desc = api.make_desc(1, 4, r_cut=130.0)
+    m = api.mtp_load(desc, np.zeros(api.mtp_describe(desc)["n_params"]))
+    dense = np.stack(np.meshgrid(np.arange(8), np.arange(8), np.arange(4), indexing="ij"), -1).reshape(-1, 3) * 1.0
+    far = np.stack(np.meshgrid(*[np.arange(20)] * 3, indexing="ij"), -1).reshape(-1, 3)[:7936] * 131.0
+    bnp = synth.concat([synth.single(dense, np.zeros(256, int), np.diag([8.0, 8.0, 4.0])),
+                        synth.single(far, np.zeros(7936, int), 2620.0 * np.eye(3), (0, 0, 0))])
+    with pytest.raises(api.MtpError) as e:
+        api.mtp_build_neighbors(m, api.Batch(bnp))
+    assert e.value.name == "MTP_ERR_UNSUPPORTED" and "pairs" in str(e.value)
