@@ -12,7 +12,8 @@
 // per center.  An image can lie in the sphere only if its fractional coordinate relative to the
 // center is within radius / face distance on every axis, so each axis gets its interval of images
 // from an FP32 fractional coordinate with a margin, and only the images in all three intervals
-// (of most atoms none) are tested in FP64.  32 centers among 16,000 atoms, radius 8 A
+// (of most atoms none) are tested in FP64.  (Where the margin would reach a quarter of a cell, an
+// atom some 10^5 cells away, the FP64 coordinate's nearest image gives the interval.)  32 centers among 16,000 atoms, radius 8 A
 // (one call for the sizes, one for the clusters: three passes): 677 -> 0.21 ms.
 #include <cuda_runtime.h>
 
@@ -146,8 +147,9 @@ __global__ void __launch_bounds__(kCutThreads) k_cut(CutArgs A) {
         // -- images n with |f + n| <= reach
         const float l = ceilf(-f - reach[a] - eps), u = floorf(-f + reach[a] + eps);
         int n_lo, n_hi;
-        if (capped || !(fabsf(l) < 1e9f) || !(fabsf(u) < 1e9f)) {
-          // thin cells, whose images are cut off at kMaxImages around the nearest one
+        if (capped || !(eps < 0.25f)) {
+          // thin cells, whose images are cut off at kMaxImages around the nearest one; atoms so far
+          // from their center that the margin would let in whole layers of images
           const double fd = (xj[0] - xc[0]) * s_G[3 * a] + (xj[1] - xc[1]) * s_G[3 * a + 1] + (xj[2] - xc[2]) * s_G[3 * a + 2];
           const int sn = static_cast<int>(rint(fd));
           n_lo = -s_K[a] - sn;

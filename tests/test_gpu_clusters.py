@@ -98,3 +98,20 @@ def test_cut_skewed_cells_and_split_ranges(api, reps, n_centers, radius):
     bnp = synth.single(pos + g.normal(0, 0.05, pos.shape), g.integers(0, 3, len(pos)), cell)
     centers = g.integers(0, len(pos), n_centers)
     check_against_oracle(api.mtp_cut_clusters(api.Batch(bnp), torch.tensor(centers), radius), bnp, centers, radius)
+
+
+@pytest.mark.parametrize("cells", [1 << 10, 1 << 17, 1 << 18, 1 << 27])
+def test_cut_of_atoms_far_outside_their_cell(api, cells):
+    """Positions of a run that never wraps them: atoms moved by whole cells (exact in FP64) give the
+    clusters of the wrapped ones, bit for bit, on both sides of the distance from which the nearest
+    image is found in FP64."""
+    g = synth.rng(72)
+    pos = np.round(g.uniform(0, 8, (12, 3)) * 4096) / 4096
+    near = synth.single(pos, g.integers(0, 2, 12), 8.0 * np.eye(3))
+    far = dict(near, pos=pos + 8.0 * cells * g.integers(-1, 2, (12, 3)))
+    centers = torch.arange(12)
+    want = api.mtp_cut_clusters(api.Batch(near), centers, 7.0)
+    got = api.mtp_cut_clusters(api.Batch(far), centers, 7.0)
+    assert len(want["src"]) > 12 * 20
+    for k in ("off", "pos", "type", "src"):
+        assert torch.equal(got[k], want[k]), k
