@@ -242,7 +242,9 @@ mtp_status mtp_get_active_set(const mtp_model* model, double* A, void* stream);
  *   source   DEVICE [m] int64 out, or NULL: -1 for a kept active row, else the index in B of
  *            the candidate now in its place
  *   n_swaps  HOST out, or NULL: swaps made
- * Requires mtp_set_active_set; MTP_ERR_SINGULAR if the final A cannot be factorised. */
+ * Requires mtp_set_active_set; MTP_ERR_SINGULAR if the final A cannot be factorised,
+ * MTP_ERR_TIMEOUT if a bounded wait of the update expired.  The swaps work in place: a call that
+ * fails once they have begun leaves the model without an active set, until mtp_set_active_set. */
 mtp_status mtp_maxvol(mtp_model* model, const double* B, int64_t n, double eps, int64_t max_swaps,
                       int64_t* source, int64_t* n_swaps, void* stream);
 
@@ -385,8 +387,15 @@ mtp_status mtp_restore(const void* buffer, int64_t size, mtp_model** model, void
  * tensor-core grade launches a single try, so the first wait not already satisfied expires and
  * the kernel takes its abort path (stops, drains its own copies and MMAs with the default
  * bound, frees tensor memory, leaves the unfinished gamma NaN; mtp_sync then returns
- * MTP_ERR_TIMEOUT).  count = 0 disarms.  Process-wide. */
-enum { MTP_FAULT_DEVICE_ALLOC = 1, MTP_FAULT_NEIGHBOR_OVERFLOW = 2, MTP_FAULT_GRADE_WAIT = 3 };
+ * MTP_ERR_TIMEOUT); MTP_FAULT_MAXVOL_WAIT lets the barriers of the next `count` MaxVol updates
+ * wait, briefly, for a block that never arrives (mtp_maxvol returns MTP_ERR_TIMEOUT and the model
+ * has no active set).  count = 0 disarms.  Process-wide. */
+enum {
+  MTP_FAULT_DEVICE_ALLOC = 1,
+  MTP_FAULT_NEIGHBOR_OVERFLOW = 2,
+  MTP_FAULT_GRADE_WAIT = 3,
+  MTP_FAULT_MAXVOL_WAIT = 4
+};
 mtp_status mtp_debug_inject(int fault, int count);
 
 /* Synchronise `stream` and report errors that asynchronous kernels of this model latched on

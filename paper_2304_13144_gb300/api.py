@@ -576,6 +576,7 @@ def mtp_restore(blob: bytes, stream=None) -> Model:
 MTP_FAULT_DEVICE_ALLOC = 1
 MTP_FAULT_NEIGHBOR_OVERFLOW = 2
 MTP_FAULT_GRADE_WAIT = 3
+MTP_FAULT_MAXVOL_WAIT = 4
 
 
 def mtp_debug_inject(fault, count):

@@ -21,6 +21,7 @@ void set_error(const std::string& msg) { g_last_error = msg; }
 std::atomic<int> g_inject_alloc{0};
 std::atomic<int> g_inject_overflow{0};
 std::atomic<int> g_inject_grade_wait{0};
+std::atomic<int> g_inject_maxvol_wait{0};
 
 bool take_injected(std::atomic<int>& c) {
   int v = c.load();
@@ -1188,6 +1189,7 @@ mtp_status mtp_debug_inject(int fault, int count) {
     if (fault == MTP_FAULT_DEVICE_ALLOC) g_inject_alloc = count;
     else if (fault == MTP_FAULT_NEIGHBOR_OVERFLOW) g_inject_overflow = count;
     else if (fault == MTP_FAULT_GRADE_WAIT) g_inject_grade_wait = count;
+    else if (fault == MTP_FAULT_MAXVOL_WAIT) g_inject_maxvol_wait = count;
     else throw Fail{MTP_ERR_ARG, "unknown fault"};
   });
 }

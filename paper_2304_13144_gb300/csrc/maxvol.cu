@@ -108,27 +108,32 @@ struct SwapArgs {
   double limit;         // 1 + eps
   long long max_swaps;  // in all
   long long last;       // this launch returns at the latest after this many swaps in all
+  int tries;            // of a barrier before it gives up
+  unsigned absent;      // blocks that a barrier waits for and that never come (fault injection)
   double *u, *v, *w;
   Best* part;           // [gridDim.x]
   long long* source;    // [m]
   SwapState* st;
 };
 
+constexpr int kBarrierTries = 4000000;
+
 // all blocks of a cooperative launch (arrivals count up from the launch's zero; release and acquire
 // at the counter order the blocks' writes); bounded: after about a second it gives up
-__device__ bool grid_barrier(SwapState* st, unsigned& round) {
+__device__ bool grid_barrier(const SwapArgs& P, unsigned& round) {
   __shared__ int s_ok;
   __syncthreads();
   ++round;
   if (threadIdx.x == 0) {
     int ok = 1;
-    const unsigned target = round * gridDim.x;
+    SwapState* const st = P.st;
+    const unsigned target = round * gridDim.x + P.absent;
     unsigned seen;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->arrived) : "memory");
     for (int tries = 0;; ++tries) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&st->arrived) : "memory");
       if (seen >= target) break;
-      if (tries > 4000000) {
+      if (tries > P.tries) {
         atomicExch(&st->timeout, 1u);
         ok = 0;
         break;
@@ -164,7 +169,7 @@ __global__ void __launch_bounds__(1024, 1) k_swaps(SwapArgs P) {
     }
     publish(b);
   }
-  if (!grid_barrier(P.st, round)) return;
+  if (!grid_barrier(P, round)) return;
   while (true) {
     Best b = kNone;
     for (int k = threadIdx.x; k < static_cast<int>(gridDim.x); k += blockDim.x)
@@ -190,7 +195,7 @@ __global__ void __launch_bounds__(1024, 1) k_swaps(SwapArgs P) {
       if (t < P.n) __stcg(P.v + t, __ldcg(P.C + t * m + j));
     }
     if (tid == 0) P.source[j] = i;
-    if (!grid_barrier(P.st, round)) return;
+    if (!grid_barrier(P, round)) return;
     // C -= v u (and the largest entry of the result), A^-1 -= w u
     Best nb = kNone;
     int64_t r = r0;
@@ -213,7 +218,7 @@ __global__ void __launch_bounds__(1024, 1) k_swaps(SwapArgs P) {
     }
     publish(nb);
     ++swaps;
-    if (!grid_barrier(P.st, round)) return;
+    if (!grid_barrier(P, round)) return;
   }
 }
 
@@ -249,26 +254,34 @@ int64_t run_maxvol(mtp_model* md, const double* B, int64_t n, double eps, int64_
     }
     MTP_CUDA(cudaMemsetAsync(st, 0, sizeof(SwapState), s));
     SwapArgs P{C, md->ainv_d.as<double>(), B, md->a_d.as<double>(), n, static_cast<int>(m), 1.0 + eps, max_swaps, 0,
-               u, v, w, part, src, st};
+               kBarrierTries, 0u, u, v, w, part, src, st};
+    if (take_injected(g_inject_maxvol_wait)) { P.tries = 1000; P.absent = 1u; }
+    // the swaps change A and A^-1 in place: until the inverse of the final A is there the model has
+    // no active set, whichever way this call ends
+    md->have_ainv = false;
     const int64_t want = (std::max<int64_t>(n * m, m * m) + 1023) / 1024;
     const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(want, nsm)));
     while (swaps < max_swaps) {
       MTP_CUDA(cudaMemsetAsync(&st->arrived, 0, sizeof(unsigned), s));
-      P.last = swaps + 4096;   // a launch ends after about 30 ms at the latest
+      P.last = swaps + 4096;   // swaps of one launch: about 45 ms at 2,000 x 222 entries
       void* args[] = {&P};
       MTP_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_swaps), dim3(grid), dim3(1024), args, 0, s));
       ProfRegion::launched();
       SwapState h{};
       MTP_CUDA(cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s));
       MTP_CUDA(cudaStreamSynchronize(s));
-      if (h.timeout) throw Fail{MTP_ERR_TIMEOUT, "a bounded wait of the MaxVol update expired"};
+      if (h.timeout) throw Fail{MTP_ERR_TIMEOUT, "a bounded wait of the MaxVol update expired; the model has no active set now"};
       swaps = h.swaps;
       if (h.stop) break;
     }
   }
   if (source) MTP_CUDA(cudaMemcpyAsync(source, src, m * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
-  if (swaps > 0) run_lu_inverse(md, md->a_d.as<double>(), m, s);
-  else MTP_CUDA(cudaStreamSynchronize(s));
+  if (swaps > 0) {
+    run_lu_inverse(md, md->a_d.as<double>(), m, s);
+  } else {
+    MTP_CUDA(cudaStreamSynchronize(s));
+    md->have_ainv = true;   // nothing was changed
+  }
   return swaps;
 }
 

@@ -374,6 +374,7 @@ int64_t run_cut_clusters(const mtp_batch* b, const int64_t* centers, int64_t n, 
 extern std::atomic<int> g_inject_alloc;
 extern std::atomic<int> g_inject_overflow;
 extern std::atomic<int> g_inject_grade_wait;
+extern std::atomic<int> g_inject_maxvol_wait;
 bool take_injected(std::atomic<int>& c);
 // Warps per group of the grouped contraction (site_group.cu), by how many groups' arrays fit an SM:
 // 16 at level 16 and below (a warp each), 6 at level 20, 1 at level 24.  Measured, ms per pass:

@@ -135,3 +135,34 @@ def test_maxvol_fewer_and_more_candidates_than_parameters(api, n, max_swaps):
     assert ns == ns_ref and 0 < ns <= max_swaps
     np.testing.assert_array_equal(src.cpu().numpy(), src_ref)
     np.testing.assert_array_equal(api.mtp_get_active_set(model).cpu().numpy(), A_ref)
+
+
+@pytest.mark.parametrize("n", [3, 700])
+def test_expired_maxvol_barrier_leaves_no_active_set(api, n):
+    """The swaps change A and A^-1 in place: when a barrier of theirs gives up, nothing may go on with
+    what is left of them (few and many blocks)."""
+    desc = api.make_desc(2, 2, 24)
+    m = api.mtp_describe(desc)["n_params"]
+    model = api.mtp_load(desc, np.zeros(m))
+    A0 = torch.tensor(synth.diag_dominant(24, m))
+    B = torch.tensor(synth.rng(25).normal(size=(n, m)) * A0.abs().max().item())
+    api.mtp_set_active_set(model, A0.cuda())
+    try:
+        api.mtp_debug_inject(api.MTP_FAULT_MAXVOL_WAIT, 1)
+        with pytest.raises(api.MtpError) as e:
+            api.mtp_maxvol(model, B)
+    finally:
+        api.mtp_debug_inject(api.MTP_FAULT_MAXVOL_WAIT, 0)
+    assert e.value.name == "MTP_ERR_TIMEOUT"
+    b = api.Batch(synth.fcc_unary_108(seed=26))
+    nb = api.mtp_build_neighbors(model, b)
+    for call in (lambda: api.mtp_get_active_set(model), lambda: api.mtp_get_active_inverse(model),
+                 lambda: api.mtp_grade(model, b, nb, "fp64"), lambda: api.mtp_maxvol(model, B)):
+        with pytest.raises(api.MtpError) as e:
+            call()
+        assert "no active set" in str(e.value)
+    api.mtp_set_active_set(model, A0.cuda())
+    src, swaps = api.mtp_maxvol(model, B)
+    A_ref, src_ref, swaps_ref = AS.maxvol(A0.numpy(), B.numpy(), 1e-3, 1_000_000)
+    assert swaps == swaps_ref
+    np.testing.assert_array_equal(api.mtp_get_active_set(model).cpu().numpy(), A_ref)
