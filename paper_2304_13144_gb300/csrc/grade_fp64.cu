@@ -261,7 +261,9 @@ __global__ void __launch_bounds__(FTHREADS, 1) k_grade_fp64(const __grid_constan
     const int quarter = warp & 3;            // tensor-memory lane quarter of this warp
     const int half = (warp - 2) >> 2;        // columns 32 half .. of the tile
     uint32_t acc_it = 0;
-    for (int64_t w = blockIdx.x; w < a.n_work && !*abort_flag; w += gridDim.x) {
+    // (an abort ends the walk at the next wait, by lane 0 for the whole warp: lanes that read the flag
+    // themselves could leave a warp whose others wait for them)
+    for (int64_t w = blockIdx.x; w < a.n_work; w += gridDim.x) {
       const int64_t tile = w / a.n_col;
       const int col0 = static_cast<int>(w - tile * a.n_col) * FN + half * EN;
       double c[EN];

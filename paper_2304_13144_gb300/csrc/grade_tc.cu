@@ -211,7 +211,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_grade_tc(const __grid_constant__
   } else {
     const int q = warp & 3;   // TMEM lane quarter accessible to this warp
     uint32_t acc_it = 0;
-    for (int64_t w = blockIdx.x; w < a.n_work && !*abort_flag; w += gridDim.x) {
+    // (an abort ends the walk at the next wait, by lane 0 for the whole warp: lanes that read the flag
+    // themselves could leave a warp whose others wait for them)
+    for (int64_t w = blockIdx.x; w < a.n_work; w += gridDim.x) {
       const int64_t tile = w / a.n_pass;
       const int pass = static_cast<int>(w - tile * a.n_pass);
       float best = -1.f;
