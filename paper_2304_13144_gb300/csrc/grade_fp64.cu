@@ -439,7 +439,8 @@ void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, do
     a.pbest = pbest;
     a.parg = parg;
     a.err = md->async_err.as<unsigned>();
-    a.wait_limit = WAIT_LIMIT;
+    // host-side fault injection: a single try per wait makes the first unsatisfied wait expire
+    a.wait_limit = take_injected(g_inject_grade_wait) ? 1u : WAIT_LIMIT;
     const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(a.n_work, nsm)));
     k_grade_fp64<<<grid, FTHREADS, FSMEM, s>>>(mA, mB, a);
     ProfRegion::launched();
