@@ -641,7 +641,7 @@ void upload_theta(mtp_model* md) {
 }
 
 void run_grade_simt(mtp_model* md, int64_t N, bool fp64, const double* rows, const float* rows_f, int64_t ld,
-                    double* gamma, int32_t* argmax, const unsigned char* only, cudaStream_t s);
+                    double* gamma, int32_t* argmax, cudaStream_t s);
 void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, double* gamma, int32_t* argmax, cudaStream_t s);
 bool grade_tc_available(const mtp_model* md);
 void run_grade_tc(mtp_model* md, int64_t N, const float* hi, const float* lo, int64_t ld, double* gamma,
@@ -783,7 +783,7 @@ void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_prec
   if (want_grade) {
     if (use_tc) run_grade_tc(m, N, o.rows_hi, o.rows_lo, ld, gamma, argmax, zrow, row_atom, s);
     else if (fp64) run_grade_fp64(m, N, o.rows, ld, gamma, argmax, s);
-    else run_grade_simt(m, N, false, nullptr, o.rows_hi, ld, gamma, argmax, nullptr, s);
+    else run_grade_simt(m, N, false, nullptr, o.rows_hi, ld, gamma, argmax, s);
     if (flagged || n_flagged) {
       int64_t* cnt = n_flagged;
       int32_t* fl = flagged;

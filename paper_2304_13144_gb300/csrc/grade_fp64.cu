@@ -13,8 +13,8 @@
 // digits are at most 2^12, so a sum of K of them over up to 4096 / K slice pairs is an integer below
 // 2^24, exact in FP32; such groups of pairs with equal s + t share an accumulator (12 of them at
 // m = 651, in two sweeps over K).  The epilogue adds the accumulators as 64-bit integers and rounds to
-// FP64 once or twice, so the result is closer to the exact sum than an FP64 accumulation.  Rows of B that hold an infinity or
-// NaN go to the SIMT kernel.
+// FP64 once or twice, so the result is closer to the exact sum than an FP64 accumulation.  Rows of B
+// that hold an infinity or NaN are graded by plain FP64 sums instead, each for itself.
 //
 // One persistent CTA per SM as in grade_tc.cu: warp 0 TMA producer (all 18 slices of a 64-wide K
 // chunk, one stage of 216 KB, 128B swizzle), warp 1 tcgen05.mma issuer (M 128, N 64, K 16), warps 2-9
@@ -30,7 +30,7 @@
 namespace mtp {
 
 void run_grade_simt(mtp_model* md, int64_t N, bool fp64, const double* rows, const float* rows_f, int64_t ld,
-                    double* gamma, int32_t* argmax, const unsigned char* only, cudaStream_t s);
+                    double* gamma, int32_t* argmax, cudaStream_t s);
 
 namespace {
 
@@ -100,7 +100,7 @@ __global__ void k_slice_x(const double* X, int64_t m, const int* g, const int* f
 }
 
 // slices of the rows r0 .. r0 + n - 1 of B: out[s][r][k] (np rows per slice), their exponents, and
-// bad[r / 64] where one of 64 rows is not finite.  A warp per row.
+// bad[r] where a row is not finite.  A warp per row.
 __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ B, int64_t ldb, int64_t m, int64_t n, const int* g, int kp,
                                                     int64_t np, uint16_t* out, int* E, unsigned char* bad) {
   const int64_t r = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ B
   if (e < -3000 || nonfinite) e = 0;
   if (lane == 0) {
     E[r] = e;
-    if (nonfinite) bad[r / 64] = 1;
+    if (nonfinite) bad[r] = 1;
   }
   for (int k = 2 * lane; k < kp; k += 64) {   // two digits of a slice per store
     uint16_t d0[NS], d1[NS];
@@ -340,6 +340,49 @@ __global__ void k_combine_fp64(int64_t N, int n_best, const double* pbest, const
   if (argmax) argmax[r] = arg;
 }
 
+// Marked rows by plain FP64 sums over k (the arithmetic, order and comparisons of the SIMT kernel): a
+// block per 32 rows, a thread per column of a row at a time.  Bound by FP64 (2 FMAs per clock and SM),
+// so a row costs a block 0.1 ms at m = 651 where the SIMT kernel's tile of 64 rows takes 7.
+constexpr int kRedoRows = 32;
+__global__ void __launch_bounds__(256) k_redo_rows(const double* __restrict__ B, int64_t ldb, const double* __restrict__ X, int64_t m,
+                                                   int64_t N, const unsigned char* bad, double* gamma, int32_t* argmax) {
+  __shared__ double s_v[8];
+  __shared__ int s_p[8];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t r0 = blockIdx.x * static_cast<int64_t>(kRedoRows);
+  unsigned marked = __ballot_sync(0xffffffffu, r0 + lane < N && bad[r0 + lane] != 0);   // the same in every warp
+  while (marked) {
+    const int64_t r = r0 + __ffs(marked) - 1;
+    marked &= marked - 1;
+    const double* b = B + r * ldb;
+    double best = -1.0;
+    int arg = 0;
+    for (int64_t p = threadIdx.x; p < m; p += 256) {
+      double acc = 0.0;
+#pragma unroll 8
+      for (int64_t k = 0; k < m; ++k) acc = fma(b[k], X[k * m + p], acc);
+      const double v = fabs(acc);
+      if (v > best) { best = v; arg = static_cast<int>(p); }
+    }
+    auto take = [&](double v, int p) {
+      if (v > best || (v == best && p < arg)) { best = v; arg = p; }
+    };
+    for (int o = 16; o; o >>= 1) {
+      const double v = __shfl_xor_sync(0xffffffffu, best, o);
+      const int p = __shfl_xor_sync(0xffffffffu, arg, o);
+      take(v, p);
+    }
+    if (lane == 0) { s_v[w] = best; s_p[w] = arg; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int u = 1; u < 8; ++u) take(s_v[u], s_p[u]);
+      gamma[r] = best;
+      if (argmax) argmax[r] = arg;
+    }
+    __syncthreads();
+  }
+}
+
 CUtensorMap slice_map(const uint16_t* base, int64_t rows, int64_t kp, int box_rows) {
   CUtensorMap t;
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(kp), static_cast<cuuint64_t>(rows)};
@@ -397,7 +440,7 @@ void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, do
   const int64_t m = md->m_active;
   if (N == 0) return;
   if (!grade_fp64_sliced(m)) {
-    run_grade_simt(md, N, true, rows, nullptr, ld, gamma, argmax, nullptr, s);
+    run_grade_simt(md, N, true, rows, nullptr, ld, gamma, argmax, s);
     return;
   }
   const XPlan x = x_plan(m, md->ainv_s.p);
@@ -405,7 +448,7 @@ void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, do
   const int n_col = x.pp / FN, n_best = x.pp / EN;
   const size_t b_sl = static_cast<size_t>(NS) * np * x.kp * sizeof(uint16_t), b_e = (np * sizeof(int) + 255) & ~size_t(255),
                b_best = static_cast<size_t>(n_best) * cn * sizeof(double), b_arg = static_cast<size_t>(n_best) * cn * sizeof(int32_t),
-               b_bad = static_cast<size_t>((N + 63) / 64);
+               b_bad = static_cast<size_t>(N);
   md->ws_grade.ensure(b_sl + b_e + b_best + b_arg + b_bad + 256, s);
   char* base = md->ws_grade.as<char>();
   uint16_t* sl = reinterpret_cast<uint16_t*>(base);
@@ -422,7 +465,7 @@ void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, do
   ProfRegion pr("grade_fp64", s);
   for (int64_t r0 = 0; r0 < N; r0 += cn) {
     const int64_t n = std::min<int64_t>(cn, N - r0);
-    k_slice_rows<<<nblk(n * 32, 256), 256, 0, s>>>(rows + r0 * ld, ld, m, n, x.g, x.kp, np, sl, E, bad + r0 / 64);
+    k_slice_rows<<<nblk(n * 32, 256), 256, 0, s>>>(rows + r0 * ld, ld, m, n, x.g, x.kp, np, sl, E, bad + r0);
     ProfRegion::launched();
     // partials start as NaN: a tile that does not run (a bounded wait expired) leaves gamma NaN
     MTP_CUDA(cudaMemsetAsync(pbest, 0xFF, static_cast<size_t>(n_best) * n * sizeof(double), s));
@@ -448,8 +491,9 @@ void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, do
     ProfRegion::launched();
     MTP_CUDA(cudaGetLastError());
   }
-  // tiles of 64 rows that hold an infinity or NaN, again with the SIMT kernel
-  run_grade_simt(md, N, true, rows, nullptr, ld, gamma, argmax, bad, s);
+  k_redo_rows<<<nblk(N, kRedoRows), 256, 0, s>>>(rows, ld, md->ainv_d.as<double>(), m, N, bad, gamma, argmax);
+  ProfRegion::launched();
+  MTP_CUDA(cudaGetLastError());
 }
 
 }  // namespace mtp

@@ -17,9 +17,8 @@
 // comparisons alone took twice that) and 123 dependent launches.  A^-1 at m = 651: 44.2 -> 3.26 ms,
 // m = 222: 6.3 -> 0.9, m = 1,636: 271 -> 18.5.
 // The grade product C = B A^-1 is fused with its row epilogue (max |C_ip| and the lowest p
-// attaining it), so C is never written.  This SIMT kernel serves small active sets and rows with
-// infinities or NaN; the mixed path uses the tensor-core kernel in grade_tc.cu, the FP64 path the
-// one in grade_fp64.cu.
+// attaining it), so C is never written.  This SIMT kernel serves small active sets; the mixed path
+// uses the tensor-core kernel in grade_tc.cu, the FP64 path the one in grade_fp64.cu.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -443,8 +442,7 @@ __global__ void k_split_ainv(const double* X, int64_t m, int64_t ld, float* hi, 
 // K steps of 16; each thread owns a 4 x 4 micro-tile.
 template <class T>
 __global__ void __launch_bounds__(256) k_grade_simt(const T* B, int64_t ldb, const T* X, int64_t m, int64_t N,
-                                                     double* gamma, int32_t* argmax, const unsigned char* only) {
-  if (only && !only[blockIdx.x]) return;   // only the marked tiles of 64 rows
+                                                     double* gamma, int32_t* argmax) {
   __shared__ T sB[16][64 + 1];
   __shared__ T sX[16][64 + 1];
   __shared__ double rowmax[64];
@@ -622,17 +620,17 @@ void run_lu_inverse(mtp_model* md, const double* A, int64_t m, cudaStream_t s) {
 }
 
 void run_grade_simt(mtp_model* md, int64_t N, bool fp64, const double* rows, const float* rows_f, int64_t ld,
-                    double* gamma, int32_t* argmax, const unsigned char* only, cudaStream_t s) {
+                    double* gamma, int32_t* argmax, cudaStream_t s) {
   const int64_t m = md->m_active;
   const unsigned g = static_cast<unsigned>((N + 63) / 64);
   if (N == 0) return;
   ProfRegion pr(fp64 ? "grade_simt_fp64" : "grade_simt_fp32", s);
   if (fp64) {
-    k_grade_simt<double><<<g, 256, 0, s>>>(rows, ld, md->ainv_d.as<double>(), m, N, gamma, argmax, only);
+    k_grade_simt<double><<<g, 256, 0, s>>>(rows, ld, md->ainv_d.as<double>(), m, N, gamma, argmax);
     ProfRegion::launched();
   } else {
     k_grade_simt<float><<<g, 256, 0, s>>>(rows_f, ld, md->ainv_f.as<float>() + 2 * md->ainv_ld * md->ainv_ld, m, N,
-                                               gamma, argmax, only);
+                                               gamma, argmax);
     ProfRegion::launched();
   }
   MTP_CUDA(cudaGetLastError());

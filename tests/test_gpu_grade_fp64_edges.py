@@ -49,3 +49,49 @@ def test_expired_waits_take_the_abort_path(api):
     again = api.mtp_grade(model, b, nb, "fp64")["gamma"]
     api.mtp_sync(model)
     assert torch.equal(again, ref)
+
+
+def expected(rows, X):
+    """gamma by the comparisons of the library: the largest |C|, a NaN column never the largest (-1 where
+    every column is NaN)."""
+    with np.errstate(all="ignore"):
+        C = np.abs(rows @ X)
+    return np.where(np.isnan(C), -1.0, C).max(1)
+
+
+def check(gamma, ref, rel):
+    plain = np.isfinite(ref) & (ref >= 0)
+    np.testing.assert_array_equal(gamma[~plain], ref[~plain])
+    np.testing.assert_allclose(gamma[plain], ref[plain], rtol=rel)
+
+
+def test_overflowing_rows_leave_the_others_alone(api):
+    """Radial coefficients of one species pair so large that the products of moments overflow: the rows
+    of atoms with such a neighbor hold infinities, the others grade as if there were none."""
+    types, lev, n = 2, 12, 5
+    md = O.OracleModel(types, lev, 2.0, 5.0)
+    nu_sum = [sum(nu for _, nu in labs) for labs, _ in md.basis]
+    theta = synth.draw_theta(5, types, md.n_rad, 8, nu_sum, [len(labs) for labs, _ in md.basis], 2.0, 5.0, 42.0)
+    big = theta.copy()
+    n_c = types * types * md.n_rad * 8
+    c = big[-n_c:].reshape(types, types, -1)
+    c[0, 1] *= 1e200
+    g = synth.rng(31)
+    pos, cell, _ = synth.cubic_supercell(synth._FCC, 3.6, n)
+    z = np.zeros(len(pos), int)
+    z[[3, 250, 499]] = 1
+    b = api.Batch(synth.single(pos + g.normal(0, 0.1, pos.shape), z, cell))
+    A = torch.tensor(synth.diag_dominant(6, md.m), device="cuda")
+    gam, rows = [], []
+    for th in (theta, big):
+        model = api.mtp_load(api.make_desc(types, lev), th)
+        nb = api.mtp_build_neighbors(model, b)
+        api.mtp_set_active_set(model, A)
+        gam.append(api.mtp_grade(model, b, nb, "fp64")["gamma"].cpu().numpy())
+        rows.append(api.mtp_param_rows(model, b, nb, "fp64").cpu().numpy())
+        X = api.mtp_get_active_inverse(model).cpu().numpy()
+    over = ~np.isfinite(rows[1]).all(1)
+    same = (rows[0] == rows[1]).all(1)
+    assert 50 < over.sum() < 300 and 200 < same.sum() < 450 and len(pos) % 64
+    np.testing.assert_array_equal(gam[1][same], gam[0][same])
+    check(gam[1][over], expected(rows[1][over], X), 1e-12)
