@@ -14,7 +14,8 @@
 // 2^24, exact in FP32; such groups of pairs with equal s + t share an accumulator (12 of them at
 // m = 651, in two sweeps over K).  The epilogue adds the accumulators as 64-bit integers and rounds to
 // FP64 once or twice, so the result is closer to the exact sum than an FP64 accumulation.  Rows of B
-// that hold an infinity or NaN are graded by plain FP64 sums instead, each for itself.
+// that hold an infinity or NaN are graded by plain FP64 sums instead, each for itself, and so are all
+// rows where X holds one.
 //
 // One persistent CTA per SM as in grade_tc.cu: warp 0 TMA producer (all 18 slices of a 64-wide K
 // chunk, one stage of 216 KB, 128B swizzle), warp 1 tcgen05.mma issuer (M 128, N 64, K 16), warps 2-9
@@ -68,13 +69,19 @@ __device__ __forceinline__ void digits_of(double v, int shift, uint16_t (&d)[NS]
   d[0] = static_cast<uint16_t>(__float_as_uint(static_cast<float>(f)) >> 16);
 }
 
-__global__ void k_x_row_scale(const double* X, int64_t m, int* g, int* f) {   // a warp per row k
+// a warp per row k; *xbad (starts 0) = 1 where X has an infinity or NaN (an inverse can overflow: its
+// pivots are judged against max |A|)
+__global__ void k_x_row_scale(const double* X, int64_t m, int* g, int* f, int* xbad) {
   const int64_t k = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
   if (k >= m) return;
   int e = -4000;
   for (int64_t p = threadIdx.x & 31; p < m; p += 32) e = max(e, exponent_of(X[k * m + p]));
   e = __reduce_max_sync(0xffffffffu, e);
-  if ((threadIdx.x & 31) == 0) { g[k] = e < -3000 ? 0 : e; f[k] = -4000; }
+  if ((threadIdx.x & 31) == 0) {
+    g[k] = e < -3000 ? 0 : e;
+    f[k] = -4000;
+    if (e > 1024) *xbad = 1;   // exponent field 0x7ff
+  }
 }
 
 __global__ void k_x_col_scale(const double* X, int64_t m, const int* g, int* f) {   // f starts very low
@@ -100,15 +107,15 @@ __global__ void k_slice_x(const double* X, int64_t m, const int* g, const int* f
 }
 
 // slices of the rows r0 .. r0 + n - 1 of B: out[s][r][k] (np rows per slice), their exponents, and
-// bad[r] where a row is not finite.  A warp per row.
-__global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ B, int64_t ldb, int64_t m, int64_t n, const int* g, int kp,
-                                                    int64_t np, uint16_t* out, int* E, unsigned char* bad) {
+// bad[r] where a row is not finite (every row where X is not).  A warp per row.
+__global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ B, int64_t ldb, int64_t m, int64_t n, const int* g, const int* xbad,
+                                                    int kp, int64_t np, uint16_t* out, int* E, unsigned char* bad) {
   const int64_t r = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
   if (r >= n) return;
   const int lane = threadIdx.x & 31;
   const double* b = B + r * ldb;
   int e = -4000;
-  bool nonfinite = false;
+  bool nonfinite = *xbad != 0;
   for (int64_t k = lane; k < m; k += 32) {
     const double v = b[k];
     nonfinite |= ((__double_as_longlong(v) >> 52) & 0x7ff) == 0x7ff;
@@ -401,7 +408,7 @@ unsigned nblk(int64_t n, int t) { return static_cast<unsigned>((n + t - 1) / t);
 struct XPlan {
   int kp, pp;
   size_t bytes;
-  int *g, *f;
+  int *g, *f, *xbad;
   uint16_t* slices;
 };
 
@@ -409,10 +416,11 @@ XPlan x_plan(int64_t m, void* base) {
   XPlan x;
   x.kp = static_cast<int>((m + FK - 1) / FK * FK);
   x.pp = static_cast<int>((m + FN - 1) / FN * FN);
-  const size_t head = (2 * static_cast<size_t>(m) * sizeof(int) + 255) & ~size_t(255);
+  const size_t head = ((2 * static_cast<size_t>(m) + 1) * sizeof(int) + 255) & ~size_t(255);
   x.bytes = head + static_cast<size_t>(NS) * x.pp * x.kp * sizeof(uint16_t);
   x.g = static_cast<int*>(base);
   x.f = x.g + m;
+  x.xbad = x.f + m;
   x.slices = reinterpret_cast<uint16_t*>(static_cast<char*>(base) + head);
   return x;
 }
@@ -427,7 +435,8 @@ void slice_active_inverse(mtp_model* md, int64_t m, cudaStream_t s) {
   md->ainv_s.ensure(x_plan(m, nullptr).bytes, s);
   const XPlan x = x_plan(m, md->ainv_s.p);
   const double* X = md->ainv_d.as<double>();
-  k_x_row_scale<<<nblk(m * 32, 256), 256, 0, s>>>(X, m, x.g, x.f);
+  MTP_CUDA(cudaMemsetAsync(x.xbad, 0, sizeof(int), s));
+  k_x_row_scale<<<nblk(m * 32, 256), 256, 0, s>>>(X, m, x.g, x.f, x.xbad);
   ProfRegion::launched();
   k_x_col_scale<<<dim3(nblk(m, 32), 16), 256, 0, s>>>(X, m, x.g, x.f);
   ProfRegion::launched();
@@ -465,7 +474,7 @@ void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, do
   ProfRegion pr("grade_fp64", s);
   for (int64_t r0 = 0; r0 < N; r0 += cn) {
     const int64_t n = std::min<int64_t>(cn, N - r0);
-    k_slice_rows<<<nblk(n * 32, 256), 256, 0, s>>>(rows + r0 * ld, ld, m, n, x.g, x.kp, np, sl, E, bad + r0);
+    k_slice_rows<<<nblk(n * 32, 256), 256, 0, s>>>(rows + r0 * ld, ld, m, n, x.g, x.xbad, x.kp, np, sl, E, bad + r0);
     ProfRegion::launched();
     // partials start as NaN: a tile that does not run (a bounded wait expired) leaves gamma NaN
     MTP_CUDA(cudaMemsetAsync(pbest, 0xFF, static_cast<size_t>(n_best) * n * sizeof(double), s));

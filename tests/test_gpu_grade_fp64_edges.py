@@ -95,3 +95,22 @@ def test_overflowing_rows_leave_the_others_alone(api):
     assert 50 < over.sum() < 300 and 200 < same.sum() < 450 and len(pos) % 64
     np.testing.assert_array_equal(gam[1][same], gam[0][same])
     check(gam[1][over], expected(rows[1][over], X), 1e-12)
+
+
+def test_inverse_that_overflows(api):
+    """A set whose every pivot is fine against max |A| and whose inverse has entries past 2^1024: the
+    grades are those of plain sums over that inverse, infinities and NaN columns included."""
+    model, b, nb = setup(api)
+    m = model.n_params
+    A = 2.0 ** -970 * (np.eye(m) - 2.0 ** 30 * np.eye(m, k=1))
+    api.mtp_set_active_set(model, torch.tensor(A, device="cuda"))
+    X = api.mtp_get_active_inverse(model).cpu().numpy()
+    assert np.isfinite(X).any() and not np.isfinite(X).all()
+    rows = api.mtp_param_rows(model, b, nb, "fp64").cpu().numpy()
+    assert np.isfinite(rows).all()
+    check(api.mtp_grade(model, b, nb, "fp64")["gamma"].cpu().numpy(), expected(rows, X), 1e-12)
+    # and a set with a finite inverse again
+    A = synth.diag_dominant(6, m)
+    api.mtp_set_active_set(model, torch.tensor(A, device="cuda"))
+    X = api.mtp_get_active_inverse(model).cpu().numpy()
+    check(api.mtp_grade(model, b, nb, "fp64")["gamma"].cpu().numpy(), expected(rows, X), 1e-11)
