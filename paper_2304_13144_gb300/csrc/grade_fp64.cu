@@ -10,12 +10,20 @@
 //   largest entry, 10 more than the factors have),
 //   C_ip = 2^(E_i + f_p) sum_{s + t < 9} 2^(-12 - 7 (s + t)) sum_k d_s,ik d'_t,kp.
 // The inner sums run as tcgen05.mma kind::f16 with FP32 accumulation in tensor memory: products of
-// digits are at most 2^12, so a sum of K of them over up to 4096 / K slice pairs is an integer below
+// digits are at most 2^12, so a sum of K of them over up to 4096 / K slice pairs is an integer of at most
 // 2^24, exact in FP32; such groups of pairs with equal s + t share an accumulator (12 of them at
 // m = 651, in two sweeps over K).  The epilogue adds the accumulators as 64-bit integers and rounds to
-// FP64 once or twice, so the result is closer to the exact sum than an FP64 accumulation.  Rows of B
-// that hold an infinity or NaN are graded by plain FP64 sums instead, each for itself, and so are all
-// rows where X holds one.
+// FP64 once per sweep.
+//
+// Precision.  The sums are exact; what is lost is the fixed point of the operands (an entry more than
+// 2^10 below the largest of its scaled row or column keeps fewer than its 53 bits) and the slice pairs
+// with s + t >= 9: at most 1.3 2^-60 2^(E_i + f_p) per term.  FP64 accumulation loses up to
+// 2^-53 sum_k |b_k X_kp| in each of its m steps, which is more as long as that sum is at least
+// 2^(E_i + f_p - 6), the largest product or a 64th of it.  k_check_fp64 bounds it from below for the column
+// that wins, by the leading digits; a row where it is not shown (large terms that cancel exactly beside
+// a column of small ones) is redone by plain FP64 sums, like the rows that hold an infinity or NaN and
+// all rows where X holds one.  (Host emulation, 21 sets of cond 1 to 1e18, levels 8 to 20: 2 of 17,544
+// rows redone; the sums are 3 to 500 times the limit.)
 //
 // One persistent CTA per SM as in grade_tc.cu: warp 0 TMA producer (all 18 slices of a 64-wide K
 // chunk, one stage of 216 KB, 128B swizzle), warp 1 tcgen05.mma issuer (M 128, N 64, K 16), warps 2-9
@@ -330,8 +338,9 @@ __global__ void __launch_bounds__(FTHREADS, 1) k_grade_fp64(const __grid_constan
   }
 }
 
-// gamma and argmax of the chunk's rows from the column tiles' maxima (in column order, strict '>')
-__global__ void k_combine_fp64(int64_t N, int n_best, const double* pbest, const int32_t* parg, const int* E, double* gamma,
+// gamma and argmax of the chunk's rows from the column tiles' maxima (in column order, strict '>');
+// the argmax also over parg's first plane
+__global__ void k_combine_fp64(int64_t N, int n_best, const double* pbest, int32_t* parg, const int* E, double* gamma,
                                int32_t* argmax) {
   const int64_t r = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (r >= N) return;
@@ -344,7 +353,33 @@ __global__ void k_combine_fp64(int64_t N, int n_best, const double* pbest, const
     if (v > best) { best = v; arg = parg[p * N + r]; }
   }
   gamma[r] = nan ? __longlong_as_double(0x7ff8000000000000LL) : scalbn(best, E[r]);
+  parg[r] = arg;
   if (argmax) argmax[r] = arg;
+}
+
+// bad[r] where sum_k |b_k X_kp| of the winning column is not shown to be at least 2^(E + f - 6): with the
+// leading digits d, d' of the scaled entries (|entry| >= (|d| - 1/2) / 64 where d is not 0) it is at least
+// 2^(E + f) sum (2 |d| - 1)(2 |d'| - 1) / 2^14.  A warp per row; rows of slice 0 only, so 2 x 2 kp bytes.
+// (Unfinished rows, gamma NaN, stay.)
+__global__ void __launch_bounds__(256) k_check_fp64(int64_t N, int kp, const uint16_t* __restrict__ sl, const uint16_t* __restrict__ xs,
+                                                    const int32_t* arg, const double* gamma, unsigned char* bad) {
+  const int64_t r = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
+  if (r >= N) return;
+  const int lane = threadIdx.x & 31;
+  const uint32_t* a = reinterpret_cast<const uint32_t*>(sl + r * kp);
+  const uint32_t* x = reinterpret_cast<const uint32_t*>(xs + static_cast<int64_t>(arg[r]) * kp);
+  auto weight = [](uint32_t bf16_bits) {
+    const float d = fabsf(__uint_as_float(bf16_bits << 16));
+    return d > 0.f ? d + d - 1.f : 0.f;
+  };
+  float sum = 0.f;
+  for (int k = lane; k < kp / 2; k += 32) {
+    const uint32_t u = a[k], v = x[k];
+    sum = fmaf(weight(u & 0xffffu), weight(v & 0xffffu), sum);
+    sum = fmaf(weight(u >> 16), weight(v >> 16), sum);
+  }
+  for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0 && !(sum >= 256.f) && gamma[r] == gamma[r]) bad[r] = 1;
 }
 
 // Marked rows by plain FP64 sums over k (the arithmetic, order and comparisons of the SIMT kernel): a
@@ -497,6 +532,8 @@ void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, do
     k_grade_fp64<<<grid, FTHREADS, FSMEM, s>>>(mA, mB, a);
     ProfRegion::launched();
     k_combine_fp64<<<nblk(n, 256), 256, 0, s>>>(n, n_best, pbest, parg, E, gamma + r0, argmax ? argmax + r0 : nullptr);
+    ProfRegion::launched();
+    k_check_fp64<<<nblk(n * 32, 256), 256, 0, s>>>(n, x.kp, sl, x.slices, parg, gamma + r0, bad + r0);
     ProfRegion::launched();
     MTP_CUDA(cudaGetLastError());
   }

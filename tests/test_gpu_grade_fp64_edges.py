@@ -114,3 +114,37 @@ def test_inverse_that_overflows(api):
     api.mtp_set_active_set(model, torch.tensor(A, device="cuda"))
     X = api.mtp_get_active_inverse(model).cpu().numpy()
     check(api.mtp_grade(model, b, nb, "fp64")["gamma"].cpu().numpy(), expected(rows, X), 1e-11)
+
+
+@pytest.mark.parametrize("types,lev", [(2, 12), (3, 20)])
+def test_winning_column_of_small_terms_beside_cancelling_large_ones(api, types, lev):
+    """An inverse made for one atom's row b: its two largest terms, in two columns of their own, cancel
+    to 2^-36, and every other column holds one product 2^-30 as large.  gamma is such a product, and must
+    be as close to it as FP64 sums are bound to be: m 2^-53 sum_k |b_k X_kp| of its column."""
+    model, b, nb = setup(api, types, lev)
+    m = model.n_params
+    rows = api.mtp_param_rows(model, b, nb, "fp64").cpu().numpy()
+    atom = 17
+    row = rows[atom]
+    k1, k2 = np.argsort(-np.abs(row))[:2]
+    g = synth.rng(9)
+    top = abs(row[k1])
+    X = np.diag(2.0 ** -30 * top * g.uniform(0.5, 1.0, m) / np.maximum(np.abs(row), 2.0 ** -6 * top))
+    q, d = row[k1] / row[k2], 2.0 ** -36
+    X[k1, k1] = X[k1, k2] = 1.0
+    X[k2, k1], X[k2, k2] = -q * (1 + d), -q * (1 - d)
+    A = np.diag(1.0 / np.diag(X))
+    det = 2 * d * q
+    A[np.ix_([k1, k2], [k1, k2])] = np.array([[X[k2, k2], -1.0], [-X[k2, k1], 1.0]]) / det
+    api.mtp_set_active_set(model, torch.tensor(A, device="cuda"))
+    X = api.mtp_get_active_inverse(model).cpu().numpy().astype(np.longdouble)
+    out = api.mtp_grade(model, b, nb, "fp64")
+    C = np.abs((row.astype(np.longdouble)[:, None] * X).sum(0))
+    p = int(C.argmax())
+    assert p not in (k1, k2)
+    bound = m * 2.0 ** -53 * (np.abs(row) * np.abs(X[:, p])).sum()
+    assert abs(out["gamma"][atom].item() - C[p]) <= bound
+    # the other rows: within the bound of their largest products
+    C = np.abs(np.stack([(r[:, None] * X).sum(0) for r in rows.astype(np.longdouble)])).max(1)
+    tol = 2.0 ** -52 * C + m * 2.0 ** -53 * (np.abs(rows) * np.abs(X).max(1)).max(1)
+    assert (np.abs(out["gamma"].cpu().numpy() - C) <= tol).all()
