@@ -389,12 +389,16 @@ mtp_status mtp_restore(const void* buffer, int64_t size, mtp_model** model, void
  * bound, frees tensor memory, leaves the unfinished gamma NaN; mtp_sync then returns
  * MTP_ERR_TIMEOUT); MTP_FAULT_MAXVOL_WAIT lets the barriers of the next `count` MaxVol updates
  * wait, briefly, for a block that never arrives (mtp_maxvol returns MTP_ERR_TIMEOUT and the model
- * has no active set).  count = 0 disarms.  Process-wide. */
+ * has no active set); MTP_FAULT_ALLOC_SKIP lets the next `count` growths succeed before an armed
+ * MTP_FAULT_DEVICE_ALLOC takes effect.  A growth that a call can do without (the workspaces of the
+ * faster of two passes) makes it take the other pass instead of failing.  count = 0 disarms.
+ * Process-wide. */
 enum {
   MTP_FAULT_DEVICE_ALLOC = 1,
   MTP_FAULT_NEIGHBOR_OVERFLOW = 2,
   MTP_FAULT_GRADE_WAIT = 3,
-  MTP_FAULT_MAXVOL_WAIT = 4
+  MTP_FAULT_MAXVOL_WAIT = 4,
+  MTP_FAULT_ALLOC_SKIP = 5
 };
 mtp_status mtp_debug_inject(int fault, int count);
 

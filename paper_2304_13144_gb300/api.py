@@ -577,6 +577,7 @@ MTP_FAULT_DEVICE_ALLOC = 1
 MTP_FAULT_NEIGHBOR_OVERFLOW = 2
 MTP_FAULT_GRADE_WAIT = 3
 MTP_FAULT_MAXVOL_WAIT = 4
+MTP_FAULT_ALLOC_SKIP = 5
 
 
 def mtp_debug_inject(fault, count):

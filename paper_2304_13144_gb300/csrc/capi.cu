@@ -19,6 +19,7 @@ static thread_local std::string g_last_error;
 void set_error(const std::string& msg) { g_last_error = msg; }
 
 std::atomic<int> g_inject_alloc{0};
+std::atomic<int> g_inject_alloc_skip{0};
 std::atomic<int> g_inject_overflow{0};
 std::atomic<int> g_inject_grade_wait{0};
 std::atomic<int> g_inject_maxvol_wait{0};
@@ -30,10 +31,16 @@ bool take_injected(std::atomic<int>& c) {
   return false;
 }
 
+// the armed allocation fault hits this growth
+static bool injected_alloc_failure() {
+  if (g_inject_alloc.load() <= 0 || take_injected(g_inject_alloc_skip)) return false;
+  return take_injected(g_inject_alloc);
+}
+
 void DevBuf::ensure(size_t need, cudaStream_t s) {
   if (need == 0) need = 16;
   if (bytes >= need) return;
-  if (take_injected(g_inject_alloc)) throw Fail{MTP_ERR_CUDA, "device allocation failed (injected fault)"};
+  if (injected_alloc_failure()) throw Fail{MTP_ERR_CUDA, "device allocation failed (injected fault)"};
   if (p) MTP_CUDA(cudaFreeAsync(p, s));
   p = nullptr;
   bytes = 0;
@@ -44,7 +51,7 @@ void DevBuf::ensure(size_t need, cudaStream_t s) {
 bool DevBuf::try_ensure(size_t need, cudaStream_t s) {
   if (need == 0) need = 16;
   if (bytes >= need) return true;
-  if (take_injected(g_inject_alloc)) return false;
+  if (injected_alloc_failure()) return false;
   if (p) MTP_CUDA(cudaFreeAsync(p, s));
   p = nullptr;
   bytes = 0;
@@ -1190,6 +1197,7 @@ mtp_status mtp_debug_inject(int fault, int count) {
     else if (fault == MTP_FAULT_NEIGHBOR_OVERFLOW) g_inject_overflow = count;
     else if (fault == MTP_FAULT_GRADE_WAIT) g_inject_grade_wait = count;
     else if (fault == MTP_FAULT_MAXVOL_WAIT) g_inject_maxvol_wait = count;
+    else if (fault == MTP_FAULT_ALLOC_SKIP) g_inject_alloc_skip = count;
     else throw Fail{MTP_ERR_ARG, "unknown fault"};
   });
 }

@@ -56,7 +56,10 @@ constexpr int S1 = 5;              // slice sums s < S1 in a first sweep over K,
                                    // 8 accumulators of FN columns each, the 512 of tensor memory
 constexpr int FTHREADS = 64 + 256;
 constexpr size_t FSMEM = NS * (FA + FB) + 256 + 1024;
-constexpr int64_t kChunkRows = 65536;   // rows sliced at a time (0.8 GB of slices at m = 651)
+// rows sliced at a time: 0.8 GB of slices at m = 651, at most 1 GB, down to kLeastRows where memory is
+// short (16 row tiles: still more tiles than SMs from m = 577 on)
+constexpr int64_t kChunkRows = 65536, kLeastRows = 2048;
+constexpr size_t kSliceBytes = size_t(1) << 30;
 
 // exponent e with |v| < 2^e (v finite), a very low one for zero
 __device__ __forceinline__ int exponent_of(double v) {
@@ -465,9 +468,10 @@ XPlan x_plan(int64_t m, void* base) {
 // from here on m the slices pay (below, a block of the SIMT kernel is done before a slice pass)
 bool grade_fp64_sliced(int64_t m) { return m >= 64 && m <= 16384; }
 
+// slices of A^-1; without the memory for them (18 m^2 bytes) the SIMT kernel grades
 void slice_active_inverse(mtp_model* md, int64_t m, cudaStream_t s) {
-  if (!grade_fp64_sliced(m)) return;
-  md->ainv_s.ensure(x_plan(m, nullptr).bytes, s);
+  md->have_slices = grade_fp64_sliced(m) && md->ainv_s.try_ensure(x_plan(m, nullptr).bytes, s);
+  if (!md->have_slices) return;
   const XPlan x = x_plan(m, md->ainv_s.p);
   const double* X = md->ainv_d.as<double>();
   MTP_CUDA(cudaMemsetAsync(x.xbad, 0, sizeof(int), s));
@@ -480,27 +484,59 @@ void slice_active_inverse(mtp_model* md, int64_t m, cudaStream_t s) {
   MTP_CUDA(cudaGetLastError());
 }
 
+namespace {
+
+// ws_grade for chunks of cn of N rows
+struct RowPlan {
+  int64_t np;
+  int n_best;
+  size_t sl, e, best, arg, bad;
+  RowPlan(const XPlan& x, int64_t cn, int64_t N)
+      : np((cn + FM - 1) / FM * FM),
+        n_best(x.pp / EN),
+        sl(static_cast<size_t>(NS) * np * x.kp * sizeof(uint16_t)),
+        e((np * sizeof(int) + 255) & ~size_t(255)),
+        best(static_cast<size_t>(n_best) * cn * sizeof(double)),
+        arg(static_cast<size_t>(n_best) * cn * sizeof(int32_t)),
+        bad(static_cast<size_t>(N)) {}
+  size_t bytes() const { return sl + e + best + arg + bad + 256; }
+};
+
+}  // namespace
+
+// Takes the workspace of an FP64 grade of N rows; returns the rows it grades at a time, 0 where the SIMT
+// kernel has to (no slices of A^-1, or no memory even for chunks of kLeastRows).
+int64_t reserve_grade_fp64(mtp_model* md, int64_t N, cudaStream_t s) {
+  if (!md->have_slices || N == 0) return 0;
+  const XPlan x = x_plan(md->m_active, md->ainv_s.p);
+  const int64_t fit = static_cast<int64_t>(kSliceBytes / (static_cast<size_t>(NS) * x.kp * sizeof(uint16_t))) / FM * FM;
+  int64_t cn = std::min<int64_t>(N, std::max(kLeastRows, std::min(kChunkRows, fit)));
+  while (!md->ws_grade.try_ensure(RowPlan(x, cn, N).bytes(), s)) {
+    if (cn <= kLeastRows) return 0;
+    cn = std::max(kLeastRows, cn / 2 / FM * FM);
+  }
+  return cn;
+}
+
 void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, double* gamma, int32_t* argmax, cudaStream_t s) {
   const int64_t m = md->m_active;
   if (N == 0) return;
-  if (!grade_fp64_sliced(m)) {
+  const int64_t cn = reserve_grade_fp64(md, N, s);
+  if (cn == 0) {
     run_grade_simt(md, N, true, rows, nullptr, ld, gamma, argmax, s);
     return;
   }
   const XPlan x = x_plan(m, md->ainv_s.p);
-  const int64_t cn = std::min<int64_t>(N, kChunkRows), np = (cn + FM - 1) / FM * FM;
-  const int n_col = x.pp / FN, n_best = x.pp / EN;
-  const size_t b_sl = static_cast<size_t>(NS) * np * x.kp * sizeof(uint16_t), b_e = (np * sizeof(int) + 255) & ~size_t(255),
-               b_best = static_cast<size_t>(n_best) * cn * sizeof(double), b_arg = static_cast<size_t>(n_best) * cn * sizeof(int32_t),
-               b_bad = static_cast<size_t>(N);
-  md->ws_grade.ensure(b_sl + b_e + b_best + b_arg + b_bad + 256, s);
+  const RowPlan rp(x, cn, N);
+  const int64_t np = rp.np;
+  const int n_col = x.pp / FN, n_best = rp.n_best;
   char* base = md->ws_grade.as<char>();
   uint16_t* sl = reinterpret_cast<uint16_t*>(base);
-  int* E = reinterpret_cast<int*>(base + b_sl);
-  double* pbest = reinterpret_cast<double*>(base + b_sl + b_e);
-  int32_t* parg = reinterpret_cast<int32_t*>(base + b_sl + b_e + b_best);
-  unsigned char* bad = reinterpret_cast<unsigned char*>(base + b_sl + b_e + b_best + b_arg);
-  MTP_CUDA(cudaMemsetAsync(bad, 0, b_bad, s));
+  int* E = reinterpret_cast<int*>(base + rp.sl);
+  double* pbest = reinterpret_cast<double*>(base + rp.sl + rp.e);
+  int32_t* parg = reinterpret_cast<int32_t*>(base + rp.sl + rp.e + rp.best);
+  unsigned char* bad = reinterpret_cast<unsigned char*>(base + rp.sl + rp.e + rp.best + rp.arg);
+  MTP_CUDA(cudaMemsetAsync(bad, 0, rp.bad, s));
   int nsm = 0;
   MTP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, md->device));
   MTP_CUDA(cudaFuncSetAttribute(k_grade_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(FSMEM)));

@@ -241,6 +241,7 @@ struct mtp_model {
   mtp::DevBuf ainv_f;          // padded FP32 (hi) and (lo) for the mixed grade
   int64_t ainv_ld = 0;
   mtp::DevBuf ainv_s;          // slices of A^-1 for the FP64 grade (grade_fp64.cu)
+  bool have_slices = false;
   // workspaces
   mtp::DevBuf ws_pair;         // per-pair gradients
   mtp::DevBuf ws_atom;         // per-atom V, W
@@ -372,6 +373,7 @@ int64_t run_cut_clusters(const mtp_batch* b, const int64_t* centers, int64_t n, 
                          double* pos, int32_t* type, int64_t* src, int64_t capacity, cudaStream_t s);
 // host-side fault injection (mtp_debug_inject): armed counts, each consumed by one event
 extern std::atomic<int> g_inject_alloc;
+extern std::atomic<int> g_inject_alloc_skip;
 extern std::atomic<int> g_inject_overflow;
 extern std::atomic<int> g_inject_grade_wait;
 extern std::atomic<int> g_inject_maxvol_wait;

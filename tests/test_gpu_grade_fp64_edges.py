@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 def api(native_lib):
     from paper_2304_13144_gb300 import api as A
     yield A
-    for f in (A.MTP_FAULT_DEVICE_ALLOC, A.MTP_FAULT_GRADE_WAIT):
+    for f in (A.MTP_FAULT_DEVICE_ALLOC, A.MTP_FAULT_ALLOC_SKIP, A.MTP_FAULT_GRADE_WAIT):
         A.mtp_debug_inject(f, 0)
 
 
@@ -148,3 +148,62 @@ def test_winning_column_of_small_terms_beside_cancelling_large_ones(api, types, 
     C = np.abs(np.stack([(r[:, None] * X).sum(0) for r in rows.astype(np.longdouble)])).max(1)
     tol = 2.0 ** -52 * C + m * 2.0 ** -53 * (np.abs(rows) * np.abs(X).max(1)).max(1)
     assert (np.abs(out["gamma"].cpu().numpy() - C) <= tol).all()
+
+
+def regions(api, call):
+    """The regions that a call runs."""
+    torch.cuda.synchronize()
+    api.mtp_profiler_enable(True)
+    try:
+        api.mtp_profiler_read()
+        call()
+        return set(api.mtp_profiler_read())
+    finally:
+        api.mtp_profiler_enable(False)
+
+
+def fail_growth(api, after, call):
+    """call() with the device allocation after `after` growths of its workspaces failing."""
+    try:
+        api.mtp_debug_inject(api.MTP_FAULT_ALLOC_SKIP, after)
+        api.mtp_debug_inject(api.MTP_FAULT_DEVICE_ALLOC, 1)
+        return call()
+    finally:
+        api.mtp_debug_inject(api.MTP_FAULT_DEVICE_ALLOC, 0)
+        api.mtp_debug_inject(api.MTP_FAULT_ALLOC_SKIP, 0)
+
+
+def test_without_memory_for_the_slices_of_rows(api):
+    """The rows' workspace exists, that of their slices cannot be had: the SIMT kernel answers."""
+    model, b, nb = setup(api)
+    api.mtp_set_active_set(model, torch.tensor(synth.diag_dominant(6, model.n_params), device="cuda"))
+    api.mtp_config_rows(model, b, nb, "fp64")
+    out = []
+    grade = lambda: out.append(api.mtp_grade(model, b, nb, "fp64")["gamma"].cpu().numpy())   # noqa: E731
+    ran = regions(api, lambda: fail_growth(api, 0, grade))
+    assert "grade_simt_fp64" in ran and "grade_fp64" not in ran
+    ran = regions(api, grade)
+    assert "grade_fp64" in ran and "grade_simt_fp64" not in ran
+    np.testing.assert_allclose(out[0], out[1], rtol=1e-12)
+
+
+def test_without_memory_for_the_slices_of_the_inverse(api):
+    """Of the allocations of an active set only the first five have to succeed (A, the factors, a flag,
+    the inverse, its mixed-precision copies); without the sixth FP64 grades take the SIMT kernel."""
+    A = None
+    out = []
+    for after in range(7):
+        model, b, nb = setup(api)
+        A = torch.tensor(synth.diag_dominant(6, model.n_params), device="cuda") if A is None else A
+        load = lambda: api.mtp_set_active_set(model, A)   # noqa: E731
+        if after < 5:
+            with pytest.raises(api.MtpError):
+                fail_growth(api, after, load)
+            load()
+        else:
+            fail_growth(api, after, load)
+        ran = regions(api, lambda: out.append(api.mtp_grade(model, b, nb, "fp64")["gamma"].cpu().numpy()))
+        assert ("grade_simt_fp64" if after == 5 else "grade_fp64") in ran, (after, ran)
+        assert len({"grade_simt_fp64", "grade_fp64"} & ran) == 1
+    for g in out:
+        np.testing.assert_allclose(g, out[0], rtol=1e-12)
