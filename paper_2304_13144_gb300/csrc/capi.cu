@@ -649,6 +649,7 @@ void upload_theta(mtp_model* md) {
 
 void run_grade_simt(mtp_model* md, int64_t N, bool fp64, const double* rows, const float* rows_f, int64_t ld,
                     double* gamma, int32_t* argmax, cudaStream_t s);
+int64_t reserve_grade_fp64(mtp_model* md, int64_t N, cudaStream_t s);
 void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, double* gamma, int32_t* argmax, cudaStream_t s);
 bool grade_tc_available(const mtp_model* md);
 void run_grade_tc(mtp_model* md, int64_t N, const float* hi, const float* lo, int64_t ld, double* gamma,
@@ -714,7 +715,7 @@ void check_model(const mtp_model* m) {
 
 // the workspace of the FP64 / dual-number pass, where the model has it; without the memory for it (a
 // value per moment and neighborhood, two in the tangent) the call runs on the generic kernel, which
-// has none
+// has none.  Callers take what they cannot do without before it, the scratch of later steps included.
 void give_wide(mtp_model* m, int64_t n_work, bool fp64, bool tangent, SiteOutputs& o, cudaStream_t s) {
   const size_t bytes = wide_workspace(m, n_work, fp64, tangent);
   if (!bytes) return;
@@ -781,7 +782,15 @@ void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_prec
     row_atom = order;
     zrow = z;
   }
-  if (fp64) give_wide(m, N, true, false, o, s);   // (last: what the call cannot do without comes first)
+  // scratch of the steps below, then (FP64) what the call can do without
+  const bool want_flags = want_grade && (flagged || n_flagged);
+  if (want_flags && !flagged) m->ws_misc.ensure(N * sizeof(int32_t) + 64, s);
+  if (fp64) {
+    const size_t red = std::max<size_t>(energy || virial ? config_sums_scratch(nb) : 0, want_flags ? flag_scratch(N) : 0);
+    if (red) m->ws_red.ensure(red, s);
+    if (want_grade) reserve_grade_fp64(m, N, s);
+    give_wide(m, N, true, false, o, s);
+  }
   run_sites(m, b, nb, fp64, o, false, nullptr, s);
   if (want_efs) {
     if (forces) run_forces(nb, fp64, o.G, forces, s);
@@ -794,10 +803,7 @@ void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_prec
     if (flagged || n_flagged) {
       int64_t* cnt = n_flagged;
       int32_t* fl = flagged;
-      if (!fl) {
-        m->ws_misc.ensure(N * sizeof(int32_t) + 64, s);
-        fl = m->ws_misc.as<int32_t>();
-      }
+      if (!fl) fl = m->ws_misc.as<int32_t>();
       if (!cnt) throw Fail{MTP_ERR_ARG, "flagged needs n_flagged"};
       run_flag(N, gamma, threshold, fl, cnt, m->ws_red, s);
     }
@@ -1387,6 +1393,7 @@ mtp_status mtp_config_rows(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb,
     cudaStream_t s = as_stream(stream);
     const int64_t m = md->sched.n_params, N = nb->n_atoms;
     md->ws_rows.ensure(std::max<int64_t>(N, 1) * m * sizeof(double), s);
+    md->ws_red.ensure(config_row_sums_scratch(nb, m), s);
     SiteOutputs o;
     o.rows = md->ws_rows.as<double>();
     o.rows_ld = m;
@@ -1411,6 +1418,7 @@ mtp_status mtp_energy_vjp(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
       work.ensure(std::max<int64_t>(K, 1) * m * sizeof(double), s);
       R = work.as<double>();
       md->ws_rows.ensure(std::max<int64_t>(N, 1) * m * sizeof(double), s);
+      md->ws_red.ensure(config_row_sums_scratch(nb, m), s);
       SiteOutputs o;
       o.rows = md->ws_rows.as<double>();
       o.rows_ld = m;
@@ -1436,6 +1444,7 @@ mtp_status mtp_config_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb
     ScopedBuf work(s);
     if (mode == MTP_GRADE_NEIGHBORHOOD) {
       work.ensure(std::max<int64_t>(nb->n_atoms, 1) * sizeof(double), s);
+      md->ws_misc.ensure(config_gamma_max_scratch(nb), s);
       efs_and_grade(md, b, nb, prec, nullptr, nullptr, nullptr, nullptr, 0.0, work.as<double>(), nullptr, nullptr,
                     nullptr, s);
       run_config_gamma_max(nb, work.as<double>(), gamma_cfg, worst, md->ws_misc, s);
@@ -1446,9 +1455,11 @@ mtp_status mtp_config_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb
       int32_t* am = reinterpret_cast<int32_t*>(rc + std::max<int64_t>(K, 1) * m);
       const int64_t N = nb->n_atoms;
       md->ws_rows.ensure(std::max<int64_t>(N, 1) * m * sizeof(double), s);
+      md->ws_red.ensure(config_row_sums_scratch(nb, m), s);
       SiteOutputs o;
       o.rows = md->ws_rows.as<double>();
       o.rows_ld = m;
+      reserve_grade_fp64(md, K, s);
       give_wide(md, N, prec == MTP_FP64, false, o, s);
       run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
       run_config_row_sums(nb, md->ws_rows.as<double>(), m, rc, md->ws_red, s);
@@ -1541,6 +1552,15 @@ mtp_status mtp_train_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     double* W = E + n_cfg;
     double* coef = W + 9 * n_cfg;
     double* Sc = coef + n_cfg;
+    // pass 2's partial gradients, and the scratch of the sums, before what the call can do without
+    const int rows_per_block = 4;
+    int dev = 0, nsm = 0;
+    MTP_CUDA(cudaGetDevice(&dev));
+    MTP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int gmax = nsm * 4;
+    const size_t part_bytes = static_cast<size_t>(gmax) * rows_per_block * m * sizeof(double);
+    md->ws_rows.ensure(part_bytes, s);
+    md->ws_red.ensure(std::max(config_sums_scratch(nb), train_prep_scratch()), s);
     SiteOutputs o;
     o.V = V; o.Wat = Wat; o.G = md->ws_pair.p;
     if (fp64) {
@@ -1559,13 +1579,6 @@ mtp_status mtp_train_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     t.U = U;
     t.Scfg = Sc;
     t.coef = coef;
-    const int rows_per_block = 4;
-    int dev = 0, nsm = 0;
-    MTP_CUDA(cudaGetDevice(&dev));
-    MTP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    const int gmax = nsm * 4;
-    const size_t part_bytes = static_cast<size_t>(gmax) * rows_per_block * m * sizeof(double);
-    md->ws_rows.ensure(part_bytes, s);
     MTP_CUDA(cudaMemsetAsync(md->ws_rows.p, 0, part_bytes, s));
     t.grad_part = md->ws_rows.as<double>();
     give_wide(md, N, fp64, true, t, s);

@@ -121,8 +121,13 @@ __global__ void k_widen_argmax(const int32_t* in, int64_t n, int64_t* out) {
 
 }  // namespace
 
+size_t config_row_sums_scratch(const mtp_nbr* nb, int64_t m) { return static_cast<size_t>(nb->n_seg) * m * sizeof(double); }
+size_t config_gamma_max_scratch(const mtp_nbr* nb) {
+  return static_cast<size_t>(std::max<int64_t>(nb->n_seg, 1)) * (sizeof(double) + sizeof(int64_t));
+}
+
 void run_config_row_sums(const mtp_nbr* nb, const double* rows, int64_t m, double* out, DevBuf& tmp, cudaStream_t s) {
-  tmp.ensure(static_cast<size_t>(nb->n_seg) * m * sizeof(double), s);
+  tmp.ensure(config_row_sums_scratch(nb, m), s);
   ProfRegion pr("config_rows_sum", s);
   const dim3 g(static_cast<unsigned>(nb->n_seg), blocks(m, 128));
   if (nb->n_seg > 0) {
@@ -137,7 +142,7 @@ void run_config_row_sums(const mtp_nbr* nb, const double* rows, int64_t m, doubl
 
 void run_config_gamma_max(const mtp_nbr* nb, const double* gamma, double* gamma_cfg, int64_t* worst, DevBuf& tmp,
                           cudaStream_t s) {
-  tmp.ensure(static_cast<size_t>(std::max<int64_t>(nb->n_seg, 1)) * (sizeof(double) + sizeof(int64_t)), s);
+  tmp.ensure(config_gamma_max_scratch(nb), s);
   double* gmax = tmp.as<double>();
   int64_t* amax = reinterpret_cast<int64_t*>(gmax + std::max<int64_t>(nb->n_seg, 1));
   ProfRegion pr("config_gamma_max", s);

@@ -399,6 +399,12 @@ int64_t run_maxvol(mtp_model* md, const double* B, int64_t n, double eps, int64_
                    cudaStream_t s);
 void run_grade(mtp_model* m, int64_t N, bool fp64, const double* rows, const float* rows_hi,
                const float* rows_lo, int64_t ld, double* gamma, int32_t* argmax, cudaStream_t s);
+// bytes of the scratch that the steps below take
+size_t config_sums_scratch(const mtp_nbr* nb);
+size_t config_row_sums_scratch(const mtp_nbr* nb, int64_t m);
+size_t config_gamma_max_scratch(const mtp_nbr* nb);
+size_t flag_scratch(int64_t N);
+size_t train_prep_scratch();
 void run_flag(int64_t N, const double* gamma, double threshold, int32_t* flagged, int64_t* n_flagged,
               DevBuf& tmp, cudaStream_t s);
 int64_t run_extract(const mtp_nbr* nb, const mtp_batch* b, const int32_t* idx, int64_t n, int64_t* off,

@@ -285,9 +285,11 @@ void run_forces(const mtp_nbr* nb, bool fp64, const void* G, double* F, cudaStre
   MTP_CUDA(cudaGetLastError());
 }
 
+size_t config_sums_scratch(const mtp_nbr* nb) { return nb->n_seg * 10 * sizeof(double); }
+
 void run_config_sums(const mtp_nbr* nb, const double* V, const double* Wat, double* E, double* W, DevBuf& tmp,
                      cudaStream_t s) {
-  tmp.ensure(nb->n_seg * 10 * sizeof(double), s);
+  tmp.ensure(config_sums_scratch(nb), s);
   ProfRegion pr("config_sums", s);
   launch_seg_sums(nb, V, Wat, tmp.as<double>(), s);
   k_cfg_sums<<<nblk(nb->n_cfg * 32, 128), 128, 0, s>>>(nb->seg.as<int64_t>(), nb->n_seg, tmp.as<double>(),
@@ -393,6 +395,14 @@ void run_species_order(const int32_t* type, int64_t N, int n_types, int32_t* zro
   MTP_CUDA(cudaGetLastError());
 }
 
+size_t flag_scratch(int64_t N) {
+  size_t bytes = 0;
+  thrust::counting_iterator<int> it(0);
+  MTP_CUDA(cub::DeviceSelect::If(nullptr, bytes, it, static_cast<int32_t*>(nullptr), static_cast<int64_t*>(nullptr),
+                                 static_cast<int>(N), AboveThreshold{nullptr, 0.0}));
+  return bytes;
+}
+
 void run_flag(int64_t N, const double* gamma, double threshold, int32_t* flagged, int64_t* n_flagged, DevBuf& tmp,
               cudaStream_t s) {
   AboveThreshold pred{gamma, threshold};
@@ -434,11 +444,16 @@ int64_t run_extract(const mtp_nbr* nb, const mtp_batch* b, const int32_t* idx, i
   return total;
 }
 
+namespace {
+constexpr int kResidualBlocks = 256;
+}
+size_t train_prep_scratch() { return kResidualBlocks * sizeof(double); }
+
 void run_train_prep(const mtp_nbr* nb, int n_cfg, const double* E, const double* F, const double* W,
                     const double* E_ref, const double* F_ref, const double* W_ref, double w_e, double w_f,
                     double w_s, double* coef, double* U, double* Scfg, double* loss, DevBuf& tmp, cudaStream_t s) {
-  const int nb_f = 256;
-  tmp.ensure(nb_f * sizeof(double), s);
+  const int nb_f = kResidualBlocks;
+  tmp.ensure(train_prep_scratch(), s);
   ProfRegion pr("train_residuals", s);
   k_train_forces<<<nb_f, 256, 0, s>>>(nb->n_atoms, F, F_ref, w_f, U, tmp.as<double>());
   ProfRegion::launched();
