@@ -577,13 +577,11 @@ void slice_active_inverse(mtp_model* md, int64_t m, cudaStream_t s);
 void run_lu_inverse(mtp_model* md, const double* A, int64_t m, cudaStream_t s) {
   ScopedBuf work(s);
   const size_t mm = static_cast<size_t>(m * m);
-  work.ensure((2 * mm + (m + kBack) * kBack + m * kPanel + kPanel * kPanel + 1) * sizeof(double) + sizeof(PanelMoves) + m * sizeof(int) + 64, s);
+  const bool panels = m <= kPanelRows;
+  const size_t panel_doubles = panels ? mm + (m + kBack) * kBack + m * kPanel + kPanel * kPanel : 0;   // W, D, Lp, Tp
+  work.ensure((mm + panel_doubles + 1) * sizeof(double) + sizeof(PanelMoves) + m * sizeof(int) + 64, s);
   double* M = work.as<double>();
-  double* W = M + mm;
-  double* D = W + mm;
-  double* Lp = D + (m + kBack) * kBack;
-  double* Tp = Lp + m * kPanel;
-  unsigned long long* maxabs = reinterpret_cast<unsigned long long*>(Tp + kPanel * kPanel);
+  unsigned long long* maxabs = reinterpret_cast<unsigned long long*>(M + mm + panel_doubles);
   PanelMoves* mv = reinterpret_cast<PanelMoves*>(maxabs + 1);
   int* perm = reinterpret_cast<int*>(mv + 1);
   md->err_flag.ensure(sizeof(unsigned), s);
@@ -598,8 +596,15 @@ void run_lu_inverse(mtp_model* md, const double* A, int64_t m, cudaStream_t s) {
   md->ainv_d.ensure(mm * sizeof(double), s);
   double* inv = md->ainv_d.as<double>();
   unsigned* flag_d = md->err_flag.as<unsigned>();
-  if (m <= kPanelRows) invert_by_panels(M, W, D, Lp, Tp, mv, perm, m, maxabs, flag_d, inv, s);
-  else invert_by_columns(M, perm, m, maxabs, flag_d, inv, s);
+  if (panels) {
+    double* W = M + mm;
+    double* D = W + mm;
+    double* Lp = D + (m + kBack) * kBack;
+    double* Tp = Lp + m * kPanel;
+    invert_by_panels(M, W, D, Lp, Tp, mv, perm, m, maxabs, flag_d, inv, s);
+  } else {
+    invert_by_columns(M, perm, m, maxabs, flag_d, inv, s);
+  }
   // mixed-path copies: K-major padded split (tensor cores) and plain FP32 (SIMT)
   const int64_t ld = grade_tc_ld(m);
   md->ainv_ld = ld;
