@@ -40,12 +40,18 @@ static bool injected_alloc_failure() {
 void DevBuf::ensure(size_t need, cudaStream_t s) {
   if (need == 0) need = 16;
   if (bytes >= need) return;
-  if (injected_alloc_failure()) throw Fail{MTP_ERR_CUDA, "device allocation failed (injected fault)"};
+  if (injected_alloc_failure()) throw Fail{MTP_ERR_CUDA, "device allocation failed (injected fault)", true};
   if (p) MTP_CUDA(cudaFreeAsync(p, s));
   p = nullptr;
   bytes = 0;
   size_t cap = need + need / 8;
-  MTP_CUDA(cudaMallocAsync(&p, cap, s));
+  const cudaError_t e = cudaMallocAsync(&p, cap, s);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    p = nullptr;
+    throw Fail{MTP_ERR_CUDA, std::string("device allocation failed: ") + cudaGetErrorString(e), true};
+  }
+  MTP_CUDA(e);
   bytes = cap;
 }
 bool DevBuf::try_ensure(size_t need, cudaStream_t s) {
@@ -70,6 +76,20 @@ void DevBuf::release() {
   if (p) cudaFree(p);
   p = nullptr;
   bytes = 0;
+}
+namespace {
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+}  // namespace
+bool give_back_optional(mtp_model* m, cudaStream_t s) {
+  if (!m || !m->ws_wide.p || m->wide_captured || capturing(s)) return false;
+  MTP_CUDA(cudaDeviceSynchronize());   // (its last pass may have run on another stream)
+  m->ws_wide.release();
+  return true;
 }
 void* PinPool::take() {
   {
@@ -719,14 +739,15 @@ void check_model(const mtp_model* m) {
 void give_wide(mtp_model* m, int64_t n_work, bool fp64, bool tangent, SiteOutputs& o, cudaStream_t s) {
   const size_t bytes = wide_workspace(m, n_work, fp64, tangent);
   if (!bytes) return;
-  if (m->ws_wide.try_ensure(bytes, s)) o.wide = m->ws_wide.p;
+  if (!m->ws_wide.try_ensure(bytes, s)) return;
+  o.wide = m->ws_wide.p;
+  if (!m->wide_captured && capturing(s)) m->wide_captured = true;
 }
 
 // Shared body of the EFS / grade / step entry points.
-void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec, double* energy,
-                   double* site_energy, double* forces, double* virial, double threshold, double* gamma,
-                   int32_t* argmax, int32_t* flagged, int64_t* n_flagged, cudaStream_t s,
-                   double* site_virial = nullptr) {
+void efs_and_grade_once(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec, double* energy,
+                        double* site_energy, double* forces, double* virial, double threshold, double* gamma,
+                        int32_t* argmax, int32_t* flagged, int64_t* n_flagged, cudaStream_t s, double* site_virial) {
   check_run(m, b, nb);
   if (prec != MTP_FP64 && prec != MTP_MIXED) throw Fail{MTP_ERR_ARG, "unknown precision"};
   const bool fp64 = prec == MTP_FP64;
@@ -808,6 +829,16 @@ void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_prec
       run_flag(N, gamma, threshold, fl, cnt, m->ws_red, s);
     }
   }
+}
+
+void efs_and_grade(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec, double* energy,
+                   double* site_energy, double* forces, double* virial, double threshold, double* gamma,
+                   int32_t* argmax, int32_t* flagged, int64_t* n_flagged, cudaStream_t s,
+                   double* site_virial = nullptr) {
+  with_memory(m, s, [&] {
+    efs_and_grade_once(m, b, nb, prec, energy, site_energy, forces, virial, threshold, gamma, argmax, flagged,
+                       n_flagged, s, site_virial);
+  });
 }
 
 }  // namespace
@@ -1229,9 +1260,9 @@ mtp_status mtp_set_active_set(mtp_model* md, const double* A, int64_t m, void* s
     if (!A || m != md->sched.n_params) throw Fail{MTP_ERR_ARG, "active-set matrix must be m x m"};
     md->have_ainv = false;
     cudaStream_t s = as_stream(stream);
-    md->a_d.ensure(m * m * sizeof(double), s);
+    with_memory(md, s, [&] { md->a_d.ensure(m * m * sizeof(double), s); });
     MTP_CUDA(cudaMemcpyAsync(md->a_d.p, A, m * m * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    run_lu_inverse(md, md->a_d.as<double>(), m, s);
+    with_memory(md, s, [&] { run_lu_inverse(md, md->a_d.as<double>(), m, s); });
   });
 }
 
@@ -1386,7 +1417,7 @@ mtp_status mtp_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mtp_p
 
 mtp_status mtp_config_rows(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec, double* rows,
                            void* stream) {
-  return guarded([&] {
+  return guarded([&] { with_memory(md, as_stream(stream), [&] {
     check_run(md, b, nb);
     if (prec != MTP_FP64 && prec != MTP_MIXED) throw Fail{MTP_ERR_ARG, "unknown precision"};
     if (!rows) throw Fail{MTP_ERR_ARG, "null rows"};
@@ -1400,12 +1431,12 @@ mtp_status mtp_config_rows(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb,
     give_wide(md, N, prec == MTP_FP64, false, o, s);
     run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
     run_config_row_sums(nb, md->ws_rows.as<double>(), m, rows, md->ws_red, s);
-  });
+  }); });
 }
 
 mtp_status mtp_energy_vjp(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec,
                           const double* gE, const double* forces, double* g_pos, double* g_theta, void* stream) {
-  return guarded([&] {
+  return guarded([&] { with_memory(md, as_stream(stream), [&] {
     check_run(md, b, nb);
     if (prec != MTP_FP64 && prec != MTP_MIXED) throw Fail{MTP_ERR_ARG, "unknown precision"};
     if (!gE || (!g_pos && !g_theta)) throw Fail{MTP_ERR_ARG, "null gE or no output requested"};
@@ -1428,13 +1459,13 @@ mtp_status mtp_energy_vjp(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     }
     run_energy_vjp(nb, R, gE, m, forces, g_pos, g_theta, s);
     MTP_CUDA(cudaStreamSynchronize(s));
-  });
+  }); });
 }
 
 mtp_status mtp_config_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec,
                             mtp_grade_mode mode, double gamma_save, double gamma_break, double* gamma_cfg,
                             int64_t* worst, int32_t* cls, void* stream) {
-  return guarded([&] {
+  return guarded([&] { with_memory(md, as_stream(stream), [&] {
     check_run(md, b, nb);
     if (!gamma_cfg) throw Fail{MTP_ERR_ARG, "null gamma_cfg"};
     if (mode != MTP_GRADE_NEIGHBORHOOD && mode != MTP_GRADE_CONFIGURATION) throw Fail{MTP_ERR_ARG, "unknown mode"};
@@ -1468,7 +1499,7 @@ mtp_status mtp_config_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb
     }
     if (cls) run_classify(gamma_cfg, K, gamma_save, gamma_break, cls, s);
     MTP_CUDA(cudaStreamSynchronize(s));
-  });
+  }); });
 }
 
 mtp_status mtp_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec, double* energy,
@@ -1528,7 +1559,7 @@ mtp_status mtp_cut_clusters(const mtp_batch* b, const int64_t* centers, int64_t 
 mtp_status mtp_train_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec,
                           const double* E_ref, const double* F_ref, const double* W_ref, double w_e, double w_f,
                           double w_s, double* loss, double* grad, void* stream) {
-  return guarded([&] {
+  return guarded([&] { with_memory(md, as_stream(stream), [&] {
     check_run(md, b, nb);
     if (!E_ref || !F_ref || !loss || !grad) throw Fail{MTP_ERR_ARG, "null argument"};
     if (w_s != 0.0 && !W_ref) throw Fail{MTP_ERR_ARG, "w_s != 0 needs W_ref"};
@@ -1589,7 +1620,7 @@ mtp_status mtp_train_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
       part_rows = static_cast<int64_t>(used) * rows_per_block;
     }
     run_sum_rows(t.grad_part, static_cast<int>(part_rows), m, grad, s);
-  });
+  }); });
 }
 
 }  // extern "C"

@@ -233,7 +233,9 @@ int64_t run_maxvol(mtp_model* md, const double* B, int64_t n, double eps, int64_
   int dev = 0, nsm = 0;
   MTP_CUDA(cudaGetDevice(&dev));
   MTP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  work.ensure(cbytes + (n + 3 * m) * sizeof(double) + nsm * sizeof(Best) + sizeof(SwapState) + 256, s);
+  with_memory(md, s, [&] {
+    work.ensure(cbytes + (n + 3 * m) * sizeof(double) + nsm * sizeof(Best) + sizeof(SwapState) + 256, s);
+  });
   long long* src = work.as<long long>();
   double* C = reinterpret_cast<double*>(src + m);
   double* v = C + n * m;
@@ -277,7 +279,7 @@ int64_t run_maxvol(mtp_model* md, const double* B, int64_t n, double eps, int64_
   }
   if (source) MTP_CUDA(cudaMemcpyAsync(source, src, m * sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
   if (swaps > 0) {
-    run_lu_inverse(md, md->a_d.as<double>(), m, s);
+    with_memory(md, s, [&] { run_lu_inverse(md, md->a_d.as<double>(), m, s); });
   } else {
     MTP_CUDA(cudaStreamSynchronize(s));
     md->have_ainv = true;   // nothing was changed

@@ -24,6 +24,7 @@ void set_error(const std::string& msg);
 struct Fail {
   mtp_status st;
   std::string msg;
+  bool no_memory = false;   // a device allocation failed
 };
 #define MTP_CUDA(call)                                                                    \
   do {                                                                                    \
@@ -293,9 +294,29 @@ struct mtp_model {
   } wide_words;
   mtp::DevBuf wide_tab;
   mtp::DevBuf ws_wide;         // its moments / their adjoints
+  bool wide_captured = false;  // a stream capture has seen ws_wide: a graph may hold its address
   mtp::DevBuf split_tab;       // slot -> component table of the split pass (uploaded by mtp_load)
   mtp::DevBuf ws_mom;          // moments / their adjoints of the split pass
 };
+
+namespace mtp {
+// Gives back the model's workspace of the FP64 / dual-number pass, the largest that a call can do
+// without and that is kept between calls; false where there is none, or where a captured graph may
+// hold its address.
+bool give_back_optional(mtp_model* m, cudaStream_t s);
+// Runs `f` (repeatable); where it fails for want of device memory, once more without that workspace.
+// (Not for list builds, which may run beside a call that uses it.)
+template <class F>
+void with_memory(mtp_model* m, cudaStream_t s, F&& f) {
+  try {
+    f();
+    return;
+  } catch (const Fail& e) {
+    if (!e.no_memory || !give_back_optional(m, s)) throw;
+  }
+  f();
+}
+}  // namespace mtp
 
 struct mtp_nbr {
   int device = 0;

@@ -97,3 +97,57 @@ def test_optional_growths_come_last(api, what, prec):
             assert np.abs(x - y).max() <= tol * max(1.0, np.abs(y).max()), (after, passed)
     assert passed == sorted(passed), passed
     assert passed[-1] and not passed[0]
+
+
+def test_kept_workspace_is_given_back_where_a_call_needs_memory(api):
+    """The FP64 pass keeps its workspace between calls.  A later call that cannot grow what it needs runs
+    again after giving it back; a second failure is reported."""
+    theta = theta_of(2, 12)
+    b = api.Batch(synth.training_batch(seed=4, n_cfg=6, n_types=2, lo=8, hi=64))
+    model = api.mtp_load(api.make_desc(2, 12), theta)
+    nb = api.mtp_build_neighbors(model, b)
+    ref = api.mtp_energy_forces_stress(api.mtp_load(api.make_desc(2, 12), theta), b, nb, "mixed")["forces"]
+    rows = api.mtp_param_rows(model, b, nb, "fp64")          # takes the workspace, and nothing else
+    with fail_growth(api, 0):
+        out = api.mtp_energy_forces_stress(model, b, nb, "mixed")["forces"]
+    assert torch.equal(out, ref)
+    with fail_growth(api, 0):                                 # the workspace is gone: to be taken again
+        plain = api.mtp_param_rows(model, b, nb, "fp64")
+    assert not torch.equal(plain, rows)                       # (the generic kernel's rounding)
+    assert (plain - rows).abs().max() <= 1e-10 * rows.abs().max()
+    assert torch.equal(api.mtp_param_rows(model, b, nb, "fp64"), rows)
+    other = api.mtp_load(api.make_desc(2, 12), theta)
+    with fail_growth(api, 0):                                 # nothing to give back
+        with pytest.raises(api.MtpError) as e:
+            api.mtp_energy_forces_stress(other, b, nb, "mixed")
+    assert e.value.name == "MTP_ERR_CUDA"
+
+
+def test_a_captured_workspace_stays(api):
+    """A graph holds the workspace's address: it is kept although another call fails for want of memory."""
+    theta = theta_of(2, 12)
+    b = api.Batch(synth.training_batch(seed=4, n_cfg=6, n_types=2, lo=8, hi=64))
+    model = api.mtp_load(api.make_desc(2, 12), theta)
+    nb = api.mtp_build_neighbors(model, b)
+    dev = {"dtype": torch.float64, "device": "cuda"}
+    out = {"energy": torch.empty(b.n_cfg, **dev), "forces": torch.empty((b.n_atoms, 3), **dev),
+           "virial": torch.empty((b.n_cfg, 3, 3), **dev)}
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        api.mtp_step(model, b, nb, "fp64", out=out, grade=False)
+    torch.cuda.synchronize()
+    ref = {k: v.clone() for k, v in out.items()}
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        api.mtp_step(model, b, nb, "fp64", out=out, grade=False)
+    big = api.Batch(synth.training_batch(seed=5, n_cfg=8, n_types=2, lo=100, hi=200))
+    nb2 = api.mtp_build_neighbors(model, big)
+    with fail_growth(api, 0):
+        with pytest.raises(api.MtpError):
+            api.mtp_config_rows(model, big, nb2, "mixed")
+    for v in out.values():
+        v.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    for k, v in out.items():
+        assert torch.equal(v, ref[k]), k
