@@ -736,9 +736,12 @@ void check_model(const mtp_model* m) {
 // the workspace of the FP64 / dual-number pass, where the model has it; without the memory for it (a
 // value per moment and neighborhood, two in the tangent) the call runs on the generic kernel, which
 // has none.  Callers take what they cannot do without before it, the scratch of later steps included.
-void give_wide(mtp_model* m, int64_t n_work, bool fp64, bool tangent, SiteOutputs& o, cudaStream_t s) {
+void give_wide(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, int64_t n_work, bool fp64, bool tangent,
+               SiteOutputs& o, cudaStream_t s) {
   const size_t bytes = wide_workspace(m, n_work, fp64, tangent);
   if (!bytes) return;
+  // FP32 rows go to the single kernel where it has the shape
+  if (!fp64 && !tangent && run_sites_fast(m, b, nb, o, s, true)) return;
   if (!m->ws_wide.try_ensure(bytes, s)) return;
   o.wide = m->ws_wide.p;
   if (!m->wide_captured && capturing(s)) m->wide_captured = true;
@@ -810,7 +813,7 @@ void efs_and_grade_once(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp
     const size_t red = std::max<size_t>(energy || virial ? config_sums_scratch(nb) : 0, want_flags ? flag_scratch(N) : 0);
     if (red) m->ws_red.ensure(red, s);
     if (want_grade) reserve_grade_fp64(m, N, s);
-    give_wide(m, N, true, false, o, s);
+    give_wide(m, b, nb, N, true, false, o, s);
   }
   run_sites(m, b, nb, fp64, o, false, nullptr, s);
   if (want_efs) {
@@ -1428,7 +1431,7 @@ mtp_status mtp_config_rows(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb,
     SiteOutputs o;
     o.rows = md->ws_rows.as<double>();
     o.rows_ld = m;
-    give_wide(md, N, prec == MTP_FP64, false, o, s);
+    give_wide(md, b, nb, N, prec == MTP_FP64, false, o, s);
     run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
     run_config_row_sums(nb, md->ws_rows.as<double>(), m, rows, md->ws_red, s);
   }); });
@@ -1453,7 +1456,7 @@ mtp_status mtp_energy_vjp(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
       SiteOutputs o;
       o.rows = md->ws_rows.as<double>();
       o.rows_ld = m;
-      give_wide(md, N, prec == MTP_FP64, false, o, s);
+      give_wide(md, b, nb, N, prec == MTP_FP64, false, o, s);
       run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
       run_config_row_sums(nb, md->ws_rows.as<double>(), m, R, md->ws_red, s);
     }
@@ -1491,7 +1494,7 @@ mtp_status mtp_config_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb
       o.rows = md->ws_rows.as<double>();
       o.rows_ld = m;
       reserve_grade_fp64(md, K, s);
-      give_wide(md, N, prec == MTP_FP64, false, o, s);
+      give_wide(md, b, nb, N, prec == MTP_FP64, false, o, s);
       run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
       run_config_row_sums(nb, md->ws_rows.as<double>(), m, rc, md->ws_red, s);
       run_grade_fp64(md, K, rc, m, gamma_cfg, am, s);
@@ -1522,7 +1525,7 @@ mtp_status mtp_param_rows(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     o.rows_ld = md->sched.n_params;
     o.atom_list = atoms;
     o.n_list = atoms ? n : nb->n_atoms;
-    give_wide(md, o.n_list, prec == MTP_FP64, false, o, as_stream(stream));
+    give_wide(md, b, nb, o.n_list, prec == MTP_FP64, false, o, as_stream(stream));
     run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, as_stream(stream));
   });
 }
@@ -1595,7 +1598,7 @@ mtp_status mtp_train_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     SiteOutputs o;
     o.V = V; o.Wat = Wat; o.G = md->ws_pair.p;
     if (fp64) {
-      give_wide(md, N, true, false, o, s);
+      give_wide(md, b, nb, N, true, false, o, s);
     } else if (split_wanted(md)) {
       // (without the memory for it: the single kernel)
       if (md->ws_mom.try_ensure(std::max<int64_t>(N, 1) * split_ldm(md->ds.n_mom) * sizeof(float), s))
@@ -1612,7 +1615,7 @@ mtp_status mtp_train_step(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     t.coef = coef;
     MTP_CUDA(cudaMemsetAsync(md->ws_rows.p, 0, part_bytes, s));
     t.grad_part = md->ws_rows.as<double>();
-    give_wide(md, N, fp64, true, t, s);
+    give_wide(md, b, nb, N, fp64, true, t, s);
     int64_t part_rows = 0;
     if (!run_sites_wide(md, b, nb, fp64, t, true, gmax * rows_per_block, &part_rows, s)) {
       int used = gmax;

@@ -412,6 +412,9 @@ inline int padded_nv(int n_values) { return (n_values + 1 + 3) & ~3; }
 // per-atom stride (floats) of the split pass's moment workspace
 inline int split_ldm(int n_mom) { return (n_mom + 3) & ~3; }
 void split_prepare(mtp_model* m);
+// single-kernel mixed pass (site_fast.cu): false, and nothing launched, where it has no shape for the
+// call; with `ask` it only answers
+bool run_sites_fast(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, const SiteOutputs& o, cudaStream_t s, bool ask);
 // whether the mixed path takes the three-kernel pass (caller's setting, else the autotuner's)
 inline bool split_wanted(const mtp_model* m) {
   return m->split_tab.p && (m->mixed_pass == 2 || (m->mixed_pass == 0 && m->tune_split != 0));

@@ -473,8 +473,8 @@ void dispatch_mode(FastParams P, int nwarps, bool efs, bool rows, cudaStream_t s
 }  // namespace
 
 // Returns false when the model's shape has no specialised instantiation (the caller then uses
-// the generic kernel).
-bool run_sites_fast(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, const SiteOutputs& o, cudaStream_t s) {
+// the generic kernel).  `ask`: answers only, launches nothing.
+bool run_sites_fast(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, const SiteOutputs& o, cudaStream_t s, bool ask) {
   const DevSchedule& d = m->ds;
   if (!d.tri_pk || d.n_q != kNQ) return false;
   const bool efs = o.V != nullptr;
@@ -531,6 +531,8 @@ bool run_sites_fast(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, const S
   bool fg = m->tune_fwd_global >= 0 ? (m->tune_fwd_global == 1 && wg > 0) : (std::min(wg, 7) > ws);
   if (!fg && ws == 0) fg = wg > 0;
   if (!fg && ws == 0) return false;
+  if (!(nr == 2 && nu0 == 2) && !(nr == 3 && nu0 == 4) && !(nr == 4 && nu0 == 6) && !(nr == 5 && nu0 == 8)) return false;
+  if (ask) return true;
   P = fg ? Pg : Ps;
   int nwarps = fg ? wg : ws;
   // untuned default: at most 7 warps with the forward schedule in global memory (8 fit at level
@@ -545,8 +547,8 @@ bool run_sites_fast(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, const S
   if (nr == 2 && nu0 == 2) { dispatch_mode<2, 2, false>(P, nwarps, efs, rows, s); return true; }
   if (nr == 3 && nu0 == 4) { dispatch_mode<3, 4, false>(P, nwarps, efs, rows, s); return true; }
   if (nr == 4 && nu0 == 6) { dispatch_mode<4, 6, false>(P, nwarps, efs, rows, s); return true; }
-  if (nr == 5 && nu0 == 8) { dispatch_mode<5, 8, false>(P, nwarps, efs, rows, s); return true; }
-  return false;
+  dispatch_mode<5, 8, false>(P, nwarps, efs, rows, s);
+  return true;
 }
 
 }  // namespace mtp

@@ -151,3 +151,21 @@ def test_a_captured_workspace_stays(api):
     torch.cuda.synchronize()
     for k, v in out.items():
         assert torch.equal(v, ref[k]), k
+
+
+@pytest.mark.parametrize("lev", [8, 16, 24])
+def test_mixed_rows_take_no_workspace_that_nothing_uses(api, lev):
+    """FP32 rows of the shapes of the single kernel (all levels of it but 24 here) need no growth: the
+    armed failure is still there for the next call."""
+    theta = theta_of(1, lev)
+    b = api.Batch(synth.fcc_unary_108())
+    model = api.mtp_load(api.make_desc(1, lev), theta)
+    nb = api.mtp_build_neighbors(model, b)
+    with fail_growth(api, 0):
+        api.mtp_param_rows(model, b, nb, "mixed")
+        if lev == 24:
+            api.mtp_energy_forces_stress(model, b, nb, "mixed")
+        else:
+            with pytest.raises(api.MtpError) as e:
+                api.mtp_energy_forces_stress(model, b, nb, "mixed")
+            assert "injected" in str(e.value)
