@@ -984,7 +984,7 @@ mtp_status mtp_autotune(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mt
     if (prec != MTP_FP64 && prec != MTP_MIXED) throw Fail{MTP_ERR_ARG, "unknown precision"};
     cudaStream_t s = as_stream(stream);
     const int64_t N = nb->n_atoms, K = nb->n_cfg;
-    DevBuf out;
+    ScopedBuf out(s);
     out.ensure((K * 10 + 4 * std::max<int64_t>(N, 1)) * sizeof(double) + 64, s);
     double* E = out.as<double>();
     double* W = E + K;

@@ -169,3 +169,19 @@ def test_mixed_rows_take_no_workspace_that_nothing_uses(api, lev):
             with pytest.raises(api.MtpError) as e:
                 api.mtp_energy_forces_stress(model, b, nb, "mixed")
             assert "injected" in str(e.value)
+
+
+def test_autotune_gives_its_outputs_back(api):
+    """Its energies, forces and grades (2 MB for this batch) go when it returns."""
+    desc = api.make_desc(1, 4)
+    model = api.mtp_load(desc, np.full(api.mtp_describe(desc)["n_params"], 0.01))
+    pos, cell, _ = synth.cubic_supercell(synth._FCC, 3.6, 26)
+    b = api.Batch(synth.single(pos + synth.rng(2).normal(0, 0.1, pos.shape), np.zeros(len(pos), int), cell))
+    nb = api.mtp_build_neighbors(model, b)
+    api.mtp_autotune(model, b, nb, "mixed")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    for _ in range(16):
+        api.mtp_autotune(model, b, nb, "mixed")
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 8 << 20
