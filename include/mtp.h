@@ -199,10 +199,10 @@ mtp_status mtp_energy_forces_stress_atoms(mtp_model* model, const mtp_batch* bat
  * module is loaded there, which mtp_load does (so it is taken when a model is created, before
  * a caller's pool grabs the rest of the memory), and it is held until the process exits.
  * Limits: at most 32768 atoms, 524288 pairs and 1024 configuration segments (4096-atom pieces
- * of the configurations), else MTP_ERR_CAPACITY.  Calls no cudaMalloc/cudaFree.  The CUDA
- * runtime still loads each kernel's code on its first launch (lazy loading) unless
- * CUDA_MODULE_LOADING=EAGER; one call of mtp_energy_forces_stress at start-up loads the same
- * kernels.  A device reset invalidates every model (their device memory is gone); a model
+ * of the configurations), else MTP_ERR_CAPACITY.  Calls no cudaMalloc/cudaFree, and mtp_load loads
+ * the code of every kernel that it launches.  It runs the kernels that need no workspace: in FP64
+ * the generic one, in mixed precision the single one, so large systems are slower than through
+ * mtp_energy_forces_stress.  A device reset invalidates every model (their device memory is gone); a model
  * loaded afterwards looks the array up again.  Calls share the array: calls that overlap on the
  * GPU race and must be serialised by the caller. */
 mtp_status mtp_energy_forces_stress_noalloc(mtp_model* model, const mtp_batch* batch, const mtp_nbr* nbr,

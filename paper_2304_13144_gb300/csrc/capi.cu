@@ -929,7 +929,7 @@ mtp_status mtp_load(const mtp_desc* desc, const double* theta, int64_t m, mtp_mo
       upload_theta(md);
       split_prepare(md);
       wide_prepare(md);
-      noalloc_prepare(md->device);
+      noalloc_prepare(md);
       { PinBlock warm(md->pins, 0); }   // (here, not in the first list build)
       md->async_err.ensure(sizeof(unsigned), 0);
       MTP_CUDA(cudaMemset(md->async_err.p, 0, sizeof(unsigned)));

@@ -440,8 +440,14 @@ void run_train_prep(const mtp_nbr* nb, int n_cfg, const double* E, const double*
 void run_sum_rows(const double* part, int nrows, int64_t m, double* out, cudaStream_t s);
 // argument checks shared by the entry points that run the per-neighborhood pass
 void check_run(const mtp_model* m, const mtp_batch* b, const mtp_nbr* nb);
-// loads the allocation-free path's module on `device` (current) and records its scratch address
-void noalloc_prepare(int device);
+// loads the allocation-free path's module on the model's device (current) and records its scratch
+// address; loads the code of the kernels that this path launches for the model
+void noalloc_prepare(const mtp_model* m);
+// the last's parts (a kernel's code is loaded at its first launch or when its attributes are asked
+// for): the generic kernel, the single mixed kernel (false: no shape for the model), the sums
+void load_efs_generic(bool fp64);
+bool load_efs_fast(const mtp_model* m);
+void load_efs_sums();
 int64_t grade_tc_ld(int64_t m);   // row stride of the split parameter rows and of A^-1
 
 }  // namespace mtp

@@ -3,10 +3,10 @@
 // Some callers cannot allocate device memory when they call in: an MD engine or an inference
 // server that owns the whole device-memory budget through its own pool allocator and does not
 // allow foreign allocations, or a time-step loop where an allocation's implicit device
-// synchronisation and its possible failure are not acceptable.  This entry point runs the same
-// kernels as mtp_energy_forces_stress but keeps its scratch (per-pair gradients, per-atom
-// energies and virials, per-segment partial sums) in one file-scope device array of fixed size
-// instead of the model's workspace.  The array belongs to this file's device module: the CUDA
+// synchronisation and its possible failure are not acceptable.  This entry point runs those kernels
+// of the method that need no workspace of their own (in FP64 the generic one, in mixed precision the
+// single one) and keeps its scratch (per-pair gradients, per-atom energies and virials, per-segment
+// partial sums) in one file-scope device array of fixed size instead of the model's workspace.  The array belongs to this file's device module: the CUDA
 // runtime commits it on a device when the module is loaded there, which mtp_load forces (it
 // looks up the array's device address with the model's device current), so the memory is taken
 // when a model is created, not at the first call, and stays until the process exits.  A call on
@@ -64,7 +64,16 @@ void* scratch_address(int device, bool refresh) {
 
 // Called by mtp_load with the model's device current: loads this file's module on the device
 // (committing the scratch array there) and records the array's address.
-void noalloc_prepare(int device) { scratch_address(device, true); }
+// Also loads the code of the kernels that a call launches (the generic kernel in FP64, the single mixed
+// kernel or the generic one in mixed precision, the force gather and the sums): a kernel's first launch
+// would load it, into device memory, and the allocating entry point launches others (the FP64 and the
+// three-kernel passes, which need a workspace).
+void noalloc_prepare(const mtp_model* m) {
+  scratch_address(m->device, true);
+  load_efs_generic(true);
+  if (!load_efs_fast(m)) load_efs_generic(false);
+  load_efs_sums();
+}
 
 }  // namespace mtp
 

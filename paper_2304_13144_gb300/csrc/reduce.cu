@@ -285,6 +285,15 @@ void run_forces(const mtp_nbr* nb, bool fp64, const void* G, double* F, cudaStre
   MTP_CUDA(cudaGetLastError());
 }
 
+void load_efs_sums() {
+  cudaFuncAttributes a;
+  MTP_CUDA(cudaFuncGetAttributes(&a, k_forces));
+  MTP_CUDA(cudaFuncGetAttributes(&a, k_forces_grp<8>));
+  MTP_CUDA(cudaFuncGetAttributes(&a, k_seg_sums<1>));
+  MTP_CUDA(cudaFuncGetAttributes(&a, k_seg_sums<10>));
+  MTP_CUDA(cudaFuncGetAttributes(&a, k_cfg_sums));
+}
+
 size_t config_sums_scratch(const mtp_nbr* nb) { return nb->n_seg * 10 * sizeof(double); }
 
 void run_config_sums(const mtp_nbr* nb, const double* V, const double* Wat, double* E, double* W, DevBuf& tmp,

@@ -441,6 +441,12 @@ int site_max_grid(mtp_model* m, bool fp64, bool tangent) {
 
 bool run_sites_split(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, const SiteOutputs& o, cudaStream_t s);
 
+void load_efs_generic(bool fp64) {
+  cudaFuncAttributes a;
+  if (fp64) MTP_CUDA(cudaFuncGetAttributes(&a, site_kernel<double, double, M_EFS>));
+  else MTP_CUDA(cudaFuncGetAttributes(&a, site_kernel<float, float, M_EFS>));
+}
+
 void run_sites(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, bool fp64, const SiteOutputs& o,
                bool tangent, int* grid_used, cudaStream_t s) {
   m->last_split = false;

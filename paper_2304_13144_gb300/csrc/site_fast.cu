@@ -551,4 +551,21 @@ bool run_sites_fast(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, const S
   return true;
 }
 
+bool load_efs_fast(const mtp_model* m) {
+  const DevSchedule& d = m->ds;
+  if (!d.tri_pk || d.n_q != kNQ) return false;
+  cudaFuncAttributes a;
+  const int nr = d.n_rad, nu0 = d.nu_max;
+  if (nr == 2 && nu0 == 2) MTP_CUDA(cudaFuncGetAttributes(&a, site_fast_kernel<2, 2, F_EFS, false>));
+  else if (nr == 3 && nu0 == 4) MTP_CUDA(cudaFuncGetAttributes(&a, site_fast_kernel<3, 4, F_EFS, false>));
+  else if (nr == 4 && nu0 == 6) MTP_CUDA(cudaFuncGetAttributes(&a, site_fast_kernel<4, 6, F_EFS, false>));
+  else if (nr == 5 && nu0 == 8) {
+    MTP_CUDA(cudaFuncGetAttributes(&a, site_fast_kernel<5, 8, F_EFS, false>));
+    MTP_CUDA(cudaFuncGetAttributes(&a, site_fast_kernel<5, 8, F_EFS, true>));   // (either, by mtp_autotune)
+  } else {
+    return false;
+  }
+  return true;
+}
+
 }  // namespace mtp

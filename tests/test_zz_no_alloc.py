@@ -116,3 +116,33 @@ def test_no_alloc_rejects_systems_beyond_its_fixed_scratch(api):
         api.mtp_energy_forces_stress_noalloc(model, b, nb, "mixed")
     assert e.value.name == "MTP_ERR_CAPACITY"
     assert "32768" in str(e.value) and "segments" in str(e.value)
+
+
+@pytest.mark.parametrize("lev", [8, 20, 22])
+def test_no_alloc_first_call_of_a_process_takes_no_device_memory(native_lib, lev):
+    """In a process of its own: after mtp_load and a list, nothing else has run, and neither precision's
+    first call loads code into device memory."""
+    import os
+    import subprocess
+    import sys
+    code = f"""
+import torch
+from paper_2304_13144_gb300 import api, synth
+desc = api.make_desc(2, {lev})
+model = api.mtp_load(desc, synth.rng(1).normal(0, 0.01, api.mtp_describe(desc)["n_params"]))
+b = api.Batch(synth.concat([synth.fcc_unary_108(), synth.fcc_unary_108(seed=2)]))
+nb = api.mtp_build_neighbors(model, b)
+outs = [torch.empty(s, dtype=torch.float64, device="cuda") for s in (2, 216, 648, 18)]
+torch.cuda.synchronize()
+for prec in (api.MTP_FP64, api.MTP_MIXED):
+    free = torch.cuda.mem_get_info()[0]
+    api._check(api.lib().mtp_energy_forces_stress_noalloc(model.h, api.ctypes.byref(b.c), nb.h, prec,
+                                                           *[api._ptr(t) for t in outs], api._stream()))
+    torch.cuda.synchronize()
+    print("taken", prec, free - torch.cuda.mem_get_info()[0])
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    taken = [int(x.split()[2]) for x in r.stdout.splitlines() if x.startswith("taken")]
+    assert taken == [0, 0], r.stdout
