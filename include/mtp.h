@@ -321,10 +321,14 @@ mtp_status mtp_fit_bfgs(mtp_model* model, const mtp_batch* batch, const mtp_nbr*
  * specialised single-kernel mixed pass, 1, 2, 4 for the generic kernel; blocks per SM then
  * follow from the occupancy) and, for the level-20 shape of the single kernel, with the
  * forward part of the contraction schedule in shared or in global memory; for the mixed path
- * also the three-kernel pass (4 or 8 warps per block of its per-pair kernels) unless mtp_set_mixed_pass fixed the single kernel.  Keeps the fastest in the model for
- * later calls of this precision (with mixed pass 0, also which pass), and returns the single
- * kernel's warps (HOST warps) and the best time of three of the chosen shape (HOST ms) --
- * either may be NULL.  Synchronises `stream`. */
+ * also the three-kernel pass (4 or 8 warps per block of its per-pair kernels) unless
+ * mtp_set_mixed_pass fixed the single kernel.  Where FP64 runs its own pass (one shape), the
+ * generic kernel's shapes are timed for the allocation-free entry point, which still runs it, if
+ * the list is within its limits; else they stay as they were (0: untuned).
+ * Keeps the fastest in the model for later calls of this precision (with mixed pass 0, also which
+ * pass), and returns the single or generic kernel's warps (HOST warps) and the best time of three
+ * of the pass and shape that later calls take (HOST ms) -- either may be NULL.  Synchronises
+ * `stream`. */
 mtp_status mtp_autotune(mtp_model* model, const mtp_batch* batch, const mtp_nbr* nbr,
                         mtp_precision prec, int32_t* warps, double* ms, void* stream);
 

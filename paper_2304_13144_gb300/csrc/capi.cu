@@ -1020,9 +1020,18 @@ mtp_status mtp_autotune(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mt
     float best_ms = 0.f;
     const int keep_pass = md->mixed_pass;
     if (fast && keep_pass != 2) md->mixed_pass = 1;   // the single-kernel shapes first
-    struct Restore { mtp_model* m; int v; ~Restore() { m->mixed_pass = v; } } restore{md, keep_pass};
+    struct Restore {
+      mtp_model* m;
+      int v;
+      ~Restore() { m->mixed_pass = v; m->force_generic = false; }
+    } restore{md, keep_pass};
+    // where the FP64 pass with its one shape serves the call, the shapes of the generic kernel (the
+    // allocation-free entry point's) are timed by themselves, for lists that it takes
+    const bool wide = !fast && md->last_wide;
+    const bool generic = !fast && (!wide || noalloc_takes(nb));
+    md->force_generic = wide;
     // candidate shapes: (forward-slab placement, warps per block); the generic kernel has only warps
-    for (int place = 0; place < (fast ? 2 : 1); ++place) {
+    for (int place = 0; place < (fast ? 2 : (generic ? 1 : 0)); ++place) {
       if (fast) md->tune_fwd_global = place;
       int last_used = -1;
       for (int w = max_w; w >= min_w; --w) {
@@ -1042,6 +1051,19 @@ mtp_status mtp_autotune(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mt
           if (rep == 0 || t < t_min) t_min = t;
         }
         if (best_w == 0 || t_min < best_ms) { best_ms = t_min; best_w = md->last_warps; best_p = place; }
+      }
+    }
+    md->force_generic = false;
+    if (wide) {   // the time of the pass that later calls make
+      run();
+      for (int rep = 0; rep < 3; ++rep) {
+        MTP_CUDA(cudaEventRecord(e0, s));
+        run();
+        MTP_CUDA(cudaEventRecord(e1, s));
+        MTP_CUDA(cudaEventSynchronize(e1));
+        float t = 0.f;
+        MTP_CUDA(cudaEventElapsedTime(&t, e0, e1));
+        if (rep == 0 || t < best_ms) best_ms = t;
       }
     }
     // the three-kernel mixed pass, when the model has one: warps per block of its per-pair
@@ -1074,6 +1096,7 @@ mtp_status mtp_autotune(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, mt
     }
     MTP_CUDA(cudaEventDestroy(e0));
     MTP_CUDA(cudaEventDestroy(e1));
+    if (!fast && !generic) best_w = keep_gen;
     knob = best_w;
     if (fast) md->tune_fwd_global = best_p;
     if (best_sw > 0) {

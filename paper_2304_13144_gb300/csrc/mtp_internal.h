@@ -256,7 +256,8 @@ struct mtp_model {
   // errors of asynchronous kernels (bit 1: a bounded wait of the tensor-core grade expired),
   // allocated and zeroed by mtp_load, OR-ed by the kernels, read and cleared by mtp_sync
   mtp::DevBuf async_err;
-  bool force_generic = false;  // route the mixed path through the generic kernel (cross-checks)
+  bool force_generic = false;  // route every pass through the generic kernel (mtp_autotune)
+  bool last_wide = false;      // the latest pass was the FP64 / dual-number one
   // launch shape of the per-neighborhood kernels: warps per block (0 = largest that fits),
   // chosen by mtp_autotune; last_warps records the shape of the latest launch
   int tune_warps_fast = 0;
@@ -443,6 +444,7 @@ void check_run(const mtp_model* m, const mtp_batch* b, const mtp_nbr* nb);
 // loads the allocation-free path's module on the model's device (current) and records its scratch
 // address; loads the code of the kernels that this path launches for the model
 void noalloc_prepare(const mtp_model* m);
+bool noalloc_takes(const mtp_nbr* nb);   // the list is within its fixed scratch
 // the last's parts (a kernel's code is loaded at its first launch or when its attributes are asked
 // for): the generic kernel, the single mixed kernel (false: no shape for the model), the sums
 void load_efs_generic(bool fp64);

@@ -62,6 +62,10 @@ void* scratch_address(int device, bool refresh) {
 
 }  // namespace
 
+bool noalloc_takes(const mtp_nbr* nb) {
+  return nb->n_atoms <= kMaxAtoms && nb->n_pairs <= kMaxPairs && nb->n_seg <= kMaxSegments;
+}
+
 // Called by mtp_load with the model's device current: loads this file's module on the device
 // (committing the scratch array there) and records the array's address.
 // Also loads the code of the kernels that a call launches (the generic kernel in FP64, the single mixed
@@ -86,7 +90,7 @@ extern "C" mtp_status mtp_energy_forces_stress_noalloc(mtp_model* md, const mtp_
     check_run(md, b, nb);
     if (prec != MTP_FP64 && prec != MTP_MIXED) throw Fail{MTP_ERR_ARG, "unknown precision"};
     if (!energy && !site_energy && !forces && !virial) throw Fail{MTP_ERR_ARG, "no output requested"};
-    if (nb->n_atoms > kMaxAtoms || nb->n_pairs > kMaxPairs || nb->n_seg > kMaxSegments)
+    if (!noalloc_takes(nb))
       throw Fail{MTP_ERR_CAPACITY, "the allocation-free path holds at most " + std::to_string(kMaxAtoms) + " atoms, " +
                                        std::to_string(kMaxPairs) + " pairs and " + std::to_string(kMaxSegments) +
                                        " configuration segments; this call has " + std::to_string(nb->n_atoms) +

@@ -449,7 +449,7 @@ void load_efs_generic(bool fp64) {
 
 void run_sites(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, bool fp64, const SiteOutputs& o,
                bool tangent, int* grid_used, cudaStream_t s) {
-  m->last_split = false;
+  m->last_split = m->last_wide = false;
   if (!fp64 && !tangent && !m->force_generic && run_sites_split(m, b, nb, o, s)) return;
   if (!fp64 && !tangent && !m->force_generic && run_sites_fast(m, b, nb, o, s, false)) return;
   if (!tangent && !m->force_generic && run_sites_wide(m, b, nb, fp64, o, false, 0, nullptr, s)) return;

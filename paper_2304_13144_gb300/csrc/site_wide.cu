@@ -813,7 +813,8 @@ bool run_sites_wide(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, bool fp
   P.words_r = m->wide_words.r;
   P.coef = m->wide_words.coef;
   P.unit = m->wide_words.unit;
-  m->last_fast = false;
+  m->last_fast = m->last_split = false;
+  m->last_wide = true;
   m->last_warps = WPB;
   if (n_part) *n_part = 0;
   if (n_work == 0) return true;

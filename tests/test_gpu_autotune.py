@@ -74,3 +74,39 @@ def test_measured_peaks_are_plausible(api):
     assert nominal32 / 3 < fp32 < nominal32 * 1.05
     assert 0 < fp64 < fp32
     assert 1100.0 / 4 < tf32 < 1100.0 * 1.3
+
+
+def test_fp64_autotune_tunes_the_generic_kernel(api):
+    """FP64 calls run a pass with one shape; the tuned warps are those of the generic kernel, which the
+    allocation-free entry point still runs, and lie in its range.  The time is that of a call."""
+    md = O.OracleModel(2, 12, 2.0, 5.0)
+    nu_sum = [sum(nu for _, nu in labs) for labs, _ in md.basis]
+    nf = [len(labs) for labs, _ in md.basis]
+    theta = synth.draw_theta(106, 2, md.n_rad, md.n_q, nu_sum, nf, 2.0, 5.0, 42.0)
+    model = api.mtp_load(api.make_desc(2, 12), theta)
+    g = synth.rng(107)
+    pos, cell, _ = synth.cubic_supercell(synth._FCC, 3.6, 9)
+    b = api.Batch(synth.single(pos + g.normal(0, 0.1, pos.shape), g.integers(0, 2, len(pos)), cell))
+    nb = api.mtp_build_neighbors(model, b)
+    ref = api.mtp_energy_forces_stress_noalloc(model, b, nb, "fp64")
+    api.mtp_profiler_enable(True)
+    try:
+        api.mtp_profiler_read()
+        w, ms = api.mtp_autotune(model, b, nb, "fp64")
+        timed = api.mtp_profiler_read()
+        api.mtp_energy_forces_stress(model, b, nb, "fp64")
+        call = api.mtp_profiler_read()
+    finally:
+        api.mtp_profiler_enable(False)
+    assert 1 <= w <= 4 and api.mtp_get_launch_shape(model)[2] == w
+    assert "site_efs" in timed and "wide_moments" in timed and "site_efs" not in call
+    sites = sum(t for k, (t, _) in call.items() if k.startswith("wide"))
+    assert 0.5 * sites < ms
+    out = api.mtp_energy_forces_stress_noalloc(model, b, nb, "fp64")
+    for k in ("energy", "forces", "virial"):
+        assert torch.equal(out[k], ref[k]), k
+    # a list that the allocation-free entry point refuses: the shape stays
+    pos, cell, _ = synth.cubic_supercell(synth._FCC, 3.6, 21)
+    b = api.Batch(synth.single(pos, g.integers(0, 2, len(pos)), cell))
+    nb = api.mtp_build_neighbors(model, b)
+    assert api.mtp_autotune(model, b, nb, "fp64")[0] == w and api.mtp_get_launch_shape(model)[2] == w
