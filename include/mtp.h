@@ -11,9 +11,10 @@
  *  - Handles (mtp_model, mtp_nbr) and their scratch are owned by the library and released
  *    by mtp_free_model / mtp_free_nbr.
  *  - Threads and streams: different models are independent.  With one model, builds of different
- *    neighbor lists (mtp_build_neighbors) may run at once, in several threads and streams; the
- *    other calls share the model's scratch, so those with one model (and calls with one list that
- *    is being rebuilt) must be ordered by the caller, on the host and on the GPU.
+ *    neighbor lists (mtp_build_neighbors) and mtp_param_rows may run at once, beside each other and
+ *    beside other calls, in several threads and streams; the other calls share the model's scratch,
+ *    so those with one model (and calls with one list that is being rebuilt) must be ordered by the
+ *    caller, on the host and on the GPU.
  *  - No C++ exception crosses the ABI.  A failing call returns a non-zero mtp_status,
  *    leaves its outputs unspecified and its handles valid; mtp_last_error() gives a
  *    thread-local message for the last failure on this thread.

@@ -86,9 +86,12 @@ bool capturing(cudaStream_t s) {
 }
 }  // namespace
 bool give_back_optional(mtp_model* m, cudaStream_t s) {
-  if (!m || !m->ws_wide.p || m->wide_captured || capturing(s)) return false;
-  MTP_CUDA(cudaDeviceSynchronize());   // (its last pass may have run on another stream)
+  if (!m || m->wide_captured || capturing(s)) return false;
+  std::lock_guard<std::mutex> lk(m->list_mu);
+  if (!m->ws_wide.p && !m->ws_list.p) return false;
+  MTP_CUDA(cudaDeviceSynchronize());   // (the last pass may have run on another stream)
   m->ws_wide.release();
+  m->ws_list.release();
   return true;
 }
 void* PinPool::take() {
@@ -747,6 +750,34 @@ void give_wide(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, int64_t n_wo
   if (!m->wide_captured && capturing(s)) m->wide_captured = true;
 }
 
+// The same for mtp_param_rows, in the workspace of its own, which a call holds from here until its
+// kernels are enqueued; the next call's stream waits for them.  Not under capture, whose replays
+// nothing could order: there the generic kernel runs.
+class ListUse {
+ public:
+  ListUse(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, bool fp64, SiteOutputs& o, cudaStream_t s) : m_(m), s_(s) {
+    const size_t bytes = wide_workspace(m, o.n_list, fp64, false);
+    if (!bytes || capturing(s) || (!fp64 && run_sites_fast(m, b, nb, o, s, true))) return;
+    lk_ = std::unique_lock<std::mutex>(m->list_mu);
+    MTP_CUDA(cudaStreamWaitEvent(s, m->list_done, 0));
+    if (!m->ws_list.try_ensure(bytes, s)) {
+      lk_.unlock();
+      return;
+    }
+    o.wide = m->ws_list.p;
+  }
+  ~ListUse() {
+    if (lk_.owns_lock()) cudaEventRecord(m_->list_done, s_);
+  }
+  ListUse(const ListUse&) = delete;
+  ListUse& operator=(const ListUse&) = delete;
+
+ private:
+  mtp_model* m_;
+  cudaStream_t s_;
+  std::unique_lock<std::mutex> lk_;
+};
+
 // Shared body of the EFS / grade / step entry points.
 void efs_and_grade_once(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp_precision prec, double* energy,
                         double* site_energy, double* forces, double* virial, double threshold, double* gamma,
@@ -931,6 +962,7 @@ mtp_status mtp_load(const mtp_desc* desc, const double* theta, int64_t m, mtp_mo
       wide_prepare(md);
       noalloc_prepare(md);
       { PinBlock warm(md->pins, 0); }   // (here, not in the first list build)
+      MTP_CUDA(cudaEventCreateWithFlags(&md->list_done, cudaEventDisableTiming));
       md->async_err.ensure(sizeof(unsigned), 0);
       MTP_CUDA(cudaMemset(md->async_err.p, 0, sizeof(unsigned)));
       MTP_CUDA(cudaDeviceSynchronize());
@@ -950,8 +982,9 @@ void mtp_free_model(mtp_model* md) {
   cudaDeviceSynchronize();
   for (DevBuf* b : {&md->sched_buf, &md->theta_buf, &md->a_d, &md->ainv_d, &md->ainv_f, &md->ainv_s, &md->ws_pair,
                     &md->ws_atom, &md->ws_rows, &md->ws_grade, &md->ws_sort, &md->ws_misc, &md->ws_red,
-                    &md->err_flag, &md->async_err, &md->split_tab, &md->ws_mom, &md->wide_tab, &md->ws_wide})
+                    &md->err_flag, &md->async_err, &md->split_tab, &md->ws_mom, &md->wide_tab, &md->ws_wide, &md->ws_list})
     b->release();
+  if (md->list_done) cudaEventDestroy(md->list_done);
   delete md;
   cudaSetDevice(cur);
 }
@@ -1548,7 +1581,7 @@ mtp_status mtp_param_rows(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb, 
     o.rows_ld = md->sched.n_params;
     o.atom_list = atoms;
     o.n_list = atoms ? n : nb->n_atoms;
-    give_wide(md, b, nb, o.n_list, prec == MTP_FP64, false, o, as_stream(stream));
+    ListUse use(md, b, nb, prec == MTP_FP64, o, as_stream(stream));
     run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, as_stream(stream));
   });
 }

@@ -294,6 +294,12 @@ struct mtp_model {
     int n_coef = 0, unit = 0;
   } wide_words;
   mtp::DevBuf wide_tab;
+  // the workspace of mtp_param_rows: calls of it may overlap, with each other and with other calls, in
+  // several threads and streams, so it has one of its own, whose users follow one another (list_done:
+  // its last use)
+  std::mutex list_mu;
+  mtp::DevBuf ws_list;
+  cudaEvent_t list_done = nullptr;
   mtp::DevBuf ws_wide;         // its moments / their adjoints
   bool wide_captured = false;  // a stream capture has seen ws_wide: a graph may hold its address
   mtp::DevBuf split_tab;       // slot -> component table of the split pass (uploaded by mtp_load)
@@ -301,11 +307,11 @@ struct mtp_model {
 };
 
 namespace mtp {
-// Gives back the model's workspace of the FP64 / dual-number pass, the largest that a call can do
-// without and that is kept between calls; false where there is none, or where a captured graph may
-// hold its address.
+// Gives back the model's workspaces of the FP64 / dual-number pass, the largest that a call can do
+// without and that are kept between calls; false where there is none, or where a captured graph may
+// hold an address.
 bool give_back_optional(mtp_model* m, cudaStream_t s);
-// Runs `f` (repeatable); where it fails for want of device memory, once more without that workspace.
+// Runs `f` (repeatable); where it fails for want of device memory, once more without them.
 // (Not for list builds, which may run beside a call that uses it.)
 template <class F>
 void with_memory(mtp_model* m, cudaStream_t s, F&& f) {

@@ -69,3 +69,62 @@ def test_lists_built_at_once_with_one_model(native_lib):
             ex = api.mtp_nbr_export(got[t][e], b)
             for k in ("off", "j", "img", "r"):
                 assert torch.equal(ex[k], ref[t][e][k]), (t, e, k)
+
+
+@pytest.mark.parametrize("prec,lev", [("fp64", 12), ("mixed", 24)])
+def test_parameter_rows_at_once_with_one_model(native_lib, prec, lev):
+    """Threads take rows of lists of their own sizes (growing and shrinking the workspace), each on its
+    stream, while another runs energies and forces: the rows of every call are those of a call alone."""
+    from oracle import oracle as O
+    from paper_2304_13144_gb300 import api
+    types = 2
+    md = O.OracleModel(types, lev, 2.0, 5.0)
+    nu_sum = [sum(nu for _, nu in labs) for labs, _ in md.basis]
+    theta = synth.draw_theta(5, types, md.n_rad, 8, nu_sum, [len(labs) for labs, _ in md.basis], 2.0, 5.0, 42.0)
+    g = synth.rng(78)
+    pos, cell, _ = synth.cubic_supercell(synth._FCC, 3.6, 6)
+    b = api.Batch(synth.single(pos + g.normal(0, 0.1, pos.shape), g.integers(0, types, len(pos)), cell))
+    model = api.mtp_load(api.make_desc(types, lev), theta)
+    nb = api.mtp_build_neighbors(model, b)
+    forces = api.mtp_energy_forces_stress(model, b, nb, prec)["forces"]
+    lists = [[torch.tensor(g.integers(0, b.n_atoms, n), device="cuda") for n in sizes]
+             for sizes in ((5, 700, 40), (864, 1, 300), (64, 900, 7))]
+    ref = [[api.mtp_param_rows(model, b, nb, prec, a).clone() for a in ls] for ls in lists]
+    model = api.mtp_load(api.make_desc(types, lev), theta)     # (no workspace yet)
+    torch.cuda.synchronize()
+    errors = []
+    start = threading.Barrier(len(lists) + 1)
+
+    def rows(t):
+        try:
+            s = torch.cuda.Stream()
+            start.wait()
+            with torch.cuda.stream(s):
+                for k in range(20):
+                    got = [api.mtp_param_rows(model, b, nb, prec, a) for a in lists[t]]
+                    s.synchronize()
+                    for x, y in zip(got, ref[t]):
+                        if not torch.equal(x, y):
+                            errors.append(f"thread {t}, pass {k}: rows differ")
+        except Exception as e:
+            errors.append(f"thread {t}: {e!r}")
+
+    def energies():
+        try:
+            s = torch.cuda.Stream()
+            start.wait()
+            with torch.cuda.stream(s):
+                for k in range(40):
+                    f = api.mtp_energy_forces_stress(model, b, nb, prec)["forces"]
+                    s.synchronize()
+                    if not torch.equal(f, forces):
+                        errors.append("forces differ")
+        except Exception as e:
+            errors.append(repr(e))
+
+    threads = [threading.Thread(target=rows, args=(t,)) for t in range(len(lists))] + [threading.Thread(target=energies)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[:5]
