@@ -352,7 +352,7 @@ mtp_status mtp_set_mixed_pass(mtp_model* model, int pass);
 
 /* Launch shape of the three-kernel pass: warps per block of its per-pair kernels (4 or 8; 0 =
  * default 8; what mtp_autotune sets).  The others, all 0, run the grouped contraction (four
- * neighborhoods side by side, fastest at every level); any of them set asks for the contraction
+ * neighborhoods side by side, two to four times as fast); any of them set asks for the contraction
  * with 1 or 2 neighborhoods per warp (0 = 1), 2 or 4 schedule words per step per lane, or 8 with
  * two neighborhoods per warp (0 = 2), and its schedule read from 1 = shared memory; 2 = global
  * memory, streamed through a shared-memory ring, the block's warps in step; 3 = tensor memory, the

@@ -14,8 +14,8 @@
 //   What bounded it: three launches per column (1,955 at m = 651) and a thread per column of the
 // inverse walking m^2 dependent steps.  Now the panels (1.3 of 3.2 ms: a pivot chain of about 2 us
 // per column, and FP64 at 2 FMAs per clock in the one SM; pivots are compared as integers, FP64
-// comparisons alone took twice that) and 123 dependent launches.  A^-1 at m = 651: 44.2 -> 3.26 ms,
-// m = 222: 6.3 -> 0.9, m = 1,636: 271 -> 18.5.
+// comparisons alone took twice that) and 174 dependent launches.  A^-1 at m = 651: 44.2 -> 3.14 ms,
+// m = 222: 6.3 -> 0.86, m = 1,636: 271 -> 18.3.
 // The grade product C = B A^-1 is fused with its row epilogue (max |C_ip| and the lowest p
 // attaining it), so C is never written.  This SIMT kernel serves small active sets; the mixed path
 // uses the tensor-core kernel in grade_tc.cu, the FP64 path the one in grade_fp64.cu.
@@ -40,7 +40,7 @@ __global__ void k_maxabs(const double* A, int64_t n, unsigned long long* out) {
   if ((threadIdx.x & 31) == 0) atomicMax(out, static_cast<unsigned long long>(__double_as_longlong(v)));
 }
 
-constexpr int kPanel = 16;   // columns per panel (m = 651: 8 columns 3.31 ms, 16 3.24; m = 222: 0.56, 0.52)
+constexpr int kPanel = 16;   // columns per panel (m = 651: 8 columns 3.31 ms, 16 3.24)
 constexpr int kBack = 32;    // rows per step of the back substitution
 constexpr int kPanelRows = 2048;   // rows a panel's block holds in registers
 

@@ -407,10 +407,11 @@ extern std::atomic<int> g_inject_grade_wait;
 extern std::atomic<int> g_inject_maxvol_wait;
 bool take_injected(std::atomic<int>& c);
 // Warps per group of the grouped contraction (site_group.cu), by how many groups' arrays fit an SM:
-// 16 at level 16 and below (a warp each), 6 at level 20, 1 at level 24.  Measured, ms per pass:
-// level 16, 128,000 atoms: 1 warp 0.215, 2 warps 0.238; level 20, 1,048,576 atoms: 1 warp 11.9,
+// 1 at level 16 and below (16 groups), 3 at level 20 (6 groups), 12 at level 24 (one).  Measured, ms per
+// pass: level 16, 128,000 atoms: 1 warp 0.215, 2 warps 0.238; level 20, 1,048,576 atoms: 1 warp 11.9,
 // 2 warps 8.26, 3 warps 7.37, 4 warps 7.62 (latency hidden against waves of a few rounds only);
-// level 24, 131,072 atoms: 8 warps 6.50, 12 warps 5.72, 16 warps 5.64 (128 registers).
+// level 24, 131,072 atoms: 8 warps 6.50, 12 warps 5.70, 16 warps 5.64 (8,192 atoms 0.385, 0.380: 1 % for
+// a third more warps, which no longer wait for latency; 12 leave a thread 168 registers, 16 128).
 constexpr int kGroupWarpsSmall = 1, kGroupWarpsMid = 3, kGroupWarpsLarge = 12;
 constexpr int kGroupPad = 4;   // rows of padding after each warp's word stream (grouped contraction)
 // per-neighborhood value slots of the specialised kernel's shared-memory arrays: the values,

@@ -533,9 +533,9 @@ __device__ __forceinline__ int nth_set_bit(uint32_t m, int rem) {   // position 
   return pos;
 }
 
-// MINB blocks per SM: bound by the latency of dependent loads, so large lists take 8 at 32 registers
-// (1,048,576 atoms 1.55 ms with 4 blocks, 1.46 with 6, 1.42 with 8), lists that do not fill the GPU
-// 4 at 64 (4,000 atoms 13 us against 17)
+// MINB blocks per SM: bound by the latency of dependent loads, so large lists take 8 at 32 registers,
+// lists that do not fill the GPU 4 at 64.  The region, 4 against 8 blocks, us: 4,000 atoms 14.7, 17.0;
+// 32,000 49.7, 53.2; 65,536 96.2, 100.7; 78,732 113.0, 113.8; 128,000 193.8, 187.4; 1,048,576 1,550, 1,418
 template <int MINB>
 __global__ void __launch_bounds__(256, MINB) k_fill_warp(NbrArgs A) {
   const unsigned full = 0xffffffffu;
@@ -749,95 +749,97 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
   if (N >= (int64_t(1) << 31)) throw Fail{MTP_ERR_UNSUPPORTED, "more than 2^31 atoms"};
   const double rc = m->desc.r_cut;
   // the plan of these cells, kept in the list while offsets, cells and periodicity stay the same
-  // values (a constant-volume run): a comparison instead of the loop below and four uploads
-  const bool same = nb->plan_valid && nb->plan_rc == rc && nb->atom_offset == ao && nb->plan_cell == cell && nb->plan_pbc == pbc;
+  // values: a comparison instead of the loop below and four uploads.  (Constant volume; a run whose
+  // cell changes from step to step makes its plan each time.)
+  const bool same = nb->plan_valid && nb->plan_rc == rc && nb->atom_offset == ao && nb->plan_cell == cell &&
+                    nb->plan_pbc == pbc;
   long long bins = nb->n_bins_total;
   size_t n_shift = nb->plan_shifts;
   int max_scan = nb->plan_max_scan;
   if (!same) {
-  nb->plan_valid = false;
-  std::vector<DevCfg> cfgs(n_cfg);
-  std::vector<float4> shi, slo;
-  bins = 0;
-  nb->seg_host.clear();
-  for (int k = 0; k < n_cfg; ++k) {
-    DevCfg& C = cfgs[k];
-    const double* H = &cell[9 * k];
-    for (int q = 0; q < 9; ++q) C.H[q] = H[q];
-    double c0[3] = {H[4] * H[8] - H[5] * H[7], H[5] * H[6] - H[3] * H[8], H[3] * H[7] - H[4] * H[6]};
-    double c1[3] = {H[7] * H[2] - H[8] * H[1], H[8] * H[0] - H[6] * H[2], H[6] * H[1] - H[7] * H[0]};
-    double c2[3] = {H[1] * H[5] - H[2] * H[4], H[2] * H[3] - H[0] * H[5], H[0] * H[4] - H[1] * H[3]};
-    const double vol = H[0] * c0[0] + H[1] * c0[1] + H[2] * c0[2];
-    if (!(std::fabs(vol) > 1e-9) || !std::isfinite(vol)) throw Fail{MTP_ERR_GEOMETRY, "degenerate cell"};
-    for (int c = 0; c < 3; ++c) { C.Hinv[c * 3 + 0] = c0[c] / vol; C.Hinv[c * 3 + 1] = c1[c] / vol; C.Hinv[c * 3 + 2] = c2[c] / vol; }
-    const double* cc[3] = {c0, c1, c2};
-    int Kmax = 0;
-    for (int a = 0; a < 3; ++a) {
-      const double h = std::fabs(vol) / std::sqrt(cc[a][0] * cc[a][0] + cc[a][1] * cc[a][1] + cc[a][2] * cc[a][2]);
-      C.pbc[a] = pbc[3 * k + a] ? 1 : 0;
-      int n = static_cast<int>(std::floor(h / rc));
-      n = std::max(1, std::min(n, 1024));
-      C.nb[a] = n;
-      C.kb[a] = static_cast<int>(std::ceil(rc * n / h - 1e-12));
-      if (!C.pbc[a]) C.kb[a] = std::min(C.kb[a], n);
-      if (C.pbc[a]) Kmax = std::max(Kmax, (C.kb[a] + n - 1) / n + 1);
-      if (C.kb[a] > 64) throw Fail{MTP_ERR_GEOMETRY, "cell too thin for the cut-off (more than 64 images)"};
-    }
-    C.K = Kmax;
-    {
-      const int v1 = 2 * C.kb[1] + 1, v2 = 2 * C.kb[2] + 1, ns = (2 * C.kb[0] + 1) * v1 * v2;
-      for (int q = 0; q < 32; ++q)
-        C.qd[q] = q < ns ? ((q / (v1 * v2) - C.kb[0] + 64) | (((q / v2) % v1 - C.kb[1] + 64) << 8) |
-                            ((q % v2 - C.kb[2] + 64) << 16))
-                         : 0;
-    }
-    C.bin_base = bins;
-    bins += static_cast<long long>(C.nb[0]) * C.nb[1] * C.nb[2];
-    C.shift_base = static_cast<long long>(shi.size());
-    for (int n0 = -Kmax; n0 <= Kmax; ++n0)
-      for (int n1 = -Kmax; n1 <= Kmax; ++n1)
-        for (int n2 = -Kmax; n2 <= Kmax; ++n2) {
-          float hh[3], ll[3];
-          for (int c = 0; c < 3; ++c) {
-            const double v = n0 * H[0 * 3 + c] + n1 * H[1 * 3 + c] + n2 * H[2 * 3 + c];
-            hh[c] = static_cast<float>(v);
-            ll[c] = static_cast<float>(v - static_cast<double>(hh[c]));
+    nb->plan_valid = false;
+    std::vector<DevCfg> cfgs(n_cfg);
+    std::vector<float4> shi, slo;
+    bins = 0;
+    nb->seg_host.clear();
+    for (int k = 0; k < n_cfg; ++k) {
+      DevCfg& C = cfgs[k];
+      const double* H = &cell[9 * k];
+      for (int q = 0; q < 9; ++q) C.H[q] = H[q];
+      double c0[3] = {H[4] * H[8] - H[5] * H[7], H[5] * H[6] - H[3] * H[8], H[3] * H[7] - H[4] * H[6]};
+      double c1[3] = {H[7] * H[2] - H[8] * H[1], H[8] * H[0] - H[6] * H[2], H[6] * H[1] - H[7] * H[0]};
+      double c2[3] = {H[1] * H[5] - H[2] * H[4], H[2] * H[3] - H[0] * H[5], H[0] * H[4] - H[1] * H[3]};
+      const double vol = H[0] * c0[0] + H[1] * c0[1] + H[2] * c0[2];
+      if (!(std::fabs(vol) > 1e-9) || !std::isfinite(vol)) throw Fail{MTP_ERR_GEOMETRY, "degenerate cell"};
+      for (int c = 0; c < 3; ++c) { C.Hinv[c * 3 + 0] = c0[c] / vol; C.Hinv[c * 3 + 1] = c1[c] / vol; C.Hinv[c * 3 + 2] = c2[c] / vol; }
+      const double* cc[3] = {c0, c1, c2};
+      int Kmax = 0;
+      for (int a = 0; a < 3; ++a) {
+        const double h = std::fabs(vol) / std::sqrt(cc[a][0] * cc[a][0] + cc[a][1] * cc[a][1] + cc[a][2] * cc[a][2]);
+        C.pbc[a] = pbc[3 * k + a] ? 1 : 0;
+        int n = static_cast<int>(std::floor(h / rc));
+        n = std::max(1, std::min(n, 1024));
+        C.nb[a] = n;
+        C.kb[a] = static_cast<int>(std::ceil(rc * n / h - 1e-12));
+        if (!C.pbc[a]) C.kb[a] = std::min(C.kb[a], n);
+        if (C.pbc[a]) Kmax = std::max(Kmax, (C.kb[a] + n - 1) / n + 1);
+        if (C.kb[a] > 64) throw Fail{MTP_ERR_GEOMETRY, "cell too thin for the cut-off (more than 64 images)"};
+      }
+      C.K = Kmax;
+      {
+        const int v1 = 2 * C.kb[1] + 1, v2 = 2 * C.kb[2] + 1, ns = (2 * C.kb[0] + 1) * v1 * v2;
+        for (int q = 0; q < 32; ++q)
+          C.qd[q] = q < ns ? ((q / (v1 * v2) - C.kb[0] + 64) | (((q / v2) % v1 - C.kb[1] + 64) << 8) |
+                              ((q % v2 - C.kb[2] + 64) << 16))
+                           : 0;
+      }
+      C.bin_base = bins;
+      bins += static_cast<long long>(C.nb[0]) * C.nb[1] * C.nb[2];
+      C.shift_base = static_cast<long long>(shi.size());
+      for (int n0 = -Kmax; n0 <= Kmax; ++n0)
+        for (int n1 = -Kmax; n1 <= Kmax; ++n1)
+          for (int n2 = -Kmax; n2 <= Kmax; ++n2) {
+            float hh[3], ll[3];
+            for (int c = 0; c < 3; ++c) {
+              const double v = n0 * H[0 * 3 + c] + n1 * H[1 * 3 + c] + n2 * H[2 * 3 + c];
+              hh[c] = static_cast<float>(v);
+              ll[c] = static_cast<float>(v - static_cast<double>(hh[c]));
+            }
+            shi.push_back(make_float4(hh[0], hh[1], hh[2], 0.f));
+            slo.push_back(make_float4(ll[0], ll[1], ll[2], 0.f));
           }
-          shi.push_back(make_float4(hh[0], hh[1], hh[2], 0.f));
-          slo.push_back(make_float4(ll[0], ll[1], ll[2], 0.f));
-        }
-    C.rc2 = rc * rc;
-    C.rc2f = static_cast<float>(rc * rc);
-    C.rcm2f = static_cast<float>((rc + 1e-3) * (rc + 1e-3));
-    for (int64_t a0 = ao[k]; a0 < ao[k + 1]; a0 += 4096) {
-      nb->seg_host.push_back(k);
-      nb->seg_host.push_back(a0);
-      nb->seg_host.push_back(std::min<int64_t>(a0 + 4096, ao[k + 1]));
+      C.rc2 = rc * rc;
+      C.rc2f = static_cast<float>(rc * rc);
+      C.rcm2f = static_cast<float>((rc + 1e-3) * (rc + 1e-3));
+      for (int64_t a0 = ao[k]; a0 < ao[k + 1]; a0 += 4096) {
+        nb->seg_host.push_back(k);
+        nb->seg_host.push_back(a0);
+        nb->seg_host.push_back(std::min<int64_t>(a0 + 4096, ao[k + 1]));
+      }
     }
-  }
-  nb->n_cfg = n_cfg;
-  nb->atom_offset = ao;
-  nb->n_bins_total = bins;
-  nb->n_seg = static_cast<int64_t>(nb->seg_host.size() / 3);
-  // device buffers
-  nb->plan.ensure(cfgs.size() * sizeof(DevCfg) + 2 * shi.size() * sizeof(float4) + 64, s);
-  DevCfg* d_cfg = nb->plan.as<DevCfg>();
-  float4* d_shi = reinterpret_cast<float4*>(reinterpret_cast<char*>(d_cfg) + ((cfgs.size() * sizeof(DevCfg) + 15) & ~size_t(15)));
-  float4* d_slo = d_shi + shi.size();
-  MTP_CUDA(cudaMemcpyAsync(d_cfg, cfgs.data(), cfgs.size() * sizeof(DevCfg), cudaMemcpyHostToDevice, s));
-  MTP_CUDA(cudaMemcpyAsync(d_shi, shi.data(), shi.size() * sizeof(float4), cudaMemcpyHostToDevice, s));
-  MTP_CUDA(cudaMemcpyAsync(d_slo, slo.data(), slo.size() * sizeof(float4), cudaMemcpyHostToDevice, s));
-  nb->seg.ensure(nb->seg_host.size() * sizeof(int64_t), s);
-  MTP_CUDA(cudaMemcpyAsync(nb->seg.p, nb->seg_host.data(), nb->seg_host.size() * sizeof(int64_t),
-                           cudaMemcpyHostToDevice, s));
-  max_scan = 0;
-  for (const DevCfg& C : cfgs) max_scan = std::max(max_scan, (2 * C.kb[0] + 1) * (2 * C.kb[1] + 1) * (2 * C.kb[2] + 1));
-  n_shift = shi.size();
-  nb->plan_shifts = n_shift;
-  nb->plan_max_scan = max_scan;
-  nb->plan_rc = rc;
-  nb->plan_cell = cell;
-  nb->plan_pbc = pbc;
+    nb->n_cfg = n_cfg;
+    nb->atom_offset = ao;
+    nb->n_bins_total = bins;
+    nb->n_seg = static_cast<int64_t>(nb->seg_host.size() / 3);
+    // device buffers
+    nb->plan.ensure(cfgs.size() * sizeof(DevCfg) + 2 * shi.size() * sizeof(float4) + 64, s);
+    DevCfg* d_cfg = nb->plan.as<DevCfg>();
+    float4* d_shi = reinterpret_cast<float4*>(reinterpret_cast<char*>(d_cfg) + ((cfgs.size() * sizeof(DevCfg) + 15) & ~size_t(15)));
+    float4* d_slo = d_shi + shi.size();
+    MTP_CUDA(cudaMemcpyAsync(d_cfg, cfgs.data(), cfgs.size() * sizeof(DevCfg), cudaMemcpyHostToDevice, s));
+    MTP_CUDA(cudaMemcpyAsync(d_shi, shi.data(), shi.size() * sizeof(float4), cudaMemcpyHostToDevice, s));
+    MTP_CUDA(cudaMemcpyAsync(d_slo, slo.data(), slo.size() * sizeof(float4), cudaMemcpyHostToDevice, s));
+    nb->seg.ensure(nb->seg_host.size() * sizeof(int64_t), s);
+    MTP_CUDA(cudaMemcpyAsync(nb->seg.p, nb->seg_host.data(), nb->seg_host.size() * sizeof(int64_t),
+                             cudaMemcpyHostToDevice, s));
+    max_scan = 0;
+    for (const DevCfg& C : cfgs) max_scan = std::max(max_scan, (2 * C.kb[0] + 1) * (2 * C.kb[1] + 1) * (2 * C.kb[2] + 1));
+    n_shift = shi.size();
+    nb->plan_shifts = n_shift;
+    nb->plan_max_scan = max_scan;
+    nb->plan_rc = rc;
+    nb->plan_cell = cell;
+    nb->plan_pbc = pbc;
   }
   nb->n_atoms = N;
   DevCfg* d_cfg = nb->plan.as<DevCfg>();

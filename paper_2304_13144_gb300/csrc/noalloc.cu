@@ -3,17 +3,17 @@
 // Some callers cannot allocate device memory when they call in: an MD engine or an inference
 // server that owns the whole device-memory budget through its own pool allocator and does not
 // allow foreign allocations, or a time-step loop where an allocation's implicit device
-// synchronisation and its possible failure are not acceptable.  This entry point runs those kernels
-// of the method that need no workspace of their own (in FP64 the generic one, in mixed precision the
-// single one) and keeps its scratch (per-pair gradients, per-atom energies and virials, per-segment
-// partial sums) in one file-scope device array of fixed size instead of the model's workspace.  The array belongs to this file's device module: the CUDA
-// runtime commits it on a device when the module is loaded there, which mtp_load forces (it
-// looks up the array's device address with the model's device current), so the memory is taken
-// when a model is created, not at the first call, and stays until the process exits.  A call on
-// a device where no model was loaded since the last device reset looks the address up itself,
-// so that first call should come before any stream capture.  All calls share the one array:
-// calls whose work overlaps on the GPU (other streams, other threads) race on it and must be
-// serialised by the caller.
+// synchronisation and its possible failure are not acceptable.  This entry point runs those
+// kernels of the method that need no workspace of their own (in FP64 the generic one, in mixed
+// precision the single one) and keeps its scratch (per-pair gradients, per-atom energies and
+// virials, per-segment partial sums) in one file-scope device array of fixed size instead of the
+// model's workspace.  The array belongs to this file's device module: the CUDA runtime commits it
+// on a device when the module is loaded there, which mtp_load forces (it looks up the array's
+// device address with the model's device current), so the memory is taken when a model is created,
+// not at the first call, and stays until the process exits.  A call on a device where no model was
+// loaded since the last device reset looks the address up itself, so that first call should come
+// before any stream capture.  All calls share the one array: calls whose work overlaps on the GPU
+// (other streams, other threads) race on it and must be serialised by the caller.
 #include <cuda_runtime.h>
 
 #include <algorithm>

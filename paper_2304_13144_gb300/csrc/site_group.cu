@@ -15,9 +15,10 @@
 // level 24 one group takes 123 KB.  The schedule's words are read from tensor memory at level 20
 // (70 KB), shared memory below, and at level 24 (0.35 MB) from L2 a step ahead.
 //
-// Per pass, before (k_contract, its default shape) and now: level 20, 1,048,576 atoms 15.3 ->
-// 7.37 ms (tensor-memory shape of k_contract: 13.1); level 16, 128,000 atoms 0.491 -> 0.215;
-// level 24, 131,072 atoms 21.2 -> 5.72 ms.
+// Per pass, before (k_contract, its default shape, words ordered for its 32-bit loads) and now: level
+// 20, 1,048,576 atoms 15.3 -> 7.37 ms (tensor-memory shape of k_contract: 13.1); level 16, 128,000
+// atoms 0.491 -> 0.215; level 24, 131,072 atoms 21.2 -> 5.72 ms.  With the words in this kernel's
+// order k_contract's shapes take 1 to 8 % more (0.498 at level 16, 23.0 at level 24).
 //
 // The terms of a destination, their order and the two accumulator chains (row parity) are those
 // of k_contract (site_split.cu), whose packed rounds this kernel walks: the results are bitwise

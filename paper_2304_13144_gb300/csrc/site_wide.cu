@@ -21,12 +21,13 @@
 //   FP64 energies, forces, rows, level 20, 16,384 atoms      14.1 -> 4.44 ms (1.21 + 1.60 + 1.63)
 //   FP64 energies and forces, level 8, 256,000 atoms         17.3 -> 6.60
 //   the same, level 24, 16,384 atoms of the liquid           83.9 -> 14.7
-//   FP64 training step, level 16, 34,968 atoms (both passes) 34.6 -> 11.1
-//   mixed training step of the same size (FP32 tangent)      3.58 -> 1.66
+//   FP64 training step, level 16, 512 cells (both passes)    32.5 -> 11.3
+//   mixed training step of the same cells (FP32 tangent)     3.58 -> 1.66
 // At level 20 the FP64 pipe would take 2.8 ms for the operations that remain.
 //
-// The order of every sum is fixed by the neighbor list, so the results do not depend on the launch
-// shape.
+// The order of every sum over pairs and terms is fixed by the neighbor list, whatever the launch shape.
+// The tangent's sums over atoms go to a row per warp or group first, so their order follows the grid
+// (the SMs of the device and the number of atoms): the same from call to call.
 #include <algorithm>
 #include <string>
 #include <type_traits>
@@ -65,7 +66,6 @@ struct WideArgs {
   int unit;                  // the coefficient index of 1
   int nbw;                   // neighborhoods per warp (per-pair kernels)
   int pb;                    // pairs per monomial batch (moments)
-  int64_t part_rows;         // tangent: rows of partial sums
   // contraction: warps per neighborhood and neighborhoods per block
   int cw, cg;
   size_t warp_bytes, c_bytes;
