@@ -159,6 +159,15 @@ inline __host__ __device__ float tf32_rn(float x) {
 #endif
 }
 
+constexpr size_t kMaxSmem = 227 * 1024;   // shared memory a block may take
+// Lets `kern` take dynamic shared memory up to what a block has beside its static arrays: always the
+// same value, whatever this launch takes, since the attribute belongs to the kernel and another
+// thread's launch may fall between this call and the caller's.
+template <class K>
+void allow_smem(K kern, size_t static_bytes = 0) {
+  MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxSmem - static_bytes)));
+}
+
 #ifdef __CUDACC__
 // |v| as an integer with the order of the absolute values (FP64 comparisons take the slow pipe);
 // NaN sorts below everything

@@ -914,7 +914,7 @@ void build_neighbors(mtp_model* m, const mtp_batch* b, mtp_nbr* nb, cudaStream_t
     if (small) {
       const size_t smem = (2 * static_cast<size_t>(bins) + 1 + N) * sizeof(int);
       if (smem > 48 * 1024)
-        MTP_CUDA(cudaFuncSetAttribute(k_bin_small, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        allow_smem(k_bin_small, 32 * sizeof(int));
       k_bin_small<<<1, 1024, smem, s>>>(A, static_cast<int>(bins));
       ProfRegion::launched();
       MTP_CUDA(cudaGetLastError());

@@ -406,8 +406,7 @@ int launch_sites(const SiteParams& P0, int* grid_used, cudaStream_t s) {
   if (P.L.total > 227 * 1024)
     throw Fail{MTP_ERR_UNSUPPORTED, "model too large for the per-neighborhood kernel's shared memory"};
   auto kern = site_kernel<S, R, MODE>;
-  MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(P.L.total)));
+  allow_smem(kern);
   int dev = 0, nsm = 0, per_sm = 0;
   MTP_CUDA(cudaGetDevice(&dev));
   MTP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));

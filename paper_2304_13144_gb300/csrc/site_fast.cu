@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(kMaxWarpsF * 32, 1) site_fast_kernel(FastParam
 template <int NR, int NU0, int MODE, bool FG>
 void launch_fast(FastParams P, int nwarps, cudaStream_t s) {
   auto kern = site_fast_kernel<NR, NU0, MODE, FG>;
-  MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(P.total)));
+  allow_smem(kern);
   int dev = 0, nsm = 0, per_sm = 0;
   MTP_CUDA(cudaGetDevice(&dev));
   MTP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));

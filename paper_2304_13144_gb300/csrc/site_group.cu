@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_contract_group(GroupArgs P) {
   }
 }
 
-constexpr size_t kSmem = 227 * 1024;
+constexpr size_t kSmem = kMaxSmem - 16;
 constexpr int kU = 4;   // words per step (the word stream has kGroupPad >= kU rows past its last round)
 static_assert(kU <= kGroupPad, "a step reads up to kU rows past the last round");
 
@@ -400,7 +400,7 @@ void launch(K kern, Plan& pl, int grid, cudaStream_t s) {
   // a block that holds the tensor-memory columns takes more than half the shared memory, so that
   // no second block shares its SM (it would wait for the columns)
   if (pl.src == SRC_TMEM) pl.smem = std::max<size_t>(pl.smem, 120 * 1024);
-  MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pl.smem)));
+  allow_smem(kern, 16);   // (its tensor-memory address)
   ProfRegion pr("site_contract", s);
   kern<<<grid, pl.groups * pl.P.d.group_warps * 32, pl.smem, s>>>(pl.P);
   ProfRegion::launched();

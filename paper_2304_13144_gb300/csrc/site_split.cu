@@ -1190,7 +1190,7 @@ int launch_split(SplitArgs P, int warps_pair, int nb_contract, int unroll, int s
   {
     const size_t smem = P.c_bytes + static_cast<size_t>(warps_pair) * GPW * stage_f4(NR) * BATCH * sizeof(float4);
     auto kern = k_moments<NR, NU0>;
-    MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    allow_smem(kern);
     const int per = blocks_per_sm(kern, warps_pair * 32, smem);
     const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((groups + warps_pair - 1) / warps_pair,
                                                                               static_cast<int64_t>(nsm) * per)));
@@ -1213,7 +1213,7 @@ int launch_split(SplitArgs P, int warps_pair, int nb_contract, int unroll, int s
       // a block that holds all 512 tensor-memory columns: more than half the shared memory, so
       // that no second block shares its SM (it would wait for the columns)
       if (sch == 3) sm = std::max<size_t>(sm, 120 * 1024);
-      MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm)));
+      allow_smem(kern, 16);   // (its tensor-memory address)
       const int per = blocks_per_sm(kern, warps * 32, sm);
       const int64_t need = (P.n_work + nb_contract - 1) / nb_contract;
       const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((need + warps - 1) / warps,
@@ -1255,7 +1255,7 @@ int launch_split(SplitArgs P, int warps_pair, int nb_contract, int unroll, int s
     const size_t gstride = static_cast<size_t>(adj_region(Slices<NR, NU0>::FLOATS, rows));
     const size_t smem = P.c_bytes + static_cast<size_t>(warps_pair) * GPW * gstride * sizeof(float);
     auto go = [&](auto kern) {
-      MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+      allow_smem(kern);
       const int per = blocks_per_sm(kern, warps_pair * 32, smem);
       const int grid = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>((groups + warps_pair - 1) / warps_pair,
                                                                                 static_cast<int64_t>(nsm) * per)));

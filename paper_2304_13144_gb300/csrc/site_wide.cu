@@ -623,7 +623,7 @@ int64_t launch_warps(K kern, WideArgs P, size_t warp_bytes, int64_t tasks, int64
   while (warps > 1 && P.c_bytes + warps * warp_bytes > kSmem) --warps;
   const size_t smem = P.c_bytes + warps * warp_bytes;
   P.warp_bytes = warp_bytes;
-  MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+  allow_smem(kern);
   int per = 0;
   MTP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, warps * 32, smem));
   int64_t grid = std::min<int64_t>((tasks + warps - 1) / warps, static_cast<int64_t>(num_sms()) * std::max(per, 1));
@@ -697,7 +697,7 @@ void launch_wide(const mtp_model* m, WideArgs P, int64_t max_part, int64_t* n_pa
     C.cw = C.cg >= 6 ? 1 : (C.cg >= 4 ? 2 : (C.cg >= 2 ? 4 : 12));
     const size_t smem = C.c_bytes + C.cg * C.warp_bytes;
     auto kern = k_wide_contract<S, R, MODE>;
-    MTP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    allow_smem(kern);
     int per = 0;
     MTP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, C.cg * C.cw * 32, smem));
     int64_t grid = std::min<int64_t>((P.n_work + C.cg - 1) / C.cg, static_cast<int64_t>(nsm) * std::max(per, 1));

@@ -128,3 +128,36 @@ def test_parameter_rows_at_once_with_one_model(native_lib, prec, lev):
     for t in threads:
         t.join()
     assert not errors, errors[:5]
+
+
+def test_lists_of_different_shared_memory_built_at_once(native_lib):
+    """One-block binning takes 57 KB of shared memory for one of these dilute gases and 87 KB for the
+    other: neither thread's launches may find the kernel limited to the other's."""
+    from paper_2304_13144_gb300 import api
+    desc = api.make_desc(1, 4)
+    model = api.mtp_load(desc, np.zeros(api.mtp_describe(desc)["n_params"]))
+    g = synth.rng(79)
+    batches = [api.Batch(synth.single(g.uniform(0, L, (n, 3)), np.zeros(n, int), L * np.eye(3)))
+               for n, L in ((8000, 95.5), (6000, 80.5))]
+    pairs = [api.mtp_build_neighbors(model, b).size()[1] for b in batches]
+    torch.cuda.synchronize()
+    errors = []
+    start = threading.Barrier(2)
+
+    def build(t):
+        s = torch.cuda.Stream()
+        nb = None
+        start.wait()
+        try:
+            for k in range(400):
+                nb = api.mtp_build_neighbors(model, batches[t], nb, stream=s)
+                assert nb.size()[1] == pairs[t]
+        except Exception as e:
+            errors.append(f"thread {t}, build {k}: {e!r}")
+
+    threads = [threading.Thread(target=build, args=(t,)) for t in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
