@@ -174,10 +174,12 @@ def fail_growth(api, after, call):
 
 
 def test_without_memory_for_the_slices_of_rows(api):
-    """The rows' workspace exists, that of their slices cannot be had: the SIMT kernel answers."""
+    """The workspaces of the rows and of the flags exist, that of the slices cannot be had: the SIMT
+    kernel answers."""
     model, b, nb = setup(api)
     api.mtp_set_active_set(model, torch.tensor(synth.diag_dominant(6, model.n_params), device="cuda"))
     api.mtp_config_rows(model, b, nb, "fp64")
+    api.mtp_grade(model, b, nb, "mixed")
     out = []
     grade = lambda: out.append(api.mtp_grade(model, b, nb, "fp64")["gamma"].cpu().numpy())   # noqa: E731
     ran = regions(api, lambda: fail_growth(api, 0, grade))
