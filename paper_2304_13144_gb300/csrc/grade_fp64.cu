@@ -519,10 +519,11 @@ int64_t reserve_grade_fp64(mtp_model* md, int64_t N, cudaStream_t s) {
   return cn;
 }
 
-void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, double* gamma, int32_t* argmax, cudaStream_t s) {
+// (cn: what reserve_grade_fp64 returned)
+void run_grade_fp64(mtp_model* md, int64_t N, int64_t cn, const double* rows, int64_t ld, double* gamma, int32_t* argmax,
+                    cudaStream_t s) {
   const int64_t m = md->m_active;
   if (N == 0) return;
-  const int64_t cn = reserve_grade_fp64(md, N, s);
   if (cn == 0) {
     run_grade_simt(md, N, true, rows, nullptr, ld, gamma, argmax, s);
     return;
