@@ -64,11 +64,11 @@ COMPANION = {"seed": 444, "cells": 8, "eps": 1e-2}
 MEASURED_TRAFFIC = {
     # the three kernels of the split per-neighborhood pass (k_moments + k_contract_group + k_adjoint)
     "site_pass": {"source": ("paper_2304_13144_gb300/csrc/site_split.cu", "paper_2304_13144_gb300/csrc/site_group.cu"),
-                  "sha1": "45a6c9c7b6db41326e24ccde531ea513bebe5937",
-                  "atoms": 131072, "bytes": (119674368 + 105439232) + (163370496 + 401006336) + (291428352 + 418724864)},
+                  "sha1": "8a3a47886beb94b5340035c81e14618ccea80583",
+                  "atoms": 131072, "bytes": (119684864 + 106204928) + (162978304 + 401152512) + (291489280 + 418325248)},
     "grade_tc_tf32x3": {"source": ("paper_2304_13144_gb300/csrc/grade_tc.cu",),
-                        "sha1": "aa11d04059de4159524f2038035c0e2c9ba829f6",
-                        "atoms": 131072, "bytes": 507607808 + 2587904},
+                        "sha1": "b8e071da25722f23f9346d0996614cd2486559ae",
+                        "atoms": 131072, "bytes": 507594240 + 2592768},
 }
 
 
