@@ -672,9 +672,7 @@ void upload_theta(mtp_model* md) {
 
 void run_grade_simt(mtp_model* md, int64_t N, bool fp64, const double* rows, const float* rows_f, int64_t ld,
                     double* gamma, int32_t* argmax, cudaStream_t s);
-int64_t reserve_grade_fp64(mtp_model* md, int64_t N, cudaStream_t s);
-void run_grade_fp64(mtp_model* md, int64_t N, int64_t cn, const double* rows, int64_t ld, double* gamma, int32_t* argmax,
-                    cudaStream_t s);
+void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, double* gamma, int32_t* argmax, cudaStream_t s);
 bool grade_tc_available(const mtp_model* md);
 void run_grade_tc(mtp_model* md, int64_t N, const float* hi, const float* lo, int64_t ld, double* gamma,
                   int32_t* argmax, const int32_t* zrow, const int64_t* row_atom, cudaStream_t s);
@@ -838,14 +836,13 @@ void efs_and_grade_once(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp
     row_atom = order;
     zrow = z;
   }
-  // scratch of the steps below, then (FP64) what the call can do without
+  // scratch of the steps below, then (FP64) what the call can do without; the grade's workspace, which
+  // it can do without too, follows in run_grade_fp64
   const bool want_flags = want_grade && (flagged || n_flagged);
   if (want_flags && !flagged) m->ws_misc.ensure(N * sizeof(int32_t) + 64, s);
-  int64_t grade_rows = 0;   // at a time, FP64
   if (fp64) {
     const size_t red = std::max<size_t>(energy || virial ? config_sums_scratch(nb) : 0, want_flags ? flag_scratch(N) : 0);
     if (red) m->ws_red.ensure(red, s);
-    if (want_grade) grade_rows = reserve_grade_fp64(m, N, s);
     give_wide(m, b, nb, N, true, false, o, s);
   }
   run_sites(m, b, nb, fp64, o, false, nullptr, s);
@@ -855,7 +852,7 @@ void efs_and_grade_once(mtp_model* m, const mtp_batch* b, const mtp_nbr* nb, mtp
   }
   if (want_grade) {
     if (use_tc) run_grade_tc(m, N, o.rows_hi, o.rows_lo, ld, gamma, argmax, zrow, row_atom, s);
-    else if (fp64) run_grade_fp64(m, N, grade_rows, o.rows, ld, gamma, argmax, s);
+    else if (fp64) run_grade_fp64(m, N, o.rows, ld, gamma, argmax, s);
     else run_grade_simt(m, N, false, nullptr, o.rows_hi, ld, gamma, argmax, s);
     if (flagged || n_flagged) {
       int64_t* cnt = n_flagged;
@@ -1551,11 +1548,10 @@ mtp_status mtp_config_grade(mtp_model* md, const mtp_batch* b, const mtp_nbr* nb
       SiteOutputs o;
       o.rows = md->ws_rows.as<double>();
       o.rows_ld = m;
-      const int64_t grade_rows = reserve_grade_fp64(md, K, s);
       give_wide(md, b, nb, N, prec == MTP_FP64, false, o, s);
       run_sites(md, b, nb, prec == MTP_FP64, o, false, nullptr, s);
       run_config_row_sums(nb, md->ws_rows.as<double>(), m, rc, md->ws_red, s);
-      run_grade_fp64(md, K, grade_rows, rc, m, gamma_cfg, am, s);
+      run_grade_fp64(md, K, rc, m, gamma_cfg, am, s);
       if (worst) run_widen_argmax(am, K, worst, s);
     }
     if (cls) run_classify(gamma_cfg, K, gamma_save, gamma_break, cls, s);

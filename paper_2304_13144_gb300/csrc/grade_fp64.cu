@@ -503,11 +503,10 @@ struct RowPlan {
   size_t bytes() const { return sl + e + best + arg + bad + 256; }
 };
 
-}  // namespace
-
 // Takes the workspace of an FP64 grade of N rows; returns the rows it grades at a time, 0 where the SIMT
-// kernel has to (no slices of A^-1, or no memory even for chunks of kLeastRows).
-int64_t reserve_grade_fp64(mtp_model* md, int64_t N, cudaStream_t s) {
+// kernel has to (no slices of A^-1, or no memory even for chunks of kLeastRows).  Asked for once the site
+// pass is enqueued: the host's allocation of up to a GB (0.2 ms) then lies beside it.
+int64_t reserve(mtp_model* md, int64_t N, cudaStream_t s) {
   if (!md->have_slices || N == 0) return 0;
   const XPlan x = x_plan(md->m_active, md->ainv_s.p);
   const int64_t fit = static_cast<int64_t>(kSliceBytes / (static_cast<size_t>(NS) * x.kp * sizeof(uint16_t))) / FM * FM;
@@ -519,11 +518,12 @@ int64_t reserve_grade_fp64(mtp_model* md, int64_t N, cudaStream_t s) {
   return cn;
 }
 
-// (cn: what reserve_grade_fp64 returned)
-void run_grade_fp64(mtp_model* md, int64_t N, int64_t cn, const double* rows, int64_t ld, double* gamma, int32_t* argmax,
-                    cudaStream_t s) {
+}  // namespace
+
+void run_grade_fp64(mtp_model* md, int64_t N, const double* rows, int64_t ld, double* gamma, int32_t* argmax, cudaStream_t s) {
   const int64_t m = md->m_active;
   if (N == 0) return;
+  const int64_t cn = reserve(md, N, s);
   if (cn == 0) {
     run_grade_simt(md, N, true, rows, nullptr, ld, gamma, argmax, s);
     return;
