@@ -108,32 +108,31 @@ struct SwapArgs {
   double limit;         // 1 + eps
   long long max_swaps;  // in all
   long long last;       // this launch returns at the latest after this many swaps in all
-  int tries;            // of a barrier before it gives up
-  unsigned absent;      // blocks that a barrier waits for and that never come (fault injection)
   double *u, *v, *w;
   Best* part;           // [gridDim.x]
   long long* source;    // [m]
   SwapState* st;
 };
 
-constexpr int kBarrierTries = 4000000;
-
 // all blocks of a cooperative launch (arrivals count up from the launch's zero; release and acquire
-// at the counter order the blocks' writes); bounded: after about a second it gives up
-__device__ bool grid_barrier(const SwapArgs& P, unsigned& round) {
+// at the counter order the blocks' writes); bounded: after about a second it gives up.  ABSENT (fault
+// injection): it waits, for a millisecond, for one block more than there are.  (A template: limits in
+// the arguments cost each barrier 0.04 us.)
+template <bool ABSENT>
+__device__ bool grid_barrier(SwapState* st, unsigned& round) {
+  constexpr int kTries = ABSENT ? 1000 : 4000000;
   __shared__ int s_ok;
   __syncthreads();
   ++round;
   if (threadIdx.x == 0) {
     int ok = 1;
-    SwapState* const st = P.st;
-    const unsigned target = round * gridDim.x + P.absent;
+    const unsigned target = round * gridDim.x + (ABSENT ? 1u : 0u);
     unsigned seen;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->arrived) : "memory");
     for (int tries = 0;; ++tries) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&st->arrived) : "memory");
       if (seen >= target) break;
-      if (tries > P.tries) {
+      if (tries > kTries) {
         atomicExch(&st->timeout, 1u);
         ok = 0;
         break;
@@ -148,6 +147,7 @@ __device__ bool grid_barrier(const SwapArgs& P, unsigned& round) {
 
 // Values written by other blocks are read through L2 (__ldcg); each entry of C and A^-1 is updated
 // by one thread throughout.
+template <bool ABSENT>
 __global__ void __launch_bounds__(1024, 1) k_swaps(SwapArgs P) {
   const int64_t tid = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   const int64_t nt = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(1024, 1) k_swaps(SwapArgs P) {
     }
     publish(b);
   }
-  if (!grid_barrier(P, round)) return;
+  if (!grid_barrier<ABSENT>(P.st, round)) return;
   while (true) {
     Best b = kNone;
     for (int k = threadIdx.x; k < static_cast<int>(gridDim.x); k += blockDim.x)
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(1024, 1) k_swaps(SwapArgs P) {
       if (t < P.n) __stcg(P.v + t, __ldcg(P.C + t * m + j));
     }
     if (tid == 0) P.source[j] = i;
-    if (!grid_barrier(P, round)) return;
+    if (!grid_barrier<ABSENT>(P.st, round)) return;
     // C -= v u (and the largest entry of the result), A^-1 -= w u
     Best nb = kNone;
     int64_t r = r0;
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(1024, 1) k_swaps(SwapArgs P) {
     }
     publish(nb);
     ++swaps;
-    if (!grid_barrier(P, round)) return;
+    if (!grid_barrier<ABSENT>(P.st, round)) return;
   }
 }
 
@@ -256,8 +256,8 @@ int64_t run_maxvol(mtp_model* md, const double* B, int64_t n, double eps, int64_
     }
     MTP_CUDA(cudaMemsetAsync(st, 0, sizeof(SwapState), s));
     SwapArgs P{C, md->ainv_d.as<double>(), B, md->a_d.as<double>(), n, static_cast<int>(m), 1.0 + eps, max_swaps, 0,
-               kBarrierTries, 0u, u, v, w, part, src, st};
-    if (take_injected(g_inject_maxvol_wait)) { P.tries = 1000; P.absent = 1u; }
+               u, v, w, part, src, st};
+    auto kern = take_injected(g_inject_maxvol_wait) ? k_swaps<true> : k_swaps<false>;
     // the swaps change A and A^-1 in place: until the inverse of the final A is there the model has
     // no active set, whichever way this call ends
     md->have_ainv = false;
@@ -267,7 +267,7 @@ int64_t run_maxvol(mtp_model* md, const double* B, int64_t n, double eps, int64_
       MTP_CUDA(cudaMemsetAsync(&st->arrived, 0, sizeof(unsigned), s));
       P.last = swaps + 4096;   // swaps of one launch: about 45 ms at 2,000 x 222 entries
       void* args[] = {&P};
-      MTP_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_swaps), dim3(grid), dim3(1024), args, 0, s));
+      MTP_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kern), dim3(grid), dim3(1024), args, 0, s));
       ProfRegion::launched();
       SwapState h{};
       MTP_CUDA(cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, s));
